@@ -19,7 +19,9 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OUT = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT, "libcg.so")
-UNITS = ["cg_api.cu", "cg_kernels.cu", "batch_kernels.cu", "blas1.cu", "batch.cu", "cluster_solve.cu"]
+UNITS = ["solve_f64_c16.cu", "solve_f64_c32.cu", "solve_mixed_c16.cu", "solve_mixed_c32.cu", "batch_f64.cu",
+         "batch_mixed.cu", "cg_kernels.cu", "layout.cu", "cg_api.cu", "batch_kernels.cu", "blas1.cu", "batch.cu",
+         "cluster_solve.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
                 f"-I{os.path.join(ROOT, 'include')}"]

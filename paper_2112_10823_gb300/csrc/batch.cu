@@ -26,10 +26,6 @@
 #include "cg_internal.h"
 #include "host_util.h"
 
-namespace cgk {
-cudaError_t launch_f64_to_f32(int64_t n, const double* src, float* dst, cudaStream_t s);
-}
-
 namespace {
 
 thread_local std::string g_batch_create_err;
@@ -138,8 +134,9 @@ bool is_device_ptr(const void* p) {
 
 // Upper bound of a system's device footprint (before its partition is known:
 // at most one step per row).
+constexpr int64_t kPadEntries = 8;
 size_t footprint_bound(int64_t n, int64_t nnz, bool mixed, bool jacobi, int nblocks) {
-  const size_t pad = cgk::kPadEntries;
+  const size_t pad = kPadEntries;
   size_t b = 0;
   b += align_up(4 * (n + 1));
   b += align_up(4 * (nnz + pad)) + align_up(8 * (nnz + pad));
@@ -236,6 +233,10 @@ struct cg_batch_ctx {
   int32_t* d_admit_err = nullptr;      // per slot, Jacobi: first row without a positive diagonal (+1)
   int32_t* h_admit_err = nullptr;      // pinned, per slot
   PinnedPool staging;                  // host arrays of the admission pass in flight
+  cgk::LayoutScan* d_scan = nullptr;   // per slot: what the column scan found
+  cgk::LayoutScan* h_scan = nullptr;   // pinned, per slot
+  char* d_stage = nullptr;             // columns and values of a request's host arrays on their way into the arena
+  int64_t stage_entries = 0;
   cgk::SolveParams* h_sys = nullptr;   // pinned
   cgk::SolveCtrl* h_ctrl = nullptr;    // pinned
   cgk::BatchQueue* h_queue = nullptr;  // pinned
@@ -311,39 +312,25 @@ void try_capture(cg_batch_ctx* b) {
   b->graph = g;
 }
 
-// Host copies of a request's CSR structure (0-based) and its validation.
-bool load_structure(const cg_request& r, bool validate, std::vector<int32_t>& rp, std::vector<int32_t>& ci,
-                    std::string& bad) {
+// Host copy of a request's row pointers (0-based) and their validation.
+bool load_structure(const cg_request& r, bool validate, std::vector<int32_t>& rp, std::string& bad) {
   const int64_t n = r.n, nnz = r.nnz;
   const int base = r.csr.index_base;
   rp.resize(static_cast<size_t>(n) + 1);
-  ci.clear();
   if (r.csr.on_device) {
     if (cudaMemcpy(rp.data(), r.csr.row_ptr, 4 * (n + 1), cudaMemcpyDeviceToHost) != cudaSuccess) {
       cudaGetLastError();
       bad = "copy of row_ptr failed";
       return false;
     }
-    if (validate && nnz > 0) {
-      ci.resize(static_cast<size_t>(nnz));
-      if (cudaMemcpy(ci.data(), r.csr.col_idx, 4 * nnz, cudaMemcpyDeviceToHost) != cudaSuccess) {
-        cudaGetLastError();
-        bad = "copy of col_idx failed";
-        return false;
-      }
-    }
   } else {
     std::memcpy(rp.data(), r.csr.row_ptr, 4 * (n + 1));
-    if (validate) ci.assign(r.csr.col_idx, r.csr.col_idx + nnz);
   }
   if (validate) {
     if (rp[0] != base) bad = "row_ptr[0] != index_base";
     for (int64_t i = 0; bad.empty() && i < n; ++i)
       if (rp[i + 1] < rp[i]) bad = "row_ptr decreases at row " + std::to_string(i);
     if (bad.empty() && static_cast<int64_t>(rp[n]) - base != nnz) bad = "row_ptr[n] != nnz + index_base";
-    for (int64_t k = 0; bad.empty() && k < nnz; ++k)
-      if (ci[k] < base || static_cast<int64_t>(ci[k]) - base >= n)
-        bad = "column index out of range at entry " + std::to_string(k);
     if (!bad.empty()) return false;
   }
   if (base)
@@ -351,13 +338,16 @@ bool load_structure(const cg_request& r, bool validate, std::vector<int32_t>& rp
   return true;
 }
 
-// A job's device layout inside its arena block.
+// A job's device layout inside its arena block: room for the matrix in either
+// column width.  Until the solve starts, r holds the row pointers and q the
+// steps' places in the streams (8 bytes per row at most).
 struct Layout {
-  size_t rp, col, val, val32, step, mode, bstep, brow, b, x, r, p, q, p32, dinv, part, total;
+  size_t len, stream, val64, step, coff, wchunk, wentry, wstep, brow, b, x, r, p, q, p32, dinv, part, total;
 };
 
-Layout layout_of(int64_t n, int64_t nnz, size_t nsteps2, int group, bool mixed, bool jacobi) {
-  const size_t pad = cgk::kPadEntries;
+Layout layout_of(int64_t n, int64_t nnz, const cgh::Partition& part, int group, bool mixed, bool jacobi) {
+  int64_t stream_units = 0, entries = 0;
+  cgh::stream_bound(nnz, mixed, part, &stream_units, &entries);
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -365,13 +355,15 @@ Layout layout_of(int64_t n, int64_t nnz, size_t nsteps2, int group, bool mixed, 
     o += align_up(bytes);
     return at;
   };
-  L.rp = take(4 * (n + 1));
-  L.col = take(4 * (nnz + pad));
-  L.val = take(8 * (nnz + pad));
-  L.val32 = mixed ? take(4 * (nnz + pad)) : 0;
-  L.step = take(sizeof(int4) * nsteps2);
-  L.mode = take(4 * nsteps2);
-  L.bstep = take(4 * (static_cast<size_t>(group) + 1));
+  const size_t warps = static_cast<size_t>(group) * cgk::kWarps;
+  L.len = take(32 * part.step.size());
+  L.stream = take(static_cast<size_t>(stream_units) * cgk::kUnit);
+  L.val64 = mixed ? take(8 * static_cast<size_t>(entries)) : 0;
+  L.step = take(sizeof(int4) * part.step.size());
+  L.coff = take(4 * (static_cast<size_t>(part.chunks) + 1));
+  L.wchunk = take(sizeof(int4) * warps);
+  L.wentry = mixed ? take(4 * warps) : 0;
+  L.wstep = take(4 * (warps + 1));
   L.brow = take(4 * (static_cast<size_t>(group) + 1));
   L.b = take(8 * n);
   L.x = take(8 * n);
@@ -385,6 +377,39 @@ Layout layout_of(int64_t n, int64_t nnz, size_t nsteps2, int group, bool mixed, 
   return L;
 }
 
+// A system's arrays in its arena block.
+struct Dev {
+  char* base;
+  const Layout& L;
+  template <typename T>
+  T* at(size_t o) const { return reinterpret_cast<T*>(base + o); }
+};
+
+// Device buffer for the columns and values of at least `least` entries of a
+// request's host arrays: kStageEntries, or what one CTA's share needs if that is
+// more; half as much, and so on, where memory is short.
+constexpr int64_t kStageEntries = int64_t(4) << 20;
+cudaError_t reserve_stage(cg_batch_ctx* b, int64_t least) {
+  if (b->stage_entries >= least && b->d_stage != nullptr) return cudaSuccess;
+  if (b->d_stage) {
+    cudaError_t e = cudaStreamSynchronize(b->copy);
+    if (e != cudaSuccess) return e;
+    cudaFree(b->d_stage);
+    b->d_stage = nullptr;
+    b->stage_entries = 0;
+  }
+  for (int64_t want = std::max(least, kStageEntries);; want = std::max(least, want / 2)) {
+    const cudaError_t e = cudaMalloc(&b->d_stage, 12 * static_cast<size_t>(want));
+    if (e == cudaSuccess) {
+      b->stage_entries = want;
+      return e;
+    }
+    b->d_stage = nullptr;
+    if (want == least) return e;
+    cudaGetLastError();
+  }
+}
+
 void finish_without_device(cg_batch_ctx* b, Job* j, int status) {
   j->res.done = 1;
   j->res.status = status;
@@ -395,14 +420,19 @@ void finish_without_device(cg_batch_ctx* b, Job* j, int status) {
 
 // Prepare and upload the queue head while memory and slots allow.  Called by
 // the worker without the lock held (the lock guards the queue only).  The
-// copies of every system of the pass go onto the copy stream back to back
-// (the host prepares the next system while the previous one's copies run);
-// the small host arrays are staged in pinned memory that stays untouched
-// until the one synchronisation at the end of the pass, after which each
-// system is checked and made resident.
+// copies and kernels of every system of the pass go onto the copy stream back
+// to back (the host prepares the next system while the previous one's work
+// runs); the small host arrays are staged in pinned memory that stays
+// untouched until the end of the pass.  The stream order of a system needs
+// one read-back, the column scan's: systems whose arrays are on the device
+// share one for the whole pass; those with host arrays, which go through one
+// staging buffer, have one each.
 void admit(cg_batch_ctx* b) {
   struct Staged {
     Job* j;
+    Layout L;
+    std::vector<int32_t> rp;
+    cgh::Partition part;
     cudaError_t e;
   };
   std::vector<Staged> staged;
@@ -421,6 +451,35 @@ void admit(cg_batch_ctx* b) {
     std::memcpy(q, src, bytes);
     return cudaMemcpyAsync(dst, q, bytes, cudaMemcpyHostToDevice, s);
   };
+  // of a system's steps [k0, k1) or rows [r0, r1), whose entries src holds
+  auto scan = [&](const Dev& d, const cgk::CsrSource& src, int slot, int32_t k0, int32_t k1, int64_t n) {
+    return cgk::launch_layout_scan(src, d.at<int4>(d.L.step), d.at<uint8_t>(d.L.len), nullptr, k0, k1, n, b->validate, b->d_scan + slot, s);
+  };
+  auto fill = [&](const Dev& d, const cgk::CsrSource& src, int slot, int32_t k0, int32_t k1, int64_t r0, int64_t r1) {
+    const cgk::DevCsr& A = b->h_sys[slot].A;
+    const cgk::StreamPlace to{A.chunk_off, d.at<uint32_t>(d.L.q), d.at<uint32_t>(d.L.q) + A.nsteps,
+                              d.at<unsigned char>(d.L.stream), b->mixed ? d.at<double>(d.L.val64) : nullptr};
+    cudaError_t e = cgk::launch_layout_fill(src, A.step, to, k0, k1, A.col16 != 0, b->mixed, s);
+    if (e == cudaSuccess && b->jacobi)
+      e = cgk::launch_jacobi_dinv(src, r0, r1, d.at<double>(d.L.dinv), b->d_admit_err + slot, s);
+    return e;
+  };
+  // once the scan has been read back: the places of the entries
+  auto place = [&](const Dev& d, const std::vector<int32_t>& rp, cgh::Partition& part, int slot) {
+    cgk::DevCsr& A = b->h_sys[slot].A;
+    A.col16 = b->h_scan[slot].span <= cgk::kColSpan16 ? 1 : 0;
+    cgh::place_steps(rp, A.nblocks, A.col16 != 0, b->mixed, part);
+    uint32_t* const q = d.at<uint32_t>(d.L.q);
+    const size_t nsteps = static_cast<size_t>(A.nsteps);
+    cudaError_t e = upload(d.at<char>(d.L.coff), part.chunk_off.data(), 4 * part.chunk_off.size());
+    if (e == cudaSuccess) e = upload(d.at<char>(d.L.wchunk), part.warp_chunk.data(), sizeof(int4) * part.warp_chunk.size());
+    if (e == cudaSuccess) e = upload(q, part.step_chunk.data(), 4 * nsteps);
+    if (b->mixed) {
+      if (e == cudaSuccess) e = upload(d.at<char>(d.L.wentry), part.warp_entry.data(), 4 * part.warp_entry.size());
+      if (e == cudaSuccess) e = upload(q + nsteps, part.step_entry.data(), 4 * nsteps);
+    }
+    return e;
+  };
   for (;;) {
     Job* j = nullptr;
     {
@@ -430,9 +489,9 @@ void admit(cg_batch_ctx* b) {
       j = b->jobs[b->queued.front()].get();
     }
     const cg_request& r = j->req;
-    std::vector<int32_t> rp, ci;
+    std::vector<int32_t> rp;
     std::string bad;
-    if (!load_structure(r, b->validate, rp, ci, bad)) {
+    if (!load_structure(r, b->validate, rp, bad)) {
       std::lock_guard<std::mutex> lk(b->mu);
       b->queued.pop_front();
       finish_without_device(b, j, CG_EINVAL);
@@ -450,8 +509,17 @@ void admit(cg_batch_ctx* b) {
       shape = b->shape;
     }
     cgh::Partition part;
-    cgh::build_partition(rp, n, group, part, shape);
-    const Layout L = layout_of(n, nnz, part.step.size(), group, b->mixed, b->jacobi);
+    cgh::build_partition(rp, n, group, b->mixed, part, shape);
+    const int32_t nsteps = static_cast<int32_t>(part.step.size()) - 1;
+    const Layout L = layout_of(n, nnz, part, group, b->mixed, b->jacobi);
+    if (L.total > b->arena.cap()) {  // (a matrix of many short steps: submit's bound allows one table less)
+      std::lock_guard<std::mutex> lk(b->mu);
+      b->queued.pop_front();
+      finish_without_device(b, j, CG_ENOMEM);
+      b->err = "request " + std::to_string(j->ticket) + " needs more memory than the budget";
+      b->cv_done.notify_all();
+      continue;
+    }
     size_t off = 0;
     int slot = -1;
     {
@@ -467,79 +535,31 @@ void admit(cg_batch_ctx* b) {
     j->group = group;
     j->bytes_step = bytes_per_step(n, nnz, b->mixed);
     j->steps_est = est_steps(b->model, n);
-    char* base = b->d_arena + off;
-    auto at = [&](size_t o) { return base + o; };
-    const size_t pad = cgk::kPadEntries;
-    cudaError_t e = cudaSuccess;
-    auto step = [&](cudaError_t x) {
-      if (e == cudaSuccess) e = x;
-    };
-    step(upload(at(L.rp), rp.data(), 4 * (n + 1)));
-    step(cudaMemsetAsync(at(L.col), 0, 4 * (nnz + pad), s));
-    step(cudaMemsetAsync(at(L.val), 0, 8 * (nnz + pad), s));
-    if (nnz > 0) {
-      // the request's own arrays stay valid until its result is final
-      const cudaMemcpyKind k = r.csr.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-      if (r.csr.index_base == 0) {
-        step(cudaMemcpyAsync(at(L.col), r.csr.col_idx, 4 * nnz, k, s));
-      } else {
-        if (ci.empty()) {  // not validated: the columns are not on the host yet
-          if (r.csr.on_device) {
-            ci.resize(static_cast<size_t>(nnz));
-            step(cudaMemcpy(ci.data(), r.csr.col_idx, 4 * nnz, cudaMemcpyDeviceToHost));
-          } else {
-            ci.assign(r.csr.col_idx, r.csr.col_idx + nnz);
-          }
-        }
-        for (auto& v : ci) v -= 1;
-        step(upload(at(L.col), ci.data(), 4 * nnz));
-      }
-      step(cudaMemcpyAsync(at(L.val), r.csr.val, 8 * nnz, k, s));
-      if (b->mixed) {
-        step(cudaMemsetAsync(at(L.val32), 0, 4 * (nnz + pad), s));
-        step(cgk::launch_f64_to_f32(nnz, reinterpret_cast<double*>(at(L.val)), reinterpret_cast<float*>(at(L.val32)),
-                                    s));
-      }
-    }
-    step(upload(at(L.step), part.step.data(), sizeof(int4) * part.step.size()));
-    step(upload(at(L.mode), part.step_mode.data(), 4 * part.step_mode.size()));
-    step(upload(at(L.bstep), part.block_step.data(), 4 * part.block_step.size()));
-    step(upload(at(L.brow), part.block_row.data(), 4 * part.block_row.size()));
-    step(cudaMemcpyAsync(at(L.b), r.b, 8 * n, is_device_ptr(r.b) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                         s));
-    step(cudaMemsetAsync(at(L.x), 0, 8 * n, s));
-    if (b->jacobi) {
-      step(cudaMemsetAsync(b->d_admit_err + slot, 0, sizeof(int32_t), s));
-      step(cgk::launch_jacobi_dinv(reinterpret_cast<int32_t*>(at(L.rp)), reinterpret_cast<int32_t*>(at(L.col)),
-                                   reinterpret_cast<double*>(at(L.val)), n, reinterpret_cast<double*>(at(L.dinv)),
-                                   b->d_admit_err + slot, s));
-      step(cudaMemcpyAsync(b->h_admit_err + slot, b->d_admit_err + slot, sizeof(int32_t), cudaMemcpyDeviceToHost,
-                           s));
-    }
-    step(cudaMemsetAsync(b->d_ctrl + slot, 0, sizeof(cgk::SolveCtrl), s));
-    cgk::SolveParams& P = b->h_sys[slot];  // pinned; read by the copy below when it runs
+    const Dev d{b->d_arena + off, L};
+    cgk::SolveParams& P = b->h_sys[slot];  // pinned; copied once the matrix has its place
     std::memset(&P, 0, sizeof(P));
-    P.A.row_ptr = reinterpret_cast<int32_t*>(at(L.rp));
-    P.A.col_idx = reinterpret_cast<int32_t*>(at(L.col));
-    P.A.val = reinterpret_cast<double*>(at(L.val));
-    P.A.val32 = b->mixed ? reinterpret_cast<float*>(at(L.val32)) : nullptr;
-    P.A.step = reinterpret_cast<int4*>(at(L.step));
-    P.A.step_mode = reinterpret_cast<int32_t*>(at(L.mode));
-    P.A.block_step = reinterpret_cast<int32_t*>(at(L.bstep));
-    P.A.block_row = reinterpret_cast<int32_t*>(at(L.brow));
+    P.A.stream = d.at<unsigned char>(L.stream);
+    P.A.val64 = b->mixed ? d.at<double>(L.val64) : nullptr;
+    P.A.step = d.at<int4>(L.step);
+    P.A.seg_len = d.at<uint8_t>(L.len);
+    P.A.chunk_off = d.at<uint32_t>(L.coff);
+    P.A.warp_chunk = d.at<int4>(L.wchunk);
+    P.A.warp_entry = b->mixed ? d.at<uint32_t>(L.wentry) : nullptr;
+    P.A.warp_step = d.at<int32_t>(L.wstep);
+    P.A.block_row = d.at<int32_t>(L.brow);
     P.A.n = static_cast<int32_t>(n);
-    P.A.nsteps = static_cast<int32_t>(part.step.size()) - 2;
+    P.A.nsteps = nsteps;
     P.A.nblocks = group;
     for (int g = 0; g < group; ++g)
       P.A.max_rows = std::max(P.A.max_rows, part.block_row[g + 1] - part.block_row[g]);
     P.A.nnz = nnz;
-    P.b = reinterpret_cast<double*>(at(L.b));
-    P.x = reinterpret_cast<double*>(at(L.x));
-    P.r = reinterpret_cast<double*>(at(L.r));
-    P.p = reinterpret_cast<double*>(at(L.p));
-    P.q = reinterpret_cast<double*>(at(L.q));
-    P.p32 = b->mixed ? reinterpret_cast<float*>(at(L.p32)) : nullptr;
-    P.partials = reinterpret_cast<double*>(at(L.part));
+    P.b = d.at<double>(L.b);
+    P.x = d.at<double>(L.x);
+    P.r = d.at<double>(L.r);
+    P.p = d.at<double>(L.p);
+    P.q = d.at<double>(L.q);
+    P.p32 = b->mixed ? d.at<float>(L.p32) : nullptr;
+    P.partials = d.at<double>(L.part);
     P.ctrl = b->d_ctrl + slot;
     P.tol = r.tol;
     P.maxit = r.maxit;
@@ -547,41 +567,117 @@ void admit(cg_batch_ctx* b) {
     P.wait_limit_ns = b->wait_ns;
     P.group = group;
     P.chunk_iters = b->chunk_iters;
-    P.dinv = b->jacobi ? reinterpret_cast<double*>(at(L.dinv)) : nullptr;
-    step(cudaMemcpyAsync(b->d_sys + slot, &P, sizeof(P), cudaMemcpyHostToDevice, s));
-    j->d_x = reinterpret_cast<double*>(at(L.x));
-    staged.push_back({j, e});
+    P.dinv = b->jacobi ? d.at<double>(L.dinv) : nullptr;
+    cudaError_t e = cudaSuccess;
+    auto step = [&](cudaError_t x) {
+      if (e == cudaSuccess) e = x;
+    };
+    step(upload(d.at<char>(L.r), rp.data(), 4 * (n + 1)));
+    step(upload(d.at<char>(L.step), part.step.data(), sizeof(int4) * part.step.size()));
+    step(upload(d.at<char>(L.wstep), part.warp_step.data(), 4 * part.warp_step.size()));
+    step(upload(d.at<char>(L.brow), part.block_row.data(), 4 * part.block_row.size()));
+    step(cudaMemcpyAsync(d.at<char>(L.b), r.b, 8 * n,
+                         is_device_ptr(r.b) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+    step(cudaMemsetAsync(d.at<char>(L.x), 0, 8 * n, s));
+    if (b->jacobi) step(cudaMemsetAsync(b->d_admit_err + slot, 0, sizeof(int32_t), s));
+    step(cudaMemsetAsync(b->d_ctrl + slot, 0, sizeof(cgk::SolveCtrl), s));
+    step(cudaMemsetAsync(b->d_scan + slot, 0, sizeof(cgk::LayoutScan), s));
+    cgk::CsrSource src{d.at<int32_t>(L.r), r.csr.col_idx, r.csr.val, 0, r.csr.index_base};
+    if (e == cudaSuccess && r.csr.on_device) {
+      step(scan(d, src, slot, 0, nsteps, n));
+    } else if (e == cudaSuccess) {
+      // host arrays: in runs of CTA shares (consecutive rows) that fit the staging
+      // buffer, scanned, read back, and uploaded again to be filled (once, if a
+      // single run holds them all)
+      auto first_entry = [&](int c) -> int64_t { return rp[part.block_row[c]]; };
+      auto first_step = [&](int c) { return part.warp_step[static_cast<size_t>(c) * cgk::kWarps]; };
+      int64_t most = 1;
+      for (int c = 0; c < group; ++c) most = std::max(most, first_entry(c + 1) - first_entry(c));
+      step(reserve_stage(b, most));
+      auto run_end = [&](int c0) {
+        int c1 = c0 + 1;
+        while (c1 < group && first_entry(c1 + 1) - first_entry(c0) <= b->stage_entries) ++c1;
+        return c1;
+      };
+      auto stage = [&](int c0, int c1, bool values) {
+        const int64_t e0 = first_entry(c0), cnt = first_entry(c1) - e0;
+        double* const v = reinterpret_cast<double*>(b->d_stage);
+        int32_t* const c = reinterpret_cast<int32_t*>(v + b->stage_entries);
+        src.e_first = e0;
+        src.col_idx = c;
+        src.val = v;
+        if (cnt == 0) return;
+        step(cudaMemcpyAsync(c, r.csr.col_idx + e0, 4 * cnt, cudaMemcpyHostToDevice, s));
+        if (values) step(cudaMemcpyAsync(v, r.csr.val + e0, 8 * cnt, cudaMemcpyHostToDevice, s));
+      };
+      const bool single = e == cudaSuccess && run_end(0) == group;
+      for (int c0 = 0, c1; e == cudaSuccess && c0 < group; c0 = c1) {
+        c1 = run_end(c0);
+        stage(c0, c1, single);
+        step(scan(d, src, slot, first_step(c0), first_step(c1), n));
+      }
+      step(cudaMemcpyAsync(b->h_scan + slot, b->d_scan + slot, sizeof(cgk::LayoutScan), cudaMemcpyDeviceToHost, s));
+      step(cudaStreamSynchronize(s));
+      if (e == cudaSuccess && b->h_scan[slot].bad_entry == 0) step(place(d, rp, part, slot));
+      for (int c0 = 0, c1; e == cudaSuccess && c0 < group && b->h_scan[slot].bad_entry == 0; c0 = c1) {
+        c1 = run_end(c0);
+        if (!single) stage(c0, c1, true);
+        step(fill(d, src, slot, first_step(c0), first_step(c1), part.block_row[c0], part.block_row[c1]));
+      }
+    }
+    j->d_x = d.at<double>(L.x);
+    staged.push_back({j, L, std::move(rp), std::move(part), e});
   }
   if (staged.empty()) return;
-  const cudaError_t es = cudaStreamSynchronize(s);
+  cudaError_t es = cudaMemcpyAsync(b->h_scan, b->d_scan, sizeof(cgk::LayoutScan) * b->max_systems,
+                                   cudaMemcpyDeviceToHost, s);
+  if (es == cudaSuccess) es = cudaStreamSynchronize(s);
+  for (Staged& st : staged) {
+    if (st.e == cudaSuccess) st.e = es;
+    const int slot = st.j->slot;
+    if (st.e != cudaSuccess || b->h_scan[slot].bad_entry != 0) continue;
+    auto step = [&](cudaError_t x) {
+      if (st.e == cudaSuccess) st.e = x;
+    };
+    const Dev d{b->d_arena + st.j->off, st.L};
+    const cg_request& r = st.j->req;
+    if (r.csr.on_device) {
+      const cgk::CsrSource src{d.at<int32_t>(st.L.r), r.csr.col_idx, r.csr.val, 0, r.csr.index_base};
+      step(place(d, st.rp, st.part, slot));
+      if (st.e == cudaSuccess) step(fill(d, src, slot, 0, b->h_sys[slot].A.nsteps, 0, r.n));
+    }
+    if (b->jacobi)
+      step(cudaMemcpyAsync(b->h_admit_err + slot, b->d_admit_err + slot, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    step(cudaMemcpyAsync(b->d_sys + slot, b->h_sys + slot, sizeof(cgk::SolveParams), cudaMemcpyHostToDevice, s));
+  }
+  es = cudaStreamSynchronize(s);
   std::vector<Job*> uploaded;
+  // a request that cannot become resident: its memory and slot are free again
+  auto give_up = [&](Job* j, int status, const std::string& why) {
+    std::lock_guard<std::mutex> lk(b->mu);
+    b->arena.release(j->off, j->bytes);
+    b->free_slots.push_back(j->slot);
+    j->slot = -1;
+    finish_without_device(b, j, status);
+    b->err = why;
+    b->cv_done.notify_all();
+  };
   for (const Staged& st : staged) {
     Job* j = st.j;
     const cudaError_t e = st.e != cudaSuccess ? st.e : es;
     const int slot = j->slot;
-    if (e == cudaSuccess && b->jacobi && b->h_admit_err[slot] != 0) {
-      std::lock_guard<std::mutex> lk(b->mu);
-      b->arena.release(j->off, j->bytes);
-      b->free_slots.push_back(slot);
-      j->slot = -1;
-      finish_without_device(b, j, CG_EINVAL);
-      b->err = "request " + std::to_string(j->ticket) + ": Jacobi preconditioner: diagonal of row " +
-               std::to_string(b->h_admit_err[slot] - 1) + " is not positive";
-      b->cv_done.notify_all();
-      continue;
-    }
     if (e != cudaSuccess) {
       cudaGetLastError();
-      std::lock_guard<std::mutex> lk(b->mu);
-      b->arena.release(j->off, j->bytes);
-      b->free_slots.push_back(slot);
-      j->slot = -1;
-      finish_without_device(b, j, CG_ECUDA);
-      b->err = cuda_msg(e, "admission copies");
-      b->cv_done.notify_all();
-      continue;
+      give_up(j, e == cudaErrorMemoryAllocation ? CG_ENOMEM : CG_ECUDA, cuda_msg(e, "admission"));
+    } else if (b->h_scan[slot].bad_entry != 0) {
+      give_up(j, CG_EINVAL, "request " + std::to_string(j->ticket) + ": invalid CSR: column index out of range at entry " +
+                                std::to_string(~b->h_scan[slot].bad_entry));
+    } else if (b->jacobi && b->h_admit_err[slot] != 0) {
+      give_up(j, CG_EINVAL, "request " + std::to_string(j->ticket) + ": Jacobi preconditioner: diagonal of row " +
+                                std::to_string(b->h_admit_err[slot] - 1) + " is not positive");
+    } else {
+      uploaded.push_back(j);
     }
-    uploaded.push_back(j);
   }
   if (!uploaded.empty()) {
     std::lock_guard<std::mutex> lk(b->mu);
@@ -648,7 +744,7 @@ std::vector<Job*> build_queue(cg_batch_ctx* b, const std::vector<Job*>& res) {
   // the systems of a round run side by side: their vectors share the L2
   int64_t reused = 0;
   for (const Job* j : in_round) reused += cgk::step_reused_bytes(j->req.n, b->mixed, b->jacobi);
-  b->h_queue->stream_rows = cgk::stream_row_ptrs(reused, b->l2_bytes) ? 1 : 0;
+  b->h_queue->stream_rows = cgk::stream_row_tables(reused, b->l2_bytes) ? 1 : 0;
   return in_round;
 }
 
@@ -764,6 +860,9 @@ void release_all(cg_batch_ctx* b) {
   if (b->d_next) cudaFree(b->d_next);
   if (b->d_admit_err) cudaFree(b->d_admit_err);
   if (b->h_admit_err) cudaFreeHost(b->h_admit_err);
+  if (b->d_scan) cudaFree(b->d_scan);
+  if (b->h_scan) cudaFreeHost(b->h_scan);
+  if (b->d_stage) cudaFree(b->d_stage);
   if (b->h_sys) cudaFreeHost(b->h_sys);
   if (b->h_ctrl) cudaFreeHost(b->h_ctrl);
   if (b->h_queue) cudaFreeHost(b->h_queue);
@@ -1088,15 +1187,18 @@ int cg_batch_create(cg_batch* out, const cg_batch_opts* opts) {
       (e = cudaMalloc(&b->d_ctrl, sizeof(cgk::SolveCtrl) * b->max_systems)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_queue, b->queue_bytes)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_next, 16)) != cudaSuccess ||
+      (e = cudaMalloc(&b->d_scan, sizeof(cgk::LayoutScan) * b->max_systems)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_admit_err, sizeof(int32_t) * b->max_systems)) != cudaSuccess)
     return fail_cuda(e, "cg_batch_create: tables");
   if ((e = cudaMallocHost(&b->h_sys, sizeof(cgk::SolveParams) * b->max_systems)) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_ctrl, sizeof(cgk::SolveCtrl) * b->max_systems)) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_queue, b->queue_bytes)) != cudaSuccess ||
+      (e = cudaMallocHost(&b->h_scan, sizeof(cgk::LayoutScan) * b->max_systems)) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_admit_err, sizeof(int32_t) * b->max_systems)) != cudaSuccess)
     return fail_cuda(e, "cg_batch_create: pinned tables");
   std::memset(b->h_queue, 0, b->queue_bytes);
   if ((e = cudaMemset(b->d_ctrl, 0, sizeof(cgk::SolveCtrl) * b->max_systems)) != cudaSuccess ||
+      (e = cudaMemset(b->d_scan, 0, sizeof(cgk::LayoutScan) * b->max_systems)) != cudaSuccess ||
       (e = cudaMemset(b->d_sys, 0, sizeof(cgk::SolveParams) * b->max_systems)) != cudaSuccess)
     return fail_cuda(e, "cg_batch_create: clear");
   b->free_slots.reserve(b->max_systems);

@@ -1,53 +1,27 @@
-// The batched persistent solve: many systems in one cooperative launch.
-// Each CTA takes tasks (a system and its rank in the system's group of CTAs)
-// from a queue; the CG arithmetic of every task is the single-system solve's
-// (cg_solve.cuh).
-#include "cg_solve.cuh"
+// Launch of the batched persistent solve (batch_kernel.cuh).
+#include <algorithm>
+#include "cg_internal.h"
 
 namespace cgk {
 
-// Many systems in one persistent launch: each CTA takes tasks (a system and
-// its rank in the system's group) from the queue, in queue order, until it is
-// empty.  The host orders the queue longest estimated time per CTA first,
-// with a group's ranks next to each other; a group's first ranks wait at its
-// first group barrier until CTAs that free up have taken the rest.  Between
-// tasks the whole CTA (producer included) joins, the producer having drained
-// its copies, and the ring barriers are reset.
-template <bool kMixed, bool kJacobi>
-__global__ void __launch_bounds__(kBlock, kCtasPerSm) cg_batch_kernel(const __grid_constant__ BatchParams B) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const RingSmem sm{smem_raw, kMixed ? 4u : 8u};  // FP32 values in the mixed solve's stream
-  __shared__ int32_t task_id;
-  bool reinit = false;
-  for (;;) {
-    if (threadIdx.x == 0) task_id = atomicAdd(B.next, 1);
-    __syncthreads();
-    const int t = task_id;
-    if (t >= B.queue->ntasks) break;
-    const BatchTask tk = B.queue->task[t];
-    const SolveParams& P = B.sys[tk.sys];
-    CtaStream cs;
-    stream_setup(sm, cs, P.A, tk.rank, reinit);
-    reinit = true;
-    if (threadIdx.x >= kConsumers) solve_producer<kMixed>(sm, cs, P);
-    else solve_consumers<kMixed, kJacobi, false, false>(sm, cs, P, tk.rank, &B.queue->stream_rows);
-    __syncthreads();  // producer drained, consumers done: the CTA is free
-  }
-}
+template <bool kMixed>
+const void* batch_kernel_of(bool jacobi);  // batch_f64.cu, batch_mixed.cu
 
 const void* batch_kernel_ptr(bool mixed, bool jacobi) {
-  if (mixed) return jacobi ? reinterpret_cast<const void*>(cg_batch_kernel<true, true>)
-                           : reinterpret_cast<const void*>(cg_batch_kernel<true, false>);
-  return jacobi ? reinterpret_cast<const void*>(cg_batch_kernel<false, true>)
-                : reinterpret_cast<const void*>(cg_batch_kernel<false, false>);
+  return mixed ? batch_kernel_of<true>(jacobi) : batch_kernel_of<false>(jacobi);
+}
+
+// A batch may hold systems of both column widths: room for either ring.
+size_t batch_smem_bytes(bool mixed) {
+  return std::max(solve_smem_bytes(mixed, false), solve_smem_bytes(mixed, true));
 }
 
 int batch_blocks_per_sm(bool mixed, bool jacobi) {
   int nb = 0;
   const void* k = batch_kernel_ptr(mixed, jacobi);
-  const size_t smem = solve_smem_bytes(mixed);
+  const size_t smem = batch_smem_bytes(mixed);
   cudaError_t e = ensure_smem_attr(k, smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kBlock, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kThreads, smem);
   return e == cudaSuccess ? nb : -1;
 }
 
@@ -56,12 +30,12 @@ int batch_blocks_per_sm(bool mixed, bool jacobi) {
 // CUDA graph.
 cudaError_t launch_batch(const BatchParams& B, bool mixed, bool jacobi, int nblocks, cudaStream_t s) {
   const void* k = batch_kernel_ptr(mixed, jacobi);
-  const size_t smem = solve_smem_bytes(mixed);
+  const size_t smem = batch_smem_bytes(mixed);
   cudaError_t e = ensure_smem_attr(k, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nblocks);
-  cfg.blockDim = dim3(kBlock);
+  cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

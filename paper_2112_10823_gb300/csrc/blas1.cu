@@ -306,22 +306,6 @@ cudaError_t launch_ewmul(int64_t n, const double* x, const double* y, double* z,
 
 }  // namespace cgk
 
-namespace cgk {
-
-// FP32 copy of the matrix values (mixed-precision handles), round to nearest.
-__global__ void f64_to_f32_kernel(int64_t n, const double* __restrict__ src, float* __restrict__ dst) {
-  const int64_t T = static_cast<int64_t>(gridDim.x) * kVecBlock;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * kVecBlock + threadIdx.x; i < n; i += T)
-    dst[i] = __double2float_rn(src[i]);
-}
-
-cudaError_t launch_f64_to_f32(int64_t n, const double* src, float* dst, cudaStream_t s) {
-  f64_to_f32_kernel<<<stream_grid(n), kVecBlock, 0, s>>>(n, src, dst);
-  return cudaGetLastError();
-}
-
-}  // namespace cgk
-
 // ---------------------------------------------------------------------------
 // Dot product without any allocation (cg_dot_noalloc).
 //

@@ -21,7 +21,6 @@ using cgh::Partition;
 using cgh::build_partition;
 
 namespace cgk {
-cudaError_t launch_f64_to_f32(int64_t n, const double* src, float* dst, cudaStream_t s);
 cudaError_t launch_dot_noalloc(int64_t n, const double* x, const double* y, double* out, cudaStream_t s);
 int64_t dot_noalloc_max_n();
 }
@@ -32,10 +31,8 @@ namespace cgh {
 // contiguous CTA ranges of about equal cost (stored entries + kRowCost per
 // row, the per-row vector work), and each CTA range into steps (see
 // cg_internal.h): up to 32 rows of <= 32 entries (one lane per row), up to 16
-// rows of <= 64 entries (two lanes per row), never more than kStepNnz entries,
-// or one longer row.  Two sentinel steps follow the last one (the kernels
-// read descriptors ahead).
-constexpr int64_t kRowCost = 6;
+// rows of <= 64 entries (two lanes per row), or one longer row.
+constexpr int64_t kRowCost = 14;
 
 int64_t cost_split(const std::vector<int32_t>& rp, int64_t lo_row, int64_t hi_row, int64_t part, int64_t parts) {
   // first row i in [lo_row, hi_row] with cost(lo_row, i) >= cost(lo_row, hi_row) * part / parts
@@ -65,53 +62,160 @@ bool StepShape::valid() const {
   return true;
 }
 
-void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end, const StepShape& shape, Partition& P) {
+// A segment of `len` entries split evenly over as few chunks as it takes: the
+// entries of one chunk.
+static int chunk_of(int64_t len, int most) {
+  if (len <= 0) return 0;
+  const int64_t parts = (len + most - 1) / most;
+  return static_cast<int>((len + parts - 1) / parts);
+}
+
+static int4 make_step(int64_t row, int lanes, int mode, bool uniform, int rem, int64_t seg, int64_t entries,
+                      int chunk) {
+  static_assert(cgk::max_chunk<double>() < 64 && cgk::max_chunk<float>() < 64, "six bits");
+  const bool pads = (lanes < 32 || !uniform) && cgk::step_pads(seg, entries);
+  unsigned int y = static_cast<unsigned int>(lanes) | static_cast<unsigned int>(mode) << cgk::kStepModeShift |
+                   (uniform ? static_cast<unsigned int>(cgk::kStepUniform) : 0u) |
+                   (pads ? static_cast<unsigned int>(cgk::kStepPadded) : 0u) |
+                   static_cast<unsigned int>(rem) << cgk::kStepRemShift |
+                   static_cast<unsigned int>(chunk_of(seg, chunk)) << cgk::kStepChunkShift;
+  return make_int4(static_cast<int>(row), static_cast<int>(y), static_cast<int>(seg), 0);
+}
+
+static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end, int chunk, const StepShape& shape,
+                       std::vector<int4>& out) {
   auto kind = [&](int64_t len) -> int { return len > kShapeMaxLen ? cgk::kLongRow : shape.mode[len]; };
   while (row < end) {
     const int64_t len0 = rp[row + 1] - rp[row];
-    if (kind(len0) == cgk::kLongRow) {  // a warp per row: one step, walked piece by piece
-      P.step.push_back(make_int4(static_cast<int>(row), static_cast<int>(row + 1), rp[row], rp[row + 1]));
-      P.step_mode.push_back(cgk::kLongRow);
+    if (kind(len0) == cgk::kLongRow) {  // a warp per row
+      const int rem = static_cast<int>(len0 % 32);
+      out.push_back(make_step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0, chunk));
       ++row;
       continue;
     }
     const int64_t start = row;
-    int64_t cnt = 0, maxlen = 0;
+    int64_t maxlen = 0, minlen = 0;
     int m = cgk::kLanePerRow;  // the widest kind so far (one lane < two lanes)
     while (row < end) {
       const int64_t len = rp[row + 1] - rp[row];
       const int k = kind(len);
-      if (k == cgk::kLongRow || cnt + len > cgk::kStepNnz) break;
+      if (k == cgk::kLongRow) break;
       const int nm = std::max(m, k);
       const int64_t cap = nm == cgk::kLanePerRow ? 32 : 16;
       if (row - start + 1 > cap) break;
-      cnt += len;
       maxlen = std::max(maxlen, len);
+      minlen = row == start ? len : std::min(minlen, len);
       m = nm;
       ++row;
     }
-    P.step.push_back(make_int4(static_cast<int>(start), static_cast<int>(row), rp[start], rp[row]));
-    const int64_t wmax = m == cgk::kLanePerRow ? maxlen : (maxlen + 1) / 2;  // longest segment of one lane
-    P.step_mode.push_back(m | static_cast<int32_t>(wmax << cgk::kWmaxShift));
+    const int rows = static_cast<int>(row - start);
+    const int64_t cnt = rp[row] - rp[start];
+    if (m == cgk::kLanePerRow)
+      out.push_back(make_step(start, rows, m, minlen == maxlen, 0, maxlen, cnt, chunk));
+    else  // two segments per row, the first one longer by an odd entry
+      out.push_back(make_step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt, chunk));
   }
 }
 
-void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, Partition& P, const StepShape& shape) {
+// Rows of step k of P.
+static int64_t rows_of(const int4& d) {
+  const int lanes = d.y & 0xff, mode = (d.y >> cgk::kStepModeShift) & 3;
+  return mode == cgk::kLanePerRow ? lanes : mode == cgk::kPairPerRow ? lanes / 2 : 1;
+}
+
+// Entries per lane of a chunk of step d.
+static int64_t chunk_size(const int4& d) { return (d.y >> cgk::kStepChunkShift) & 63; }
+
+void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, bool mixed, Partition& P,
+                     const StepShape& shape) {
+  const int chunk = mixed ? cgk::max_chunk<float>() : cgk::max_chunk<double>();
   P.step.clear();
-  P.step_mode.clear();
-  P.block_step.assign(static_cast<size_t>(nblocks) + 1, 0);
   P.block_row.assign(static_cast<size_t>(nblocks) + 1, 0);
   for (int b = 0; b <= nblocks; ++b) P.block_row[b] = static_cast<int32_t>(cost_split(rp, 0, n, b, nblocks));
   P.block_row[nblocks] = static_cast<int32_t>(n);
+  P.warp_step.clear();
+  std::vector<int4> rows;  // a CTA's steps in row order
   for (int b = 0; b < nblocks; ++b) {
-    P.block_step[b] = static_cast<int32_t>(P.step.size());
-    warp_steps(rp, P.block_row[b], P.block_row[b + 1], shape, P);
+    rows.clear();
+    warp_steps(rp, P.block_row[b], P.block_row[b + 1], chunk, shape, rows);
+    for (int w = 0; w < cgk::kWarps; ++w) {
+      P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
+      for (size_t k = static_cast<size_t>(w); k < rows.size(); k += cgk::kWarps) P.step.push_back(rows[k]);
+    }
   }
-  P.block_step[nblocks] = static_cast<int32_t>(P.step.size());
-  for (int t = 0; t < 2; ++t) {  // sentinels
-    P.step.push_back(make_int4(static_cast<int>(n), static_cast<int>(n), rp[n], rp[n]));
-    P.step_mode.push_back(cgk::kLanePerRow);
+  P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
+  P.chunks = 0;
+  for (const int4& d : P.step)
+    if (d.z > 0) P.chunks += (d.z + chunk_size(d) - 1) / chunk_size(d);
+  P.step.push_back(make_step(n, 32, cgk::kLanePerRow, true, 0, 0, 0, chunk));  // the sentinel: no entries
+}
+
+// Calls f(entries) for each chunk of step d, in order.
+template <typename F>
+static void for_chunks(const std::vector<int32_t>& rp, const int4& d, bool col16, F&& f) {
+  const int64_t size = chunk_size(d), lanes = d.y & 0xff, seg = d.z;
+  const int mode = (d.y >> cgk::kStepModeShift) & 3;
+  const bool padded = col16 && (d.y & cgk::kStepPadded), uniform = (d.y & cgk::kStepUniform) != 0;
+  for (int64_t u = 0; u < seg; u += size) {  // (size > 0 when seg is)
+    const int64_t cnt = std::min(size, seg - u);
+    if (padded) {
+      f(32 * cnt);
+    } else if (uniform) {
+      f(lanes * cnt);
+    } else if (mode == cgk::kLongRow) {  // all lanes but in the last, partial stride
+      const int64_t rem = (d.y >> cgk::kStepRemShift) & 0x3f;
+      f(u + cnt == seg ? 32 * (cnt - 1) + rem : 32 * cnt);
+    } else {
+      int64_t tot = 0;
+      const int64_t rows = rows_of(d);
+      for (int64_t i = d.x; i < d.x + rows; ++i) {
+        const int64_t len = rp[i + 1] - rp[i];
+        auto part = [&](int64_t l) { return std::max<int64_t>(0, std::min(l - u, cnt)); };
+        tot += mode == cgk::kLanePerRow ? part(len) : part((len + 1) / 2) + part(len / 2);
+      }
+      f(tot);
+    }
   }
+}
+
+void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool mixed, Partition& P) {
+  const size_t warps = static_cast<size_t>(nblocks) * cgk::kWarps;
+  P.step_chunk.assign(P.step.size(), 0);
+  P.step_entry.assign(mixed ? P.step.size() : 0, 0);
+  P.warp_chunk.assign(warps, int4{0, 0, 0, 0});
+  P.warp_entry.assign(mixed ? warps : 0, 0);
+  P.chunk_off.clear();
+  P.chunk_off.reserve(static_cast<size_t>(P.chunks) + 1);
+  int64_t at = 0, entry = 0;
+  for (size_t bw = 0; bw < warps; ++bw) {
+    const size_t c0 = P.chunk_off.size();
+    if (mixed) P.warp_entry[bw] = static_cast<uint32_t>(entry);
+    for (int k = P.warp_step[bw]; k < P.warp_step[bw + 1]; ++k) {
+      P.step_chunk[k] = static_cast<uint32_t>(P.chunk_off.size());
+      if (mixed) P.step_entry[k] = static_cast<uint32_t>(entry);
+      for_chunks(rp, P.step[k], col16, [&](int64_t cnt) {
+        P.chunk_off.push_back(static_cast<uint32_t>(at));
+        at += cgk::chunk_units(cnt, col16 ? 2 : 4, mixed ? 4 : 8);
+        entry += cnt;
+      });
+    }
+    P.warp_chunk[bw].x = static_cast<int32_t>(c0);
+    P.warp_chunk[bw].y = static_cast<int32_t>(P.chunk_off.size() - c0);
+  }
+  P.chunk_off.push_back(static_cast<uint32_t>(at));
+  for (int4& c : P.warp_chunk) {
+    c.z = static_cast<int32_t>(P.chunk_off[static_cast<size_t>(c.x)]);
+    c.w = static_cast<int32_t>(P.chunk_off[static_cast<size_t>(c.x) + (c.y > 0)]);
+  }
+  P.stream_units = at;
+  P.entries = entry;
+}
+
+void stream_bound(int64_t nnz, bool mixed, const Partition& P, int64_t* stream_units, int64_t* entries) {
+  // 32-bit columns without padding, or 16-bit ones with an eighth of it (less);
+  // at most a unit lost behind the columns and behind the values of a chunk
+  *stream_units = cgk::units((mixed ? 8 : 12) * nnz) + 2 * P.chunks;
+  *entries = nnz + nnz / 8;
 }
 
 }  // namespace cgh
@@ -130,15 +234,22 @@ struct cg_ctx {
   int max_rows = 0;  // most rows in one CTA's range
   int cluster_R = 0;  // > 0: cg_solve runs the cluster kernel, R rows and E entries per CTA
   int cluster_E = 0;
-  // device memory owned by the handle
-  int32_t* d_row_ptr = nullptr;
-  int32_t* d_col = nullptr;
-  double* d_val = nullptr;
-  float* d_val32 = nullptr;
+  bool col16 = false;  // columns stored as 16-bit offsets
+  // device memory owned by the handle: the matrix in stream order
+  unsigned char* d_stream = nullptr;
+  double* d_val64 = nullptr;
   int4* d_step = nullptr;
-  int32_t* d_step_mode = nullptr;
-  int32_t* d_block_step = nullptr;
+  int32_t* d_step_cmax = nullptr;
+  uint8_t* d_seg_len = nullptr;
+  uint32_t* d_chunk_off = nullptr;
+  int4* d_warp_chunk = nullptr;
+  uint32_t* d_warp_entry = nullptr;
+  int32_t* d_warp_step = nullptr;
   int32_t* d_block_row = nullptr;
+  // the CSR arrays (0-based), kept for the cluster kernel only
+  int32_t* d_csr_row_ptr = nullptr;
+  int32_t* d_csr_col = nullptr;
+  double* d_csr_val = nullptr;
   double* d_r = nullptr;
   double* d_p = nullptr;
   double* d_q = nullptr;
@@ -210,19 +321,23 @@ bool is_device_ptr(const void* p) {
 
 cgk::DevCsr dev_view(const cg_ctx* h) {
   cgk::DevCsr A;
-  A.row_ptr = h->d_row_ptr;
-  A.col_idx = h->d_col;
-  A.val = h->d_val;
-  A.val32 = h->d_val32;
+  A.stream = h->d_stream;
+  A.val64 = h->d_val64;
   A.step = h->d_step;
-  A.step_mode = h->d_step_mode;
-  A.block_step = h->d_block_step;
+  A.step_cmax = h->d_step_cmax;
+  A.seg_len = h->d_seg_len;
+  A.chunk_off = h->d_chunk_off;
+  A.warp_chunk = h->d_warp_chunk;
+  A.warp_entry = h->d_warp_entry;
+  A.warp_step = h->d_warp_step;
   A.block_row = h->d_block_row;
   A.n = static_cast<int32_t>(h->n);
   A.nsteps = h->nsteps;
   A.nblocks = h->nblocks;
   A.max_rows = h->max_rows;
   A.nnz = h->nnz;
+  A.col16 = h->col16 ? 1 : 0;
+  A.pad = 0;
   return A;
 }
 
@@ -472,8 +587,16 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   }
 
   Partition part;
-  build_partition(rp, n, h->nblocks, part);
-  h->nsteps = static_cast<int>(part.step.size()) - 2;
+  const bool mixed = o.precision == CG_PREC_MIXED;
+  // A system of at most 16 rows per warp of the whole GPU: two lanes per row, so
+  // that more warps work and each row's FMA chain, which bounds so small a
+  // product, is half as long.  By the size alone, so that a product's bits do not
+  // depend on the CTA count.
+  cgh::StepShape shape;
+  if (n <= static_cast<int64_t>(sms) * 16 * cgk::kWarps)
+    for (int L = 0; L <= cgk::kLaneMax; ++L) shape.mode[L] = static_cast<int8_t>(cgk::kPairPerRow);
+  build_partition(rp, n, h->nblocks, mixed, part, shape);
+  h->nsteps = static_cast<int>(part.step.size()) - 1;
   for (int b = 0; b < h->nblocks; ++b)
     h->max_rows = std::max(h->max_rows, part.block_row[b + 1] - part.block_row[b]);
   // Small plain FP64 systems (the CTA count left automatic): one cluster of
@@ -496,13 +619,10 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
     }
   }
 
-  const size_t pad = cgk::kPadEntries;
-  CG_TRY(dalloc(h, &h->d_row_ptr, n + 1), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_col, nnz + pad), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_val, nnz + pad), "cg_create: cudaMalloc");
   CG_TRY(dalloc(h, &h->d_step, part.step.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_step_mode, part.step_mode.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_block_step, part.block_step.size()), "cg_create: cudaMalloc");
+  CG_TRY(dalloc(h, &h->d_step_cmax, part.step.size()), "cg_create: cudaMalloc");
+  CG_TRY(dalloc(h, &h->d_seg_len, 32 * static_cast<size_t>(h->nsteps) + 64), "cg_create: cudaMalloc");
+  CG_TRY(dalloc(h, &h->d_warp_step, part.warp_step.size()), "cg_create: cudaMalloc");
   CG_TRY(dalloc(h, &h->d_block_row, part.block_row.size()), "cg_create: cudaMalloc");
   CG_TRY(dalloc(h, &h->d_r, n), "cg_create: cudaMalloc");
   CG_TRY(dalloc(h, &h->d_p, n), "cg_create: cudaMalloc");
@@ -516,56 +636,117 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
     h->d_ctrl = reinterpret_cast<cgk::SolveCtrl*>(blk);
     h->d_flags = reinterpret_cast<unsigned long long*>(blk + ctrl_flags_offset());
   }
-  CG_TRY(dalloc(h, &h->d_err, 4), "cg_create: cudaMalloc");
+  CG_TRY(dalloc(h, &h->d_err, 16), "cg_create: cudaMalloc");
   if (o.precision == CG_PREC_MIXED) {
-    CG_TRY(dalloc(h, &h->d_val32, nnz + pad), "cg_create: cudaMalloc");
     CG_TRY(dalloc(h, &h->d_p32, n), "cg_create: cudaMalloc");
   }
   if (o.preconditioner == CG_PRECOND_JACOBI) CG_TRY(dalloc(h, &h->d_dinv, n), "cg_create: cudaMalloc");
   CG_TRY(cudaMallocHost(&h->h_ctrl, sizeof(cgk::SolveCtrl)), "cg_create: cudaMallocHost");
 
-  CG_TRY(cudaMemcpy(h->d_row_ptr, rp.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice), "cg_create: upload");
-  CG_TRY(cudaMemset(h->d_col, 0, sizeof(int32_t) * (nnz + pad)), "cg_create: memset");
-  CG_TRY(cudaMemset(h->d_val, 0, sizeof(double) * (nnz + pad)), "cg_create: memset");
-  if (nnz > 0) {
-    if (!ci.empty())
-      CG_TRY(cudaMemcpy(h->d_col, ci.data(), sizeof(int32_t) * nnz, cudaMemcpyHostToDevice), "cg_create: upload");
-    else
-      CG_TRY(cudaMemcpy(h->d_col, csr->col_idx, sizeof(int32_t) * nnz, cudaMemcpyDeviceToDevice),
-             "cg_create: upload");
-    CG_TRY(cudaMemcpy(h->d_val, csr->val, sizeof(double) * nnz,
-                      csr->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
-           "cg_create: upload");
-  }
   CG_TRY(cudaMemcpy(h->d_step, part.step.data(), sizeof(int4) * part.step.size(), cudaMemcpyHostToDevice),
          "cg_create: upload");
-  CG_TRY(cudaMemcpy(h->d_step_mode, part.step_mode.data(), sizeof(int32_t) * part.step_mode.size(),
-                    cudaMemcpyHostToDevice),
-         "cg_create: upload");
-  CG_TRY(cudaMemcpy(h->d_block_step, part.block_step.data(), sizeof(int32_t) * part.block_step.size(),
+  CG_TRY(cudaMemcpy(h->d_warp_step, part.warp_step.data(), sizeof(int32_t) * part.warp_step.size(),
                     cudaMemcpyHostToDevice),
          "cg_create: upload");
   CG_TRY(cudaMemcpy(h->d_block_row, part.block_row.data(), sizeof(int32_t) * part.block_row.size(),
                     cudaMemcpyHostToDevice),
          "cg_create: upload");
-  CG_TRY(cudaMemset(h->d_err, 0, 16), "cg_create: memset");
-  if (o.precision == CG_PREC_MIXED) {
-    CG_TRY(cudaMemset(h->d_val32, 0, sizeof(float) * (nnz + pad)), "cg_create: memset");
-    if (nnz > 0) CG_TRY(cgk::launch_f64_to_f32(nnz, h->d_val, h->d_val32, nullptr), "cg_create: FP32 copy");
-  }
-  if (o.preconditioner == CG_PRECOND_JACOBI) {
-    CG_TRY(cgk::launch_jacobi_dinv(h->d_row_ptr, h->d_col, h->d_val, n, h->d_dinv, h->d_err, nullptr),
-           "cg_create: Jacobi diagonal");
-    int32_t bad_row = 0;
-    CG_TRY(cudaMemcpy(&bad_row, h->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost), "cg_create: read-back");
-    if (bad_row != 0) {
-      release(h);
-      delete h;
-      return fail(nullptr, CG_EINVAL, "cg_create: Jacobi preconditioner: diagonal of row " +
-                                          std::to_string(bad_row - 1) + " is not positive (A is not SPD)");
+  CG_TRY(cudaMemset(h->d_err, 0, 64), "cg_create: memset");
+
+  // The CSR arrays on the device for the time of the conversion: the caller's
+  // own where they are there already, else copies that go when this returns.
+  // The cluster kernel keeps 0-based copies.
+  std::vector<void*> temps;
+  auto temp_of = [&](const void* src, size_t bytes, cudaMemcpyKind kind, const void** out) -> cudaError_t {
+    void* q = nullptr;
+    cudaError_t et = cudaMalloc(&q, bytes ? bytes : 16);
+    if (et != cudaSuccess) return et;
+    temps.push_back(q);
+    *out = q;
+    return bytes ? cudaMemcpy(q, src, bytes, kind) : cudaSuccess;
+  };
+  struct TempGuard {
+    std::vector<void*>& v;
+    ~TempGuard() {
+      for (void* q : v) cudaFree(q);
     }
-    CG_TRY(cudaMemset(h->d_err, 0, 16), "cg_create: memset");
+  } temp_guard{temps};
+  const bool keep_csr = h->cluster_R > 0;
+  cgk::CsrSource src{};
+  src.base = base;
+  {
+    const void* q = nullptr;
+    CG_TRY(temp_of(rp.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, &q), "cg_create: upload");
+    src.row_ptr = static_cast<const int32_t*>(q);
+    if (csr->on_device && !(keep_csr && base != 0)) {
+      src.col_idx = csr->col_idx;
+    } else {
+      CG_TRY(temp_of(ci.data(), sizeof(int32_t) * nnz, cudaMemcpyHostToDevice, &q), "cg_create: upload");
+      src.col_idx = static_cast<const int32_t*>(q);
+      src.base = 0;  // ci is rebased
+    }
+    if (csr->on_device) {
+      src.val = csr->val;
+    } else {
+      CG_TRY(temp_of(csr->val, sizeof(double) * nnz, cudaMemcpyHostToDevice, &q), "cg_create: upload");
+      src.val = static_cast<const double*>(q);
+    }
   }
+  if (keep_csr) {
+    CG_TRY(dalloc(h, &h->d_csr_row_ptr, n + 1), "cg_create: cudaMalloc");
+    CG_TRY(dalloc(h, &h->d_csr_col, nnz), "cg_create: cudaMalloc");
+    CG_TRY(dalloc(h, &h->d_csr_val, nnz), "cg_create: cudaMalloc");
+    CG_TRY(cudaMemcpyAsync(h->d_csr_row_ptr, src.row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToDevice, nullptr),
+           "cg_create: copy");
+    if (nnz > 0) {
+      CG_TRY(cudaMemcpyAsync(h->d_csr_col, src.col_idx, sizeof(int32_t) * nnz, cudaMemcpyDeviceToDevice, nullptr),
+             "cg_create: copy");
+      CG_TRY(cudaMemcpyAsync(h->d_csr_val, src.val, sizeof(double) * nnz, cudaMemcpyDeviceToDevice, nullptr),
+             "cg_create: copy");
+    }
+  }
+  // d_q holds the steps' places in the streams until the handle's first solve
+  // (a step has at least one row: two words of 4 bytes in its 8)
+  static_assert(sizeof(double) >= 2 * sizeof(uint32_t), "step_chunk and step_entry fit q");
+  uint32_t* const d_step_chunk = reinterpret_cast<uint32_t*>(h->d_q);
+  uint32_t* const d_step_entry = d_step_chunk + h->nsteps;
+  cgk::LayoutScan* const d_scan = reinterpret_cast<cgk::LayoutScan*>(h->d_err + 4);
+  CG_TRY(cgk::launch_layout_scan(src, h->d_step, h->d_seg_len, h->d_step_cmax, 0, h->nsteps, n, false, d_scan, nullptr),
+         "cg_create: column scan");
+  if (o.preconditioner == CG_PRECOND_JACOBI)
+    CG_TRY(cgk::launch_jacobi_dinv(src, 0, n, h->d_dinv, h->d_err, nullptr),
+           "cg_create: Jacobi diagonal");
+  struct {
+    int32_t err[4];
+    cgk::LayoutScan scan;
+  } found{};
+  CG_TRY(cudaMemcpy(&found, h->d_err, sizeof(found), cudaMemcpyDeviceToHost), "cg_create: read-back");
+  if (found.err[0] != 0) {
+    release(h);
+    delete h;
+    return fail(nullptr, CG_EINVAL, "cg_create: Jacobi preconditioner: diagonal of row " +
+                                        std::to_string(found.err[0] - 1) + " is not positive (A is not SPD)");
+  }
+  h->col16 = found.scan.span <= cgk::kColSpan16;
+  cgh::place_steps(rp, h->nblocks, h->col16, mixed, part);
+  CG_TRY(dalloc(h, &h->d_stream, static_cast<size_t>(part.stream_units) * cgk::kUnit), "cg_create: cudaMalloc");
+  CG_TRY(dalloc(h, &h->d_chunk_off, part.chunk_off.size()), "cg_create: cudaMalloc");
+  CG_TRY(dalloc(h, &h->d_warp_chunk, part.warp_chunk.size()), "cg_create: cudaMalloc");
+  auto up = [&](void* dst, const auto& v, size_t count) {
+    return count ? cudaMemcpy(dst, v.data(), sizeof(v[0]) * count, cudaMemcpyHostToDevice) : cudaSuccess;
+  };
+  CG_TRY(up(h->d_chunk_off, part.chunk_off, part.chunk_off.size()), "cg_create: upload");
+  CG_TRY(up(h->d_warp_chunk, part.warp_chunk, part.warp_chunk.size()), "cg_create: upload");
+  CG_TRY(up(d_step_chunk, part.step_chunk, static_cast<size_t>(h->nsteps)), "cg_create: upload");
+  if (mixed) {
+    CG_TRY(dalloc(h, &h->d_val64, static_cast<size_t>(part.entries)), "cg_create: cudaMalloc");
+    CG_TRY(dalloc(h, &h->d_warp_entry, part.warp_entry.size()), "cg_create: cudaMalloc");
+    CG_TRY(up(h->d_warp_entry, part.warp_entry, part.warp_entry.size()), "cg_create: upload");
+    CG_TRY(up(d_step_entry, part.step_entry, static_cast<size_t>(h->nsteps)), "cg_create: upload");
+  }
+  const cgk::StreamPlace to{h->d_chunk_off, d_step_chunk, d_step_entry, h->d_stream, h->d_val64};
+  CG_TRY(cgk::launch_layout_fill(src, h->d_step, to, 0, h->nsteps, h->col16, mixed, nullptr),
+         "cg_create: stream order");
   CG_TRY(cudaDeviceSynchronize(), "cg_create: synchronize");
 #undef CG_TRY
   *out = h;
@@ -796,13 +977,13 @@ int cg_solve(cg_handle h, const double* b, double* x, double tol, int64_t maxit,
   P.replace_every = h->replace_every;
   P.wait_limit_ns = h->wait_limit_ns;
   P.group = h->nblocks;
-  P.stream_rows = cgk::stream_row_ptrs(
+  P.stream_rows = cgk::stream_row_tables(
       cgk::step_reused_bytes(h->n, h->precision == CG_PREC_MIXED, h->d_dinv != nullptr), l2_bytes(h->device));
   P.chunk_iters = 0;
   P.dinv = h->d_dinv;
   P.flags = h->nblocks > 1 ? h->d_flags : nullptr;
   if (h->cluster_R > 0)
-    e = cgk::launch_cluster_solve(h->d_row_ptr, h->d_col, h->d_val, db, dx, h->d_ctrl, tol, maxit,
+    e = cgk::launch_cluster_solve(h->d_csr_row_ptr, h->d_csr_col, h->d_csr_val, db, dx, h->d_ctrl, tol, maxit,
                                   static_cast<int32_t>(h->n), h->cluster_R, h->cluster_E, h->stream);
   else
     e = cgk::launch_solve(P, h->precision == CG_PREC_MIXED, h->stream);

@@ -80,26 +80,27 @@ __device__ __forceinline__ int ld_volatile_i32(const int32_t* p) {
   return *reinterpret_cast<const volatile int32_t*>(p);
 }
 
-// Barrier of the consumer warps only (named barrier 1): the producer warp of
-// a solve CTA never takes part in CTA-wide synchronisation.
-__device__ __forceinline__ void cta_sync() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kConsumers) : "memory");
+// Barrier of the computing warps only (named barrier 1): the producer warp
+// takes no part in it.
+__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kBlock) : "memory"); }
+
+__device__ __forceinline__ void st_release_shared(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
 
-// AND of a per-thread condition over the consumer warps (named barrier 1).
-// Every consumer thread must reach it; used after each product pass so that a
-// warp that gave up on a wait and the others leave the kernel together.
-__device__ __forceinline__ bool cta_and(bool v) {
-  int r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.s32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, 1, %2, p;\n\t"
-      "selp.s32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"(static_cast<int>(v)), "n"(kConsumers)
-      : "memory");
-  return r != 0;
+__device__ __forceinline__ uint32_t ld_acquire_shared(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+
+// threadIdx.x, read anew: what is computed from it is not kept in registers
+// from one pass over the matrix to the next (the compiler would move it out of
+// the step loop, and spill it).
+__device__ __forceinline__ int fresh_tid() {
+  int t;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+  return t;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -173,9 +174,9 @@ __device__ __forceinline__ FxPart fx_warp(double v) {
 
 // Sum of up to 32 partials, one per lane (`valid` lanes), realigned to the
 // largest exponent (each partial rounded once, to nearest, ties away from
-// zero) and converted to double once.  The result depends only on the
-// partials, not on their order.  Every lane gets it.
-__device__ __forceinline__ double fx_combine(FxPart p, bool valid) {
+// zero).  The result depends only on the partials, not on their order.  Every
+// lane gets it.
+__device__ __forceinline__ FxPart fx_combine(FxPart p, bool valid) {
   const int E = static_cast<int>(__reduce_max_sync(0xffffffffu, valid ? static_cast<unsigned int>(p.e) : 0u));
   const int nf = __any_sync(0xffffffffu, valid && p.nf);
   long long m = 0;
@@ -191,9 +192,24 @@ __device__ __forceinline__ double fx_combine(FxPart p, bool valid) {
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  if (nf) return __longlong_as_double(0x7ff8000000000000ll);
-  if (E == 0) return 0.0;
-  return ldexp(static_cast<double>(m), E - 1074);
+  return FxPart{m, E, nf};
+}
+
+// m 2^k for a double m of magnitude below 2^64 (an integer's conversion), by its
+// exponent field where the result is a normal number (ldexp takes four FP64
+// operations one after another).
+__device__ __forceinline__ double fx_scale(double m, int k) {
+  const long long bits = __double_as_longlong(m);
+  const int e = static_cast<int>((bits >> 52) & 0x7ff);
+  if (e != 0 && e + k > 0 && e + k < 2047) return __longlong_as_double(bits + (static_cast<long long>(k) << 52));
+  return ldexp(m, k);
+}
+
+// The double nearest to a partial.
+__device__ __forceinline__ double fx_value(FxPart p) {
+  if (p.nf) return __longlong_as_double(0x7ff8000000000000ll);
+  if (p.e == 0) return 0.0;
+  return fx_scale(static_cast<double>(p.m), p.e - 1074);
 }
 
 // Exact fixed-point sum, over the calling warp, of src[0 .. count), read
@@ -270,9 +286,121 @@ __device__ __forceinline__ double fx_warp_sum_array(const double* src, int count
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  if (nf) return __longlong_as_double(0x7ff8000000000000ll);
-  if (E == 0) return 0.0;
-  return ldexp(static_cast<double>(m), E - 1074);
+  return fx_value(FxPart{m, E, nf});
+}
+
+// ---- sums through accumulators
+//
+// A group sum costs, beyond its arithmetic, what the CTAs' meeting costs.  The
+// general form (publish a value, meet at the barrier, read all values) takes a
+// fence before the arrival, a fence behind it and one more trip to the L2, and
+// the two sums of a CG step need none of that: the data they order is the sum
+// itself.  Here every CTA adds its value, as an integer, into two 64-bit words
+// with relaxed atomics, and a count of arrivals travels in the same words: who
+// sees all arrivals has the sum.  Integer addition commutes, so every CTA gets
+// the same bits.  The words are never cleared: a CTA keeps what it saw last and
+// takes the difference; a word is used again only after another such sum, which
+// every CTA enters with the last one read.
+//
+// The integers' unit is set by the last sum of the same kind, of biased exponent
+// eb: 2^(eb - 1085), i.e. that sum was about 2^62 units.  A CTA's value is
+// rounded to a unit (152 of them: 2^-54 of a sum as large as the last).  Values
+// of up to 2^73 units go in (growth by 2^11), split in a signed high part (53
+// bits) and 32 low bits; anything else, or a sum that came out below 2^54 units
+// (its precision would suffer), makes every CTA take the general form instead.
+// Low word: 42 bits of low parts, 11 of CTAs that could not add theirs, 11 of
+// arrivals; high word: 53 bits of high parts, 11 of arrivals.
+constexpr int kAccUnit = 1085;
+constexpr unsigned int kAccCount = 0x7ff;  // most CTAs of a group: 1024 (cg_create)
+
+// What a CTA adds for the partial p.
+__device__ __forceinline__ void acc_words(FxPart p, int eb, unsigned long long* lo, unsigned long long* hi) {
+  const unsigned long long a = static_cast<unsigned long long>(p.m < 0 ? -p.m : p.m);
+  const int sh = p.e - 1074 - (eb - kAccUnit);  // p is m 2^sh units
+  unsigned long long l = 0, h = 0;
+  bool fits = p.nf == 0;
+  if (a != 0) {
+    if (sh >= 0) {
+      fits = fits && 64 - __clzll(static_cast<long long>(a)) + sh <= 73;
+      if (fits) {  // (then sh < 74)
+        l = sh < 64 ? a << sh : 0ull;
+        h = sh == 0 ? 0ull : sh < 64 ? a >> (64 - sh) : a << (sh - 64);
+      }
+    } else if (sh > -64) {
+      l = (a + (1ull << (-sh - 1))) >> -sh;
+    }
+  }
+  if (p.m < 0) {  // two's complement
+    l = ~l + 1ull;
+    h = ~h + (l == 0 ? 1ull : 0ull);
+  }
+  const unsigned long long high = (h << 32) | (l >> 32);
+  *lo = ((l & 0xffffffffull) << 22) + 1ull;
+  *hi = (high << 11) + 1ull;
+  if (!fits) {
+    *lo = (1ull << 11) + 1ull;
+    *hi = 1ull;
+  }
+}
+
+// The sum that the words' differences hold (all arrivals in); false if the
+// general form has to give it.
+__device__ __forceinline__ bool acc_sum(unsigned long long lo, unsigned long long hi, unsigned int count, int eb,
+                                        double* sum) {
+  if ((lo >> 11) & kAccCount) return false;
+  const long long high = static_cast<long long>(hi - count) >> 11;
+  const unsigned long long low = lo >> 22;
+  unsigned long long l = (static_cast<unsigned long long>(high) << 32) + low;
+  unsigned long long h = static_cast<unsigned long long>(high >> 32) + (l < low ? 1ull : 0ull);
+  const bool neg = (h >> 63) != 0;
+  if (neg) {
+    l = ~l + 1ull;
+    h = ~h + (l == 0 ? 1ull : 0ull);
+  }
+  int k = 0;
+  if (h != 0) {  // the leading 64 bits, the rest as a sticky bit
+    k = 64 - __clzll(static_cast<long long>(h));
+    const unsigned long long rest = l << (64 - k);
+    l = (h << (64 - k)) | (l >> k) | (rest != 0 ? 1ull : 0ull);
+  }
+  if (k == 0 && l < (1ull << 54)) return false;
+  const double v = __ull2double_rn(l);
+  const long long bits = __double_as_longlong(v);
+  const int add = k + eb - kAccUnit, e = static_cast<int>(bits >> 52) + add;
+  if (e <= 0 || e >= 2047) return false;
+  const double r = __longlong_as_double(bits + (static_cast<long long>(add) << 52));
+  *sum = neg ? -r : r;
+  return true;
+}
+
+// Biased exponent of a sum that the next one of its kind can be measured by (0: none).
+__device__ __forceinline__ int acc_exponent(double v) {
+  const int e = static_cast<int>((__double_as_longlong(v) >> 52) & 0x7ff);
+  return e == 0x7ff ? 0 : e;
+}
+
+// Waits until the words at `word` hold `count` arrivals more than lo0, hi0; *lo
+// and *hi get their values.  Returns false after a wait longer than limit_ns or
+// an abort raised by another CTA.
+__device__ __forceinline__ bool acc_wait(SolveCtrl* ctrl, const unsigned long long* word, unsigned long long lo0,
+                                         unsigned long long hi0, unsigned int count, unsigned long long limit_ns,
+                                         unsigned long long* lo, unsigned long long* hi) {
+  unsigned long long t0 = 0;
+  uint32_t spins = 0;
+  for (;;) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(*lo), "=l"(*hi) : "l"(word) : "memory");
+    if (((*lo - lo0) & kAccCount) == count && ((*hi - hi0) & kAccCount) == count) return true;
+    if ((++spins & 255u) == 0) {
+      if (*reinterpret_cast<const volatile int32_t*>(&ctrl->abort)) return false;
+      const unsigned long long now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > limit_ns) {
+        atomicExch(&ctrl->abort, 1);
+        atomicExch(&ctrl->timeout_site, kAccSite);
+        return false;
+      }
+    }
+  }
 }
 
 // Arrival and bounded wait of thread 0 at the group barrier of a system
@@ -317,7 +445,24 @@ __device__ __forceinline__ bool group_barrier_t0(SolveCtrl* ctrl, unsigned long 
 // Per-CTA state of a solve, in shared memory: written by thread 0 (between
 // CTA barriers), read by all.  Keeping it out of registers leaves the
 // product in the step loop the registers it needs.
+// What a product reads and writes besides the warp's ring.  In shared memory and
+// read where it is used: the product's registers hold what it gathers.
+struct PassIo {
+  const int4* step;
+  const uint8_t* seg_len;
+  const double* aux;           // with_dot: the vector whose product with the result is summed
+  double* out;
+  unsigned long long limit_ns;
+  int32_t nsteps;
+  int32_t stream_rows;         // tables with the evict-first policy
+};
+__device__ __forceinline__ PassIo pass_io(const DevCsr& A, int32_t stream_rows, const double* aux, double* out,
+                                          unsigned long long limit_ns) {
+  return PassIo{A.step, A.seg_len, aux, out, limit_ns, A.nsteps, stream_rows};
+}
+
 struct CtaState {
+  PassIo io;
   double rho;                  // r.z (r.r without a preconditioner)
   double rr;                   // r.r of the current iterate
   double bnorm2;               // b.b
@@ -330,9 +475,13 @@ struct CtaState {
   int32_t site;                // diagnostics: group waits so far
   int32_t ok;                  // the last group sum or barrier succeeded
   int32_t flags;               // kFlag* below
+  int32_t pass;                // what the next product is for (kPass* below)
+  unsigned long long acc_seen[3][2];  // accumulators p.q, r.r, r.z: their words when last summed
+  int32_t acc_exp[3];                 // and the exponents of those sums (0: none yet)
   int32_t dep_lo, dep_hi;      // CTAs whose rows this CTA's columns reach (columns first, then ranks)
 };
-enum : int32_t { kFlagDone = 1, kFlagBreakdown = 2, kFlagReplace = 4, kFlagResumed = 8 };
+enum : int32_t { kFlagDone = 1, kFlagBreakdown = 2, kFlagReplace = 4 };
+enum : int32_t { kPassSetup, kPassStep, kPassReplace, kPassEnd };
 
 // Warp partials of a CTA sum (up to three values per thread) and each
 // warp's vote.
@@ -342,90 +491,88 @@ struct SumScratch {
   int32_t ok[kWarps];
 };
 
-// Dynamic shared memory of a persistent CTA: the value ring (values of vb
-// bytes: 8 for FP64, 4 for FP32, so that an FP32 stream leaves more of the
-// SM's 256 KB to L1 for the gathers) and the column-index ring, each followed
-// by its kMirror-entry mirror, the full/empty mbarriers of every slot, the
-// CTA state of a solve, the warp partials of its sums, a few words (stop
-// flag), and in the small-share solve the r of the CTA's rows.
+// A warp's stream of the matrix: the chunks of its steps, one after another,
+// pass after pass, through the slots of its ring.  The warp's side of it,
+// kept here between passes:
+struct WarpStream {
+  uint32_t consumed;  // chunks of this task the warp is done with (read by the producer)
+  uint32_t phases;    // the parity that each slot's barrier completes next (a bit per slot)
+  int32_t tail;       // slot of the next chunk
+  int32_t failed;     // a wait gave up
+  // its first two steps and the lanes' segment lengths: every pass begins with
+  // them, and a load from L2 there would be on its critical path
+  int4 step[2];
+  uint8_t seg_len[2][32];
+};
+
+// Dynamic shared memory of a persistent CTA: the full mbarrier of every ring
+// slot, the CTA state of a solve, the warp partials of its sums, then the rings
+// (values of type T, columns of type C) of every warp, and in the small-share
+// solve the r of the CTA's rows.  The parts before the rings sit at the same
+// place whatever T and C are.
+constexpr int kMaxSlots = 5;  // of any ring: the place of the barriers
+
+template <typename T, typename C>
 struct RingSmem {
-  static constexpr int kRingAlloc = kRing + kMirror;
-  static constexpr size_t kColBytes = sizeof(int32_t) * kRingAlloc;
-  static constexpr size_t kStateBytes = (sizeof(CtaState) + 15) & ~size_t(15);
-  static constexpr size_t kSumBytes = (sizeof(SumScratch) + 15) & ~size_t(15);
-  __host__ __device__ static constexpr size_t bar_off(size_t vb) {
-    return (vb * kRingAlloc + kColBytes + 15) & ~size_t(15);
-  }
-  __host__ __device__ static constexpr size_t state_off(size_t vb) { return bar_off(vb) + 16 * kSlots; }
-  __host__ __device__ static constexpr size_t sum_off(size_t vb) { return state_off(vb) + kStateBytes; }
-  __host__ __device__ static constexpr size_t misc_off(size_t vb) { return sum_off(vb) + kSumBytes; }
-  // Bytes of the whole layout for ring values of vb bytes.
-  __host__ __device__ static constexpr size_t bytes(size_t vb) { return misc_off(vb) + 64; }
+  using Val = T;
+  using Col = C;
+  static constexpr int kSlots = ring_slots<T, C>();
+  static_assert(kSlots <= kMaxSlots, "barriers");
+  static constexpr int kSlotBytes = static_cast<int>(kUnit * chunk_units(32 * max_chunk<T>(), sizeof(C), sizeof(T)));
+  static constexpr size_t kStateOff = (8 * kMaxSlots * kWarps + 15) & ~size_t(15);
+  static constexpr size_t kSumOff = kStateOff + ((sizeof(CtaState) + 15) & ~size_t(15));
+  static constexpr size_t kStreamOff = (kSumOff + sizeof(SumScratch) + 15) & ~size_t(15);
+  static constexpr size_t kRingOff = (kStreamOff + sizeof(WarpStream) * kWarps + 16 + 127) & ~size_t(127);
+  static constexpr size_t kBytes = kRingOff + static_cast<size_t>(kSlotBytes) * kSlots * kWarps;
 
   unsigned char* base;
-  uint32_t vb = sizeof(double);  // bytes per value in the ring
-  template <typename T>
-  __device__ T* val() const { return reinterpret_cast<T*>(base); }
-  __device__ int32_t* col() const { return reinterpret_cast<int32_t*>(base + static_cast<size_t>(vb) * kRingAlloc); }
-  __device__ uint64_t* full(int s) const { return reinterpret_cast<uint64_t*>(base + bar_off(vb)) + s; }
-  __device__ uint64_t* empty(int s) const { return reinterpret_cast<uint64_t*>(base + bar_off(vb)) + kSlots + s; }
-  __device__ CtaState* state() const { return reinterpret_cast<CtaState*>(base + state_off(vb)); }
-  __device__ SumScratch* sums() const { return reinterpret_cast<SumScratch*>(base + sum_off(vb)); }
-  __device__ int32_t* flag() const { return reinterpret_cast<int32_t*>(base + misc_off(vb)); }
-  __device__ int32_t* stop() const { return reinterpret_cast<int32_t*>(base + misc_off(vb) + 4); }
-  __device__ double* scalars() const { return reinterpret_cast<double*>(base + misc_off(vb) + 16); }
-  // r of the CTA's rows in a small-share solve, behind the layout
-  // (kLocalRows entries).
-  __device__ double* local() const { return reinterpret_cast<double*>(base + bytes(vb)); }
+  __device__ unsigned char* slot(int w, int s) const { return base + kRingOff + (w * kSlots + s) * kSlotBytes; }
+  __device__ uint64_t* full(int w, int slot) const { return reinterpret_cast<uint64_t*>(base) + w * kMaxSlots + slot; }
+  __device__ WarpStream* stream(int w) const { return reinterpret_cast<WarpStream*>(base + kStreamOff) + w; }
+  __device__ int32_t* stop() const { return reinterpret_cast<int32_t*>(base + kStreamOff + sizeof(WarpStream) * kWarps); }
+  __device__ CtaState* state() const { return reinterpret_cast<CtaState*>(base + kStateOff); }
+  __device__ SumScratch* sums() const { return reinterpret_cast<SumScratch*>(base + kSumOff); }
+  // r of the CTA's rows in a small-share solve, behind the rings (kLocalRows entries).
+  __device__ double* local() const { return reinterpret_cast<double*>(base + kBytes); }
 };
 
-// Dynamic shared memory of the kernels whose step-loop product streams
-// values of type T; `local`: with the small-share solve's r.
-template <typename T>
+// Dynamic shared memory of a kernel whose step-loop product streams values of
+// type T and columns of type C; `local`: with the small-share solve's r.
+template <typename T, typename C>
 constexpr size_t ring_smem_bytes(bool local = false) {
-  return RingSmem::bytes(sizeof(T)) + (local ? sizeof(double) * kLocalRows : 0);
+  return RingSmem<T, C>::kBytes + (local ? sizeof(double) * kLocalRows : 0);
 }
 
-// The CTA's part of the matrix stream (identical in every thread).  Pieces
-// are numbered globally across passes (piece j of pass k is k * npieces + j);
-// global piece g sits in slot g % kSlots and completes phase g / kSlots of
-// that slot's full barrier.
-struct CtaStream {
-  int kb = 0;        // first entry of the CTA's range, rounded down to a multiple of 4
-  int ke = 0;        // end of the CTA's entry range
-  int npieces = 0;   // pieces per pass
-  int s0 = 0, s1 = 0;  // the CTA's steps [s0, s1)
-};
-
-__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
-  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Initialise the ring barriers for the CTA's share `rank` of A's partition
-// (all threads of the CTA call; ends with a full CTA barrier).  `reinit`:
-// the barriers hold a previous stream, already drained (a CTA taking another
-// task of a batched solve); they are invalidated first.
-__device__ __forceinline__ void stream_setup(const RingSmem& sm, CtaStream& cs, const DevCsr& A, int rank,
-                                             bool reinit = false) {
-  if (threadIdx.x < kSlots) {
-    if (reinit) {
-      mbar_inval(sm.full(threadIdx.x));
-      mbar_inval(sm.empty(threadIdx.x));
-    }
-    mbar_init(sm.full(threadIdx.x), 1);
-    mbar_init(sm.empty(threadIdx.x), kConsumerWarps);
+// Initialises every ring barrier and stream (all threads of the CTA call; ends
+// with a CTA barrier).  Once per kernel: the phases are kept count of through
+// all tasks.
+template <typename Ring>
+__device__ __forceinline__ void ring_init(const Ring& sm) {
+  if (threadIdx.x < kMaxSlots * kWarps) {
+    mbar_init(reinterpret_cast<uint64_t*>(sm.base) + threadIdx.x, 1);
+    fence_mbar_init();
+  }
+  if (threadIdx.x < kWarps) {
+    WarpStream* const ws = sm.stream(threadIdx.x);
+    ws->consumed = ws->phases = 0;
+    ws->tail = ws->failed = 0;
   }
   if (threadIdx.x == 0) *sm.stop() = 0;
-  if (threadIdx.x < kSlots) fence_mbar_init();
   __syncthreads();
-  cs.s0 = A.block_step[rank];
-  cs.s1 = A.block_step[rank + 1];
-  cs.kb = cs.ke = cs.npieces = 0;
-  if (cs.s1 > cs.s0) {
-    cs.kb = A.step[cs.s0].z & ~3;
-    cs.ke = A.step[cs.s1 - 1].w;
-    cs.npieces = (cs.ke - cs.kb + kPiece - 1) >> kPieceLog;
+}
+
+// Readies the streams for the CTA's next task (the last one's warps are all
+// through, the producer included; a CTA barrier follows before the streams are
+// used).
+template <typename Ring>
+__device__ __forceinline__ void ring_reset(const Ring& sm) {
+  if (threadIdx.x < kWarps) {
+    WarpStream* const ws = sm.stream(threadIdx.x);
+    ws->consumed = 0;
+    ws->tail = 0;
+    ws->failed = 0;
   }
+  if (threadIdx.x == 0) *sm.stop() = 0;
 }
 
 // Bounded wait on an mbarrier phase; false if it gave up.  If `stop` is
@@ -445,100 +592,150 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return true;
 }
 
-// Producer (one lane of the producer warp): stream the CTA's range pass after
-// pass (max_passes < 0: until told to stop) with values of type T.  Before
-// refilling a slot it waits for every consumer warp to release the slot's
-// previous piece.  On stop it waits for its copies still in flight, so no
-// bulk copy lands after the CTA is gone.  Returns false on a timeout.
-template <typename T>
-__device__ __forceinline__ bool producer_loop(const RingSmem& sm, const CtaStream& cs, const T* val,
-                                              const int32_t* col, int max_passes, unsigned long long limit_ns) {
-  bool ok = true;
-  uint32_t g = 0;
+// The producer warp of CTA `rank`: lane w copies the chunks of warp w's stream,
+// pass after pass (`once`: one pass), into its ring as the warp gives slots
+// back, until the computing warps say stop.  One lane per warp: a copy takes
+// some thirty instructions, which are no part of any computing warp's chain,
+// and all warps that wait for one are served together.  On stop every lane
+// waits for its copies in flight, so that none lands after the CTA is gone or
+// in a ring that the next task has taken over, and leaves the phases to that
+// task's warps.  Returns false (uniformly) if nothing moved for
+// limit_ns, or a copy did not arrive in that time.
+template <typename Ring>
+__device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int rank, bool once,
+                                         unsigned long long limit_ns) {
+  const int w = threadIdx.x & 31;
+  const bool mine = w < kWarps;
+  WarpStream* const ws = sm.stream(mine ? w : 0);
+  // the bounds of chunk `next`, and the ends of the two after it (the stream
+  // goes round: chunk nchunks is chunk 0 again), loaded ahead
+  int c0 = 0, nchunks = 0, next = 0;
+  uint32_t first = 0, start = 0, end0 = 0, end1 = 0, end2 = 0;
+  auto end_of = [&](int j) { return A.chunk_off[c0 + j % nchunks + 1]; };
+  if (mine) {
+    // (the first copy waits for this load alone)
+    const int4 c = A.warp_chunk[rank * kWarps + w];
+    c0 = c.x;
+    nchunks = c.y;
+    first = start = static_cast<uint32_t>(c.z);
+    end0 = static_cast<uint32_t>(c.w);
+    if (nchunks > 0) {
+      end1 = end_of(1);
+      end2 = end_of(2);
+    }
+  }
   const uint64_t pol = l2_evict_first_policy();
-  if (cs.npieces > 0) {
-    const int ke4 = (cs.ke + 3) & ~3;  // copy whole 16-byte groups (<= 3 padding entries)
-    for (int pass = 0; ok && (max_passes < 0 || pass < max_passes); ++pass) {
-      for (int j = 0; j < cs.npieces; ++j, ++g) {
-        const int slot = static_cast<int>(g % kSlots);
-        if (g >= kSlots && !mbar_wait_bounded(sm.empty(slot), ((g / kSlots) - 1) & 1u, limit_ns, sm.stop())) {
-          ok = ld_volatile_i32(sm.stop()) != 0;  // a stop is the normal way out
-          goto drain;
-        }
-        const int e0 = cs.kb + j * kPiece;
-        const int e1 = e0 + kPiece < ke4 ? e0 + kPiece : ke4;
-        const int pos = slot * kPiece;
-        const uint32_t bv = static_cast<uint32_t>(e1 - e0) * sizeof(T);
-        const uint32_t bc = static_cast<uint32_t>(e1 - e0) * 4u;
-        // slot 0 also fills the mirror behind the ring end with its first entries
-        const int nm = slot == 0 ? (e1 - e0 < kMirror ? e1 - e0 : kMirror) : 0;  // a multiple of 4
-        const uint32_t mv = static_cast<uint32_t>(nm) * sizeof(T), mc = static_cast<uint32_t>(nm) * 4u;
-        mbar_arrive_expect_tx(sm.full(slot), bv + bc + mv + mc);
-        bulk_g2s_hint(sm.val<T>() + pos, val + e0, bv, sm.full(slot), pol);
-        bulk_g2s_hint(sm.col() + pos, col + e0, bc, sm.full(slot), pol);
-        if (nm) {
-          bulk_g2s_hint(sm.val<T>() + kRing, val + e0, mv, sm.full(slot), pol);
-          bulk_g2s_hint(sm.col() + kRing, col + e0, mc, sm.full(slot), pol);
+  uint32_t phases = ws->phases, issued = 0;
+  int head = 0;
+  bool ok = true;
+  unsigned long long t0 = 0;
+  uint32_t idle = 0;
+  for (;;) {
+    const bool more = nchunks > 0 && (!once || issued < static_cast<uint32_t>(nchunks));
+    if (!__any_sync(0xffffffffu, more) || __any_sync(0xffffffffu, ld_volatile_i32(sm.stop()) != 0)) break;
+    const bool free = more && issued - ld_acquire_shared(&ws->consumed) < static_cast<uint32_t>(Ring::kSlots);
+    if (free) {
+      uint64_t* const bar = sm.full(w, head);
+      const uint32_t bytes = (end0 - start) * static_cast<uint32_t>(kUnit);
+      mbar_arrive_expect_tx(bar, bytes);
+      bulk_g2s_hint(sm.slot(w, head), A.stream + static_cast<size_t>(start) * kUnit, bytes, bar, pol);
+      phases ^= 1u << head;
+      head = head + 1 == Ring::kSlots ? 0 : head + 1;
+      ++issued;
+      next = next + 1 == nchunks ? 0 : next + 1;
+      start = next == 0 ? first : end0;
+      end0 = end1;
+      end1 = end2;
+      end2 = end_of(next + 2);
+    }
+    if (__any_sync(0xffffffffu, free)) {
+      idle = 0;
+    } else {
+      __nanosleep(32);
+      if ((++idle & 255u) == 0) {
+        const unsigned long long now = global_timer_ns();
+        if (idle == 256u) t0 = now;
+        else if (now - t0 > limit_ns) {
+          ok = false;
+          break;
         }
       }
     }
   }
-drain:
-  // the newest piece of every slot may still be in flight
-  for (uint32_t k = g > kSlots ? g - kSlots : 0; k < g; ++k)
-    mbar_wait_bounded(sm.full(k % kSlots), (k / kSlots) & 1u, limit_ns, nullptr);
+  if (mine) {
+    for (int k = 0; k < Ring::kSlots; ++k)  // the latest copy into each slot
+      if (issued > static_cast<uint32_t>(k))
+        ok = mbar_wait_bounded(sm.full(w, k), ((phases >> k) & 1u) ^ 1u, limit_ns, nullptr) && ok;
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  // (no computing warp reads its phases any more: in a solve they have said
+  // stop, a single pass keeps its own)
+  if (!once && mine && nchunks > 0) ws->phases = phases;
   return ok;
 }
 
-// Consumer-side position of the CTA in the stream (identical in all
-// consumer threads): global number of piece 0 of the next ring pass.
-struct ConsumerCursor {
-  uint32_t gbase = 0;
-};
-
-// Gathers of one lane's row segment: xv[u] = x[cp[u]] for its len entries,
-// cp pointing at the segment's column indices in the ring (contiguous thanks
-// to the mirror).  N is the step's longest per-lane segment (lanes with a
-// shorter segment, or none, are predicated off for the tail), so the code is
-// branch-free and no instruction is issued for a slot no lane needs.
-template <typename X, int N, int U>
-__device__ __forceinline__ void seg_gather_n(const int32_t* cp, int len, const X* x, X (&xv)[U]) {
-#pragma unroll
-  for (int u = 0; u < N; ++u)
-    if (u < len) xv[u] = x[cp[u]];
+// The computing warps of a task are through (all of their threads call).
+template <typename Ring>
+__device__ __forceinline__ void stop_producer(const Ring& sm) {
+  cta_sync();
+  if (threadIdx.x == 0) *reinterpret_cast<volatile int32_t*>(sm.stop()) = 1;
 }
 
-// Multiply-adds of a gathered segment, in storage order, with FMA.
-template <typename T, typename X, typename Acc, int N, int U>
-__device__ __forceinline__ Acc seg_fma_n(const T* vp, int len, const X (&xv)[U], Acc s) {
-#pragma unroll
-  for (int u = 0; u < N; ++u)
-    if (u < len) s = fma(Acc(vp[u]), Acc(xv[u]), s);
-  return s;
+// ---- steps
+
+__device__ __forceinline__ int step_lanes(const int4& d) { return d.y & 0xff; }
+__device__ __forceinline__ int step_mode(const int4& d) { return (d.y >> kStepModeShift) & 3; }
+
+__device__ __forceinline__ int step_chunk(const int4& d) { return (d.y >> kStepChunkShift) & 63; }
+
+// Whether step d is stored padded (with columns of type C).
+template <typename C>
+__device__ __forceinline__ bool step_padded(const int4& d) {
+  return sizeof(C) == 2 && (d.y & kStepPadded) != 0;
 }
 
-// The step's longest per-lane segment (1..32) selects the unrolled code once
-// per step (dispatch_tree below).
+// The tables that are read once per product: step s, and the length of this
+// lane's segment in it where the step itself does not tell.  io.stream_rows: with
+// the evict-first policy, so that in a solve whose vectors and tables together
+// outgrow the L2 the tables give way to the vectors that the step reads again.
+__device__ __forceinline__ int4 load_step(const PassIo& io, int s) {
+  return io.stream_rows ? __ldcs(io.step + s) : io.step[s];
+}
+__device__ __forceinline__ int load_seg_len(const PassIo& io, int s, int lane) {
+  const uint8_t* p = io.seg_len + static_cast<size_t>(s) * 32 + lane;
+  return io.stream_rows ? __ldcs(p) : *p;
+}
 
-// The multiply-adds of a lane's first 16 entries (xv holds their gathered
-// values), each followed by the gather of entry 16 + u into the register it
-// frees (N2 = entries of the second batch the step needs, at most 16): the
-// second batch's loads are in flight during the first batch's FMA chain.
-template <typename T, typename X, typename Acc, int N2>
-__device__ __forceinline__ Acc seg_fma_refill_n(const T* vp, const int32_t* cp2, int len, const X* x, X (&xv)[16]) {
-  Acc s = Acc(0);
-#pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    if (u < len) s = fma(Acc(vp[u]), Acc(xv[u]), s);
-    if (u < N2 && 16 + u < len) xv[u] = x[cp2[u]];
+// Entries of this lane's segment of step d (len: from load_seg_len).
+__device__ __forceinline__ int lane_segment(const int4& d, int len, int lane) {
+  if (step_mode(d) == kLongRow)
+    return d.z - ((d.y & kStepUniform) || lane < ((d.y >> kStepRemShift) & 0x3f) ? 0 : 1);
+  return len;
+}
+
+// The row of step d whose result this lane holds once its segment is summed
+// (and the lanes of a pair or of a long row are combined); -1 if none.
+__device__ __forceinline__ int result_row(const int4& d, int lane) {
+  const int mode = step_mode(d);
+  if (mode == kLanePerRow) return lane < step_lanes(d) ? d.x + lane : -1;
+  if (mode == kPairPerRow) return lane < step_lanes(d) && !(lane & 1) ? d.x + (lane >> 1) : -1;
+  return lane == 0 ? d.x : -1;
+}
+
+// Sum of a step's row from its lanes' segment sums.
+template <typename Acc>
+__device__ __forceinline__ Acc combine_lanes(int mode, Acc part) {
+  if (mode == kPairPerRow) return part + __shfl_xor_sync(0xffffffffu, part, 1);  // first half + second half
+  if (mode == kLongRow) {
+    if constexpr (sizeof(Acc) == 8) return warp_sum(part);
+    else return warp_sum_f(part);
   }
-  return s;
+  return part;
 }
 
-// Calls f(std::integral_constant<int, v>) for v in [LO, HI] (values below LO
-// call f with LO) through a binary tree of warp-uniform conditional branches:
-// no indirect jump (a jump table's target must be resolved before the warp
-// can go on).
+// Calls f(std::integral_constant<int, v>) for v in [LO, HI] through a binary
+// tree of warp-uniform conditional branches: no indirect jump (a jump table's
+// target must be resolved before the warp can go on).
 template <int LO, int HI, typename F>
 __device__ __forceinline__ void dispatch_tree(int v, F&& f) {
   if constexpr (LO == HI) {
@@ -550,227 +747,354 @@ __device__ __forceinline__ void dispatch_tree(int v, F&& f) {
   }
 }
 
-template <typename T, typename X, typename Acc>
-__device__ __forceinline__ Acc seg_fma_refill(const T* vp, const int32_t* cp2, int len, int n2, const X* x,
-                                              X (&xv)[16]) {
-  Acc s = Acc(0);
-  dispatch_tree<1, 16>(n2, [&](auto N) { s = seg_fma_refill_n<T, X, Acc, decltype(N)::value>(vp, cp2, len, x, xv); });
-  return s;
-}
-
-template <typename X, int U>
-__device__ __forceinline__ void seg_gather(const int32_t* cp, int len, int wmax, const X* x, X (&xv)[U]) {
-  static_assert(U == 32 || U == 16, "dispatch covers 1..U");
-  dispatch_tree<1, U>(wmax, [&](auto N) { seg_gather_n<X, decltype(N)::value, U>(cp, len, x, xv); });
-}
-
-template <typename T, typename X, typename Acc, int U>
-__device__ __forceinline__ Acc seg_fma(const T* vp, int len, int wmax, const X (&xv)[U], Acc s) {
-  static_assert(U == 32 || U == 16, "dispatch covers 1..U");
-  dispatch_tree<1, U>(wmax, [&](auto N) { s = seg_fma_n<T, X, Acc, decltype(N)::value, U>(vp, len, xv, s); });
-  return s;
-}
-
-// A segment longer than the unrolled capacity (up to kMirror entries: rows of
-// 17..64 entries split over two lanes), contiguous in the ring: gathers and
-// multiply-adds 8 at a time.
-template <typename T, typename X, typename Acc>
-__device__ __forceinline__ Acc seg_dot_loop(const T* vp, const int32_t* cp, int len, const X* x) {
-  Acc s = Acc(0);
-  int t = 0;
-  for (; t + 8 <= len; t += 8) {
-    X xv[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) xv[u] = x[cp[t + u]];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) s = fma(Acc(vp[t + u]), Acc(xv[u]), s);
-  }
-  for (; t < len; ++t) s = fma(Acc(vp[t]), Acc(x[cp[t]]), s);
-  return s;
-}
-
-// Lane-private part of a lane-per-row or pair-per-row step.  The row
-// pointers are loaded when a step is two steps ahead and only consumed one
-// step later, so their latency stays off the critical path.  *stream != 0:
-// load them with the evict-first policy (__ldcs), so that in a solve whose
-// vectors and row pointers together outgrow the L2 the row pointers, read
-// once per product, give way to the vectors that the step reads again.  The
-// flag is read where it is used (a kernel parameter or an L1 hit) rather
-// than held in a register through the product.
-struct LaneRaw {
-  int row;   // row whose (partial) sum this lane computes, -1 if none
-  int ks;    // row_ptr[row]
-  int ke;    // row_ptr[row + 1]
-};
-
-__device__ __forceinline__ LaneRaw lane_raw(const int32_t* row_ptr, int4 d, int mode, bool valid,
-                                            const int32_t* stream) {
+// Loads what ring_pass keeps of the warp's first steps (each computing warp of
+// the CTA calls, with its steps [s, s1)).
+template <typename Ring>
+__device__ __forceinline__ void load_first_steps(const Ring& sm, const PassIo& v, int s, int s1) {
   const int lane = threadIdx.x & 31;
-  LaneRaw r{-1, 0, 0};
-  if (valid && mode != kLongRow) {
-    const int i = d.x + (mode == kLanePerRow ? lane : (lane >> 1));
-    if (i < d.y) {
-      r.row = i;
-      if (*stream) {
-        r.ks = __ldcs(row_ptr + i);
-        r.ke = __ldcs(row_ptr + i + 1);
-      } else {
-        r.ks = row_ptr[i];
-        r.ke = row_ptr[i + 1];
-      }
+  WarpStream* const ws = sm.stream(threadIdx.x >> 5);
+  if (s < s1) {
+    for (int j = 0; j < 2; ++j) ws->seg_len[j][lane] = v.seg_len[static_cast<size_t>(min(s + j, s1 - 1)) * 32 + lane];
+    if (lane < 2) ws->step[lane] = v.step[s + lane < s1 ? s + lane : v.nsteps];
+  }
+  __syncwarp();
+}
+
+// The product over the warp's steps [s, s1) from its ring, gathering x (after
+// load_first_steps):
+// out[i] = (A x)_i; returns the sum over this lane's rows of aux[i] (A x)_i
+// (0 if aux is nullptr).  Every segment is one FMA chain in storage order.
+//
+// What bounds it is the FP64 pipe (an FMA occupies a sub-partition for 64
+// cycles, whatever its active lanes, and a predicated-off one as well; its
+// dependent latency is 115) beside the matrix stream.  So the loop keeps two
+// things in flight ahead of the chains: the ring's copies (all slots but the
+// two of the chunk being summed and of the next one; the producer warp starts
+// them), and the gathers of the warp's next chunk, of the same step or of the next one, each issued into the
+// register that the current chunk's FMA has just freed.  A warp-uniform branch,
+// not a predicate, ends a chunk's FMAs.  The stream's `failed` is raised if a wait gave up.
+template <typename Ring, typename X>
+__device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, const X* x, bool with_dot) {
+  using T = typename Ring::Val;
+  using C = typename Ring::Col;
+  constexpr int kU = max_chunk<T>();
+  const Ring sm{smem};
+  const PassIo& io = sm.state()->io;
+  const int tid = fresh_tid(), w = tid >> 5, lane = tid & 31;
+  const unsigned int below = (1u << lane) - 1u;
+  if (s >= s1) return 0.0;
+  double dot = 0.0;
+  WarpStream* const ws = sm.stream(w);
+  uint32_t consumed = ws->consumed, phases = ws->phases;
+  int tail = ws->tail;
+  auto leave = [&](bool ok) -> double {
+    if (lane == 0) {
+      ws->phases = phases;
+      ws->tail = tail;
+      if (!ok) ws->failed = 1;
     }
-  }
-  return r;
-}
-
-// This lane's entries [a, a + len) of its row (half of it in a pair step).
-__device__ __forceinline__ void lane_span(const LaneRaw& r, int mode, int& a, int& len) {
-  if (r.row < 0) {
-    a = 0;
-    len = 0;
-  } else if (mode == kLanePerRow) {
-    a = r.ks;
-    len = r.ke - r.ks;
-  } else {
-    const int half = (r.ke - r.ks + 1) >> 1;
-    const bool second = threadIdx.x & 1;
-    a = second ? r.ks + half : r.ks;
-    len = second ? (r.ke - r.ks - half) : half;
-  }
-}
-
-// The product over the CTA's steps with values `val` (type T), gathering x;
-// consumer warp w computes steps s0 + w, s0 + w + kConsumerWarps, ...  Each
-// row's result goes to epi(i, yi, aux[i]) from one lane (aux[i] = 0 when aux
-// is nullptr).  kRingPass: entries come from the ring (the producer streams
-// them; the warp waits on the full barrier of the pieces a step spans and
-// releases pieces on the empty barriers once its next step starts beyond
-// them); otherwise entries are read directly from global memory (values
-// `val`, column indices A.col_idx).  Step descriptors are loaded two steps
-// ahead, row pointers and aux values one step ahead; *stream_rows != 0: row
-// pointers with the evict-first policy (lane_raw).  Returns false
-// (uniformly over the warp) if a wait gave up.
-template <bool kRingPass, typename T, typename X, typename Acc, typename Epi>
-__device__ __forceinline__ bool spmv_pass(const RingSmem& sm, const CtaStream& cs, ConsumerCursor& cur,
-                                          const DevCsr& A, const T* val, const X* x, const double* aux, Epi& epi,
-                                          unsigned long long limit_ns, const int32_t* stream_rows) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const T* rv = kRingPass ? sm.val<T>() : val;
-  const int32_t* rc = kRingPass ? sm.col() : A.col_idx;
-  const int32_t* row_ptr = A.row_ptr;
-  const uint32_t gbase = cur.gbase;
-  // entry k sits at rv[pos(k)]: in the ring at (k + off) & kRingMask
-  const int off = static_cast<int>((gbase % kSlots) * kPiece) - cs.kb;
-  auto pos = [&](int k) { return kRingPass ? ((k + off) & kRingMask) : k; };
-  auto wait_piece = [&](int j) {
-    const uint32_t g = gbase + static_cast<uint32_t>(j);
-    return __all_sync(0xffffffffu, mbar_wait_bounded(sm.full(g % kSlots), (g / kSlots) & 1u, limit_ns, nullptr));
+    __syncwarp();
+    return dot;
   };
-  int released = 0;  // pieces of this pass this warp has released
-  auto release_upto = [&](int upto) -> bool {
-    for (; released < upto; ++released) {
-      if (!wait_piece(released)) return false;  // the piece must be the slot's current one
-      __syncwarp();
-      if (lane == 0) mbar_arrive(sm.empty((gbase + static_cast<uint32_t>(released)) % kSlots));
-    }
+  auto wait_next = [&]() -> bool {
+    uint64_t* const bar = sm.full(w, tail);
+    const uint32_t parity = (phases >> tail) & 1u;
+    if (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity)) &&
+        !__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, io.limit_ns, nullptr)))
+      return false;
+    phases ^= 1u << tail;
+    tail = tail + 1 == Ring::kSlots ? 0 : tail + 1;
     return true;
   };
-  auto sd = [&](int k) { return k < A.nsteps + 2 ? k : A.nsteps + 1; };  // two sentinels follow the last step
-  auto holds_result = [&](int mode, const LaneRaw& r) {
-    return r.row >= 0 && (mode == kLanePerRow || (lane & 1) == 0);
+  // a chunk: entries [u, u + cnt) of every lane's segment of one step
+  struct Chunk {
+    int cnt;      // entries per lane (warp-uniform; 0: the step has none; -1: no chunk)
+    int len;      // of them, those this lane's segment has
+    bool full;    // cnt entries are stored for every lane, else only what the segments have
+    bool ends;    // the last one of its step
+    int slot;
+    int val_off;  // its values' place in the slot
+    int row;      // the step's first row and kind word
+    int kind;
+    double aux;   // of the row whose sum this lane gets (if it ends the step)
   };
-  constexpr int kStride = kConsumerWarps;
-  int s = cs.s0 + w;
-  int4 d0 = A.step[sd(s)], d1 = A.step[sd(s + kStride)];
-  int m0 = A.step_mode[sd(s)], m1 = A.step_mode[sd(s + kStride)];
-  LaneRaw r0 = lane_raw(row_ptr, d0, m0 & 3, s < cs.s1, stream_rows);
-  double a0 = (aux != nullptr && s < cs.s1 && holds_result(m0 & 3, r0)) ? aux[r0.row] : 0.0;
-  for (; s < cs.s1; s += kStride) {
-    const bool has1 = s + kStride < cs.s1;
-    // prefetch: descriptor two steps ahead, row pointers and aux value of the next step
-    const int4 d2 = A.step[sd(s + 2 * kStride)];
-    const int m2 = A.step_mode[sd(s + 2 * kStride)];
-    const LaneRaw r1 = lane_raw(row_ptr, d1, m1 & 3, has1, stream_rows);
-    const double a1 = (aux != nullptr && has1 && holds_result(m1 & 3, r1)) ? aux[r1.row] : 0.0;
-    const int mode = m0 & 3;
-    if (kRingPass && d0.w > d0.z) {
-      // release what lies before this step; a short step then waits for the
-      // (at most two) pieces it spans
-      if (!release_upto((d0.z - cs.kb) >> kPieceLog)) return false;
-      if (mode != kLongRow) {
-        const int jh = (d0.w - 1 - cs.kb) >> kPieceLog;
-        for (int j = (d0.z - cs.kb) >> kPieceLog; j <= jh; ++j)
-          if (!wait_piece(j)) return false;
-      }
+  // steps and their segment lengths are loaded one ahead
+  auto step_at = [&](int k) { return k < s1 ? k : io.nsteps; };  // (the sentinel has no entries)
+  int4 d = ws->step[0], dn = ws->step[1];
+  int seg = ws->seg_len[0][lane], seg_n = ws->seg_len[1][lane];
+  seg = lane_segment(d, seg, lane);
+  int u = 0;
+  // the stream's next chunk
+  auto next_chunk = [&]() -> Chunk {
+    Chunk c;
+    if (s >= s1) {
+      c.cnt = -1;
+      c.len = 0;
+      c.full = true;
+      c.ends = false;
+      c.slot = c.val_off = c.row = c.kind = 0;
+      c.aux = 0.0;
+      return c;
     }
-    if (mode == kLongRow) {
-      // lanes stride the row; in a ring pass piece by piece, each piece
-      // released once done (the warp's next step starts after this row)
-      Acc acc = Acc(0);
-      if (kRingPass) {
-        const int jl = (d0.z - cs.kb) >> kPieceLog, jh = (d0.w - 1 - cs.kb) >> kPieceLog;
-        for (int j = jl; j <= jh; ++j) {
-          if (!wait_piece(j)) return false;
-          const int lo = max(d0.z, cs.kb + j * kPiece), hi = min(d0.w, cs.kb + (j + 1) * kPiece);
-          for (int k = lo + lane; k < hi; k += 32) {
-            const int p = pos(k);
-            acc = fma(Acc(rv[p]), Acc(x[rc[p]]), acc);
-          }
-          if (j < jh && !release_upto(j + 1)) return false;
-        }
-      } else {
-        for (int k = d0.z + lane; k < d0.w; k += 32) acc = fma(Acc(rv[k]), Acc(x[rc[k]]), acc);
-      }
-      Acc tot;
-      if constexpr (sizeof(Acc) == 8) tot = warp_sum(acc);
-      else tot = warp_sum_f(acc);
-      if (lane == 0) epi(d0.x, tot, aux != nullptr ? aux[d0.x] : 0.0);
+    c.cnt = min(step_chunk(d), d.z - u);
+    c.len = max(0, min(seg - u, c.cnt));
+    c.full = step_padded<C>(d) || __all_sync(0xffffffffu, u + c.cnt <= seg);
+    c.slot = tail;
+    if (c.full) {
+      c.val_off = c.cnt * 32 * static_cast<int>(sizeof(C));
     } else {
-      int a, len;
-      lane_span(r0, mode, a, len);
-      const int p0 = pos(a);
-      Acc part;
-      if constexpr (kRingPass) {
-        const int wmax = (m0 >> kWmaxShift) & 0xff;
-        if constexpr (sizeof(X) == 8) {
-          // FP64 gathers in batches of 16 (the same FMAs in the same order;
-          // half the registers held by gathered values); the second batch is
-          // loaded during the first batch's FMAs
-          X xv[16];
-          const int w0 = wmax < 16 ? wmax : 16;
-          seg_gather<X, 16>(rc + p0, len, w0, x, xv);
-          if (wmax > 16) {
-            part = seg_fma_refill<T, X, Acc>(rv + p0, rc + p0 + 16, len, wmax - 16, x, xv);
-            part = seg_fma<T, X, Acc, 16>(rv + p0 + 16, len - 16, wmax - 16, xv, part);
-          } else {
-            part = seg_fma<T, X, Acc, 16>(rv + p0, len, w0, xv, Acc(0));
-          }
-        } else {
-          X xv[kLaneMax];
-          seg_gather<X, kLaneMax>(rc + p0, len, wmax, x, xv);
-          part = seg_fma<T, X, Acc, kLaneMax>(rv + p0, len, wmax, xv, Acc(0));
+      const int tot = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(c.len)));
+      c.val_off = (tot * static_cast<int>(sizeof(C)) + kUnit - 1) & ~(kUnit - 1);
+    }
+    u += c.cnt;
+    c.row = d.x;
+    c.kind = d.y;
+    c.ends = u >= d.z;
+    c.aux = 0.0;
+    return c;
+  };
+  auto next_step = [&] {
+    ++s;
+    u = 0;
+    d = dn;
+    seg = lane_segment(d, seg_n, lane);
+    dn = load_step(io, step_at(s + 1));
+    seg_n = load_seg_len(io, min(s + 1, s1 - 1), lane);
+  };
+  auto cols = [&](const Chunk& c) { return reinterpret_cast<const C*>(sm.slot(w, c.slot)); };
+  auto vals = [&](const Chunk& c) { return reinterpret_cast<const T*>(sm.slot(w, c.slot) + c.val_off); };
+  // x of the columns of the step of the chunk being gathered: 16-bit columns are
+  // offsets from the step's smallest one
+  auto x_of = [&]() -> const X* { return sizeof(C) == 2 ? x + d.w : x; };
+  T acc = T(0);
+  if constexpr (sizeof(T) == 4) {
+    // FP32: an FMA takes no time beside its operands, so nothing hides a chunk's
+    // gathers but other gathers: those of two chunks (a 27-entry row) together,
+    // and the other warps'.  What bounds it then are the instructions issued: no
+    // bookkeeping from chunk to chunk.
+    auto gather = [&](const Chunk& c, X* xv) {
+      const X* const xb = x_of();
+      const C* cp = cols(c);
+      if (c.full) {
+        cp += lane;
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          if (k % 3 == 0 && k >= c.cnt) break;
+          if (k < c.len) xv[k] = xb[cp[32 * k]];
         }
       } else {
-        // the direct pass (rare: residual replacements) uses the compact
-        // loop: the same FMAs in the same order, far fewer registers
-        part = seg_dot_loop<T, X, Acc>(rv + p0, rc + p0, len, x);
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          if (k >= c.cnt) break;
+          const unsigned int m = __ballot_sync(0xffffffffu, k < c.len);
+          if (k < c.len) xv[k] = xb[cp[__popc(m & below)]];
+          cp += __popc(m);
+        }
       }
-      if (mode == kPairPerRow) {
-        // first half + second half: the same value in both lanes (commutative add)
-        const Acc sum = part + __shfl_xor_sync(0xffffffffu, part, 1);
-        if (holds_result(mode, r0)) epi(r0.row, sum, a0);
-      } else if (holds_result(mode, r0)) {
-        epi(r0.row, part, a0);
+    };
+    auto sum = [&](const Chunk& c, const X* xv) {
+      const T* vp = vals(c);
+      if (c.full) {
+        vp += lane;
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          if (k % 3 == 0 && k >= c.cnt) break;
+          if (k < c.len) acc = fma(vp[32 * k], xv[k], acc);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          if (k >= c.cnt) break;
+          const unsigned int m = __ballot_sync(0xffffffffu, k < c.len);
+          if (k < c.len) acc = fma(vp[__popc(m & below)], xv[k], acc);
+          vp += __popc(m);
+        }
+      }
+      __syncwarp();  // every lane has read the chunk: its slot is free
+      ++consumed;
+      if (lane == 0) st_release_shared(&ws->consumed, consumed);
+    };
+    while (s < s1) {
+      const int4 dc = d;
+      const int i = result_row(d, lane);
+      const double ai = with_dot && i >= 0 ? io.aux[i] : 0.0;
+      acc = T(0);
+      while (u < d.z) {
+        // (zero: a register that is only written under a predicate is live from
+        // the kernel's start on, and these would all be spilled)
+        X xa[kU], xb[kU];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) xa[k] = xb[k] = X(0);
+        Chunk a = next_chunk(), b;
+        if (!wait_next()) return leave(false);
+        gather(a, xa);
+        const bool two = u < d.z;
+        if (two) {
+          b = next_chunk();
+          if (!wait_next()) return leave(false);
+          gather(b, xb);
+        }
+        sum(a, xa);
+        if (two) sum(b, xb);
+      }
+      next_step();
+      const T tot = combine_lanes(step_mode(dc), acc);
+      if (i >= 0) {
+        const double y = static_cast<double>(tot);
+        io.out[i] = y;
+        dot = fma(ai, y, dot);
       }
     }
-    d0 = d1; m0 = m1; r0 = r1; a0 = a1;
-    d1 = d2; m1 = m2;
+    return leave(true);
   }
-  if (kRingPass) {
-    if (!release_upto(cs.npieces)) return false;
-    cur.gbase = gbase + static_cast<uint32_t>(cs.npieces);
+  // FP64: behind next_chunk, once its gathers are under way: the next step
+  auto after_gather = [&](Chunk& c) {
+    if (!c.ends) return;
+    const int i = with_dot ? result_row(d, lane) : -1;
+    if (i >= 0) c.aux = io.aux[i];
+    next_step();
+  };
+  // the first chunk: gathered, nothing to sum yet
+  X xv[kU];
+#pragma unroll
+  for (int k = 0; k < kU; ++k) xv[k] = X(0);
+  Chunk c = next_chunk();
+  if (c.cnt > 0) {
+    if (!wait_next()) return leave(false);
+    const X* const xb = x_of();
+    const C* cp = cols(c);
+    const int stored = c.full ? c.cnt : c.len;
+#pragma unroll
+    for (int k = 0; k < kU; ++k) {
+      const unsigned int m = __ballot_sync(0xffffffffu, k < stored);
+      if (k < stored) xv[k] = xb[cp[__popc(m & below)]];
+      cp += __popc(m);
+    }
   }
-  return true;
+  after_gather(c);
+  // sums chunk c, whose x values are in xv, and gathers those of chunk n
+  for (;;) {
+    Chunk n = next_chunk();
+    if (n.cnt > 0 && !wait_next()) return leave(false);
+    const X* const xb = x_of();
+    if (c.full && n.full) {
+      const T* const vp = vals(c) + lane;
+      const C* const cp = cols(n) + lane;
+      // straight-line code for each size of c
+      dispatch_tree<0, kU>(c.cnt, [&](auto N) {
+#pragma unroll
+        for (int k = 0; k < decltype(N)::value; ++k) {
+          if (k < c.len) acc = fma(vp[32 * k], xv[k], acc);
+          if (k < n.cnt) xv[k] = xb[cp[32 * k]];
+        }
+      });
+      if (n.cnt > c.cnt) {
+#pragma unroll
+        for (int k = 0; k < kU; ++k)
+          if (k >= c.cnt && k < n.cnt) xv[k] = xb[cp[32 * k]];
+      }
+    } else {
+      // only the segments' entries are stored: counted as they come
+      const T* vp = vals(c);
+      const C* cp = cols(n);
+      const int cs = c.full ? c.cnt : c.len, ns = n.full ? n.cnt : n.len;
+#pragma unroll
+      for (int k = 0; k < kU; ++k) {
+        if (k >= c.cnt) break;
+        const unsigned int mv = __ballot_sync(0xffffffffu, k < cs);
+        if (k < c.len) acc = fma(vp[__popc(mv & below)], xv[k], acc);
+        vp += __popc(mv);
+        const unsigned int mc = __ballot_sync(0xffffffffu, k < ns);
+        if (k < ns) xv[k] = xb[cp[__popc(mc & below)]];
+        cp += __popc(mc);
+      }
+      if (n.cnt > c.cnt) {
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          const bool on = k >= c.cnt && k < ns;
+          const unsigned int mc = __ballot_sync(0xffffffffu, on);
+          if (on) xv[k] = xb[cp[__popc(mc & below)]];
+          cp += __popc(mc);
+        }
+      }
+    }
+    after_gather(n);
+    if (c.cnt > 0) {
+      __syncwarp();  // every lane has read the chunk: its slot is free
+      ++consumed;
+      if (lane == 0) st_release_shared(&ws->consumed, consumed);
+    }
+    if (c.ends) {
+      const int4 dc = make_int4(c.row, c.kind, 0, 0);
+      const T tot = combine_lanes(step_mode(dc), acc);
+      const int i = result_row(dc, lane);
+      if (i >= 0) {
+        const double y = static_cast<double>(tot);
+        io.out[i] = y;
+        if (with_dot) dot = fma(c.aux, y, dot);
+      }
+      if (n.cnt < 0) return leave(true);
+      acc = T(0);
+    }
+    c = n;
+  }
+}
+
+// out = A x in FP64 over the warp's steps [s, s1), read directly from global memory in
+// stream order: the passes outside a solve's step loop (its setup, the final
+// true residual, the mixed solve's residual replacements) take it, which leaves
+// the ring's contents alone.
+template <typename Ring>
+__device__ __forceinline__ void direct_pass(const DevCsr& A, int chunk, int64_t entry, int s,
+                                         int s1, const double* x, double* out) {
+  using T = typename Ring::Val;
+  using C = typename Ring::Col;
+  constexpr int kU = 9;  // entries per lane in flight
+  const int lane = fresh_tid() & 31;
+  const unsigned int below = (1u << lane) - 1u;
+  for (; s < s1; ++s) {
+    const int4 d = A.step[s];
+    const int seg = lane_segment(d, A.seg_len[static_cast<size_t>(s) * 32 + lane], lane);
+    const double* const xb = sizeof(C) == 2 ? x + d.w : x;
+    const bool padded = step_padded<C>(d);
+    const int size = step_chunk(d);
+    double acc = 0.0;
+    for (int u = 0; u < d.z; u += size, ++chunk) {
+      const int cnt = min(size, d.z - u), len = max(0, min(seg - u, cnt));
+      const int stored = padded ? cnt : len;
+      const int tot = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(stored)));
+      const unsigned char* const at = A.stream + static_cast<size_t>(A.chunk_off[chunk]) * kUnit;
+      const C* cp = reinterpret_cast<const C*>(at);
+      const double* vp;
+      if constexpr (sizeof(T) == 4) vp = A.val64 + entry;
+      else vp = reinterpret_cast<const double*>(at + ((tot * static_cast<int>(sizeof(C)) + kUnit - 1) & ~(kUnit - 1)));
+      for (int k0 = 0; k0 < cnt; k0 += kU) {
+        double a[kU], g[kU];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) a[k] = g[k] = 0.0;  // (not live before: no spills)
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          const unsigned int m = __ballot_sync(0xffffffffu, k0 + k < stored);
+          if (k0 + k < len) {
+            const int e = __popc(m & below);
+            a[k] = __ldcs(vp + e);
+            g[k] = xb[__ldcs(cp + e)];
+          }
+          vp += __popc(m);
+          cp += __popc(m);
+        }
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          if (k0 + k >= cnt) break;
+          if (k0 + k < len) acc = fma(a[k], g[k], acc);
+        }
+      }
+      entry += tot;
+    }
+    const double tot = combine_lanes(step_mode(d), acc);
+    const int i = result_row(d, lane);
+    if (i >= 0) out[i] = tot;
+  }
 }
 
 }  // namespace cgk

@@ -6,69 +6,100 @@
 
 namespace cgk {
 
-// The persistent kernels run one CTA per SM: kConsumerWarps consumer warps
-// that compute, plus one producer warp that streams the CSR matrix into a
-// shared-memory ring with 1-D TMA bulk copies (warp specialisation).
-constexpr int kConsumerWarps = 15;  // with the producer: four warps per SM sub-partition
-constexpr int kConsumers = kConsumerWarps * 32;  // 480 computing threads
-constexpr int kBlock = kConsumers + 32;          // + the producer warp
+// The persistent kernels run one CTA per SM: kWarps warps that compute, each
+// its own steps of the CTA's rows from its own ring in shared memory, and one
+// producer warp, whose lane w fills warp w's ring with 1-D TMA bulk copies.
+constexpr int kWarps = 19;               // computing warps: with the producer five per SM sub-partition
+constexpr int kBlock = kWarps * 32;      // their threads
+constexpr int kThreads = kBlock + 32;    // and the producer warp
 constexpr int kCtasPerSm = 1;
-constexpr int kWarps = kConsumerWarps;           // warps taking part in CTA reductions
 
-// Matrix stream of a CTA: its CSR values and column indices, one pass after
-// another, flow through a ring of kSlots pieces of kPiece entries.  Each slot
-// has a "full" mbarrier (TMA completion) and an "empty" mbarrier on which
-// every consumer warp arrives once it no longer needs the piece.
-constexpr int kPieceLog = 11;
-constexpr int kPiece = 1 << kPieceLog;  // 2048 entries: 16 KB of FP64 values + 8 KB of indices
-constexpr int kSlots = 8;
-constexpr int kRing = kPiece * kSlots;  // 16384 entries
-constexpr int kRingMask = kRing - 1;
-// Entries mirrored behind the end of the ring: the head of the piece in
-// slot 0 is copied there as well, so a row segment of up to kMirror entries
-// starting anywhere in the ring reads contiguously, without wrapping.
-constexpr int kMirror = 32;
-// A step is what a consumer warp computes at once: up to 32 rows of <= 32
-// entries (one lane per row), up to 16 rows of 33..64 entries (two lanes per
-// row), both at most kStepNnz entries (so they span at most two pieces), or
-// one longer row, whose entries the warp walks piece by piece (lanes stride
-// them), releasing each piece as soon as it is done with it, so a row may be
-// longer than the ring.  Steps of a CTA go to its consumer warps round-robin.
-constexpr int kStepNnz = 1024;
+// A step is what a warp computes at once: 32 lanes, each summing one segment
+// of at most kLaneMax entries (up to 32 rows of <= 32 entries, one lane per
+// row; up to 16 rows of 33..64 entries, two lanes per row), or one longer row,
+// whose entries the lanes stride (a segment per lane of any length).  Step k
+// of a CTA goes to computing warp k modulo their number.
+//
+// The handle stores the matrix as one stream per warp: the entries of the
+// warp's steps in the order in which the warp consumes them.  Within a step
+// that is entry u of every lane's segment, in lane order, then entry u + 1, and
+// so on: one shared-memory read per entry and warp, free of bank conflicts.
+// A warp works through a step in chunks of a few entries per lane;
+// a chunk is one slot of the warp's ring, so that the ring gives back its
+// oldest bytes after every few entries and not only after a whole step.
+// 9: a 27-entry row is three full chunks, an 18-entry one two.  (FP64: 14, i.e. two
+// chunks, was slower: 64^3 33.1 against 29.3 us per step; FP32: 14, 18 and 28, with
+// up to a third of the warps for their registers: 29.1, 30.2 and 31.3 against
+// 27.1 us.)
+template <typename T> __host__ __device__ constexpr int max_chunk() { return sizeof(T) == 8 ? 9 : 14; }
+// Slots of a warp's ring: the chunk being summed, the next one and copies in
+// flight, in some 130 KB of shared memory.  The rest of the SM's 256 KB serves
+// the gathers as L1.
+template <typename T, typename C> __host__ __device__ constexpr int ring_slots() {
+  return 3;
+}
 constexpr int kLaneMax = 32;  // longest row computed by a single lane
 // Largest CTA share (rows) of the small-share solve kernels, which keep the
 // share's r in shared memory (20 KB behind the ring layout; the FP64 layout
-// then takes 218 KB of the 227 KB a CTA may have).
+// with 32-bit columns then takes 216 KB of the 227 KB a CTA may have).
 constexpr int kLocalRows = 2560;
 
-// Padding (in entries) behind val/col allocations so that rounding a copy's
-// end up to 16 bytes never reads past the allocation.
-constexpr int kPadEntries = 8;
+// A chunk in memory, and in a slot: its columns, then its values, each padded
+// to a multiple of kUnit bytes (the granularity of a bulk copy: one copy per
+// chunk).  Full chunks (every lane has all of their entries) need no padding.
+constexpr int kUnit = 16;
+__host__ __device__ constexpr int64_t units(int64_t bytes) { return (bytes + kUnit - 1) / kUnit; }
+__host__ __device__ constexpr int64_t chunk_units(int64_t entries, int col_bytes, int val_bytes) {
+  return units(entries * col_bytes) + units(entries * val_bytes);
+}
 
 enum StepMode : int32_t {
   kLanePerRow = 0,   // lane l computes row r0 + l (rows of <= kLaneMax entries)
   kPairPerRow = 1,   // lanes 2t, 2t+1 split row r0 + t (rows of <= 2 kLaneMax entries)
-  kLongRow = 2,      // the whole row r0 (entries [e0, e1)); lanes stride it
+  kLongRow = 2,      // the whole row r0; lanes stride it
 };
-// Bits 8..15 of a step's mode word: the longest per-lane segment of the step
-// (precomputed so that the lanes need no warp reduction to bound their loops).
-constexpr int kWmaxShift = 8;
+// The fields of a step: {first row, kind word, longest segment, smallest column}.
+// Kind word: bits 0..7 the lanes that hold a segment (from lane 0), bits 8..9
+// the StepMode, bit 10 set if all of them have the longest segment's length,
+// bit 11 the padding rule below, bits 16..21 (kLongRow) the lanes of the last,
+// partial stride, bits 24..29 the chunk (entries per lane): the segment split
+// evenly over as few chunks as it takes.
+constexpr int kStepModeShift = 8;
+constexpr int kStepUniform = 1 << 10;
+constexpr int kStepPadded = 1 << 11;
+constexpr int kStepRemShift = 16;
+constexpr int kStepChunkShift = 24;
+// Columns are stored as 16-bit offsets from their step's smallest column when
+// every step of the matrix spans at most this much, and as 32-bit columns
+// otherwise.
+constexpr int64_t kColSpan16 = 65535;
+// With 16-bit columns, a step whose lanes differ in length, or that fills only
+// some lanes, is padded to the longest segment in all 32 lanes where that adds
+// at most an eighth (the 2 bytes per entry saved on columns pay for it): an
+// entry's place is then a constant offset.  Other steps hold their entries
+// only, placed by counting the lanes before them.  Padding is never multiplied.
+constexpr bool step_pads(int64_t longest, int64_t entries) { return 8 * 32 * longest <= 9 * entries; }
 
-// Device view of a CSR matrix with its step partition.
+// Device view of a CSR matrix in stream order.
 struct DevCsr {
-  const int32_t* row_ptr;     // [n+1], 0-based
-  const int32_t* col_idx;     // [nnz + kPadEntries]
-  const double* val;          // [nnz + kPadEntries]
-  const float* val32;         // [nnz + kPadEntries] FP32 copy (mixed precision) or nullptr
-  const int4* step;           // [nsteps + 2] {r0, r1, e0, e1} (two trailing sentinels)
-  const int32_t* step_mode;   // [nsteps + 2] StepMode | flags
-  const int32_t* block_step;  // [nblocks + 1] first step of each CTA
+  const unsigned char* stream;  // the chunks: columns (col16) and FP64 values, or FP32 ones (mixed precision)
+  const double* val64;        // mixed precision: FP64 values in stream order (entries, padding included)
+  const int4* step;           // [nsteps + 1] see above (one trailing sentinel)
+  const int32_t* step_cmax;   // [nsteps] largest column of each step (-1: no entries), or nullptr
+  const uint8_t* seg_len;     // [32 * nsteps] entries of each lane's segment (not of kLongRow steps)
+  const uint32_t* chunk_off;  // [chunks + 1] first unit of each chunk, stream by stream
+  const int4* warp_chunk;     // [nblocks * kWarps] each warp's stream: first chunk, number of chunks,
+                              // start and end of the first one (units)
+  const uint32_t* warp_entry; // mixed precision: [nblocks * kWarps] its first entry in val64
+  const int32_t* warp_step;   // [nblocks * kWarps + 1] first step of each warp (stream by stream)
   const int32_t* block_row;   // [nblocks + 1] first row of each CTA (vector phases)
   int32_t n;
   int32_t nsteps;
   int32_t nblocks;            // CTAs the partition was balanced for
   int32_t max_rows;           // most rows in one CTA's range (host side; 0 if unknown)
   int64_t nnz;
+  int32_t col16;              // 1: 16-bit column offsets
+  int32_t pad;
 };
 
 // Whether a solve of A in one launch (chunk_iters <= 0) runs the small-share
@@ -96,7 +127,15 @@ struct SolveCtrl {
   unsigned long long rounds;    // group-barrier rounds completed so far
   int32_t slot;                 // partial-sum slot the next group sum uses
   int32_t pad;
+  // The step sums' accumulators (group_sum_fast): two words for each of p.q, r.r
+  // and r.z, never cleared during a solve; their values and the exponents of the
+  // last sums at the end of a launch.
+  alignas(16) unsigned long long acc[3][2];
+  unsigned long long acc_seen[3][2];
+  int32_t acc_exp[3];
+  int32_t pad2;
 };
+static_assert(sizeof(SolveCtrl) % 16 == 0, "accumulators on 16 bytes in a table");
 
 struct SolveParams {
   DevCsr A;
@@ -113,7 +152,7 @@ struct SolveParams {
   int64_t replace_every;        // mixed precision: true-residual period
   unsigned long long wait_limit_ns;  // bound on every device-side wait
   int32_t group;                // CTAs that solve this system together (its partition's CTA count)
-  int32_t stream_rows;          // single-system kernels: row pointers evict-first (stream_row_ptrs)
+  int32_t stream_rows;          // single-system kernels: row tables evict-first (stream_row_tables)
   int64_t chunk_iters;          // steps per launch (<= 0: until the solve ends)
   const double* dinv;           // Jacobi preconditioner 1/diag(A), or nullptr (plain CG)
   // Single-system solves: one epoch flag per CTA (zeroed before the launch).
@@ -132,7 +171,7 @@ struct BatchTask {
 };
 struct BatchQueue {
   int32_t ntasks;
-  int32_t stream_rows;          // row pointers evict-first in this launch (stream_row_ptrs)
+  int32_t stream_rows;          // row tables evict-first in this launch (stream_row_tables)
   BatchTask task[1];            // ntasks entries (allocated to capacity)
 };
 struct BatchParams {
@@ -142,22 +181,19 @@ struct BatchParams {
 };
 
 // Bytes that a step of the CG iteration on n rows reads again in the next
-// step: p, q and r, the row pointers, the FP32 copy of p (mixed precision)
-// and 1/diag(A) (Jacobi).  x and the matrix stream through with the
-// evict-first policy.
+// step: p, q and r, up to 4 bytes per row of row and step tables, the FP32
+// copy of p (mixed precision) and 1/diag(A) (Jacobi).  x and the matrix stream
+// through with the evict-first policy.
 inline int64_t step_reused_bytes(int64_t n, bool mixed, bool jacobi) {
   return n * (28 + (mixed ? 4 : 0) + (jacobi ? 8 : 0));
 }
 
-// Whether the product loads the row pointers with the evict-first policy:
-// when the bytes that the running steps read again take more than 4/7 of
-// the L2.  Below that, row pointers and vectors both stay in the L2 from
-// step to step; above it the row pointers, read once per product, are the
-// better ones to give up.  On GB300 with the Q1 systems: 128^3 was 5.7 %
-// (mixed 3.5 %) and 136^3 0.5 % slower with them streamed; 136^3 mixed,
-// 144^3 and larger 0.3 to 1.8 % faster, and a batch of 256 systems of 8^3
-// to 48^3 4.5 % (mixed 8.9 %).
-inline bool stream_row_ptrs(int64_t reused_bytes, int64_t l2_bytes) {
+// Whether the product loads the row and step tables (read once per product)
+// with the evict-first policy: when the bytes that the running steps read
+// again take more than 4/7 of the L2.  Below that, tables and vectors both
+// stay in the L2 from step to step; above it the tables are the better ones
+// to give up.
+inline bool stream_row_tables(int64_t reused_bytes, int64_t l2_bytes) {
   return l2_bytes > 0 && 7 * reused_bytes > 4 * l2_bytes;
 }
 
@@ -168,10 +204,48 @@ enum : int32_t {
 };
 
 // Launchers (defined in the .cu files; return the CUDA error of the launch).
-// dinv[i] = 1 / (sum of row i's stored entries in column i); err set to the
-// first row (+1) whose diagonal is not positive.
-cudaError_t launch_jacobi_dinv(const int32_t* row_ptr, const int32_t* col_idx, const double* val, int64_t n,
-                               double* dinv, int32_t* err, cudaStream_t s);
+// ---- stream order (layout.cu)
+// Source of a matrix in CSR form on the device: row_ptr 0-based; col_idx and
+// val hold the entries from e_first on, columns based at `base`.
+struct CsrSource {
+  const int32_t* row_ptr;
+  const int32_t* col_idx;
+  const double* val;
+  int64_t e_first;
+  int32_t base;
+};
+// What layout_scan found, cleared before it: the widest step (largest minus
+// smallest column), and (if asked to check) the first entry whose column lies
+// outside [base, n + base).
+struct LayoutScan {
+  int32_t span;
+  int32_t pad;
+  unsigned long long bad_entry;  // ~entry (so that a maximum finds the first), 0: none
+};
+// For steps [s0, s1): the lanes' segment lengths into seg_len[], the smallest
+// column into step[].w (0 for a step without entries), the largest into cmax[]
+// (if not nullptr; -1 without entries), span and bad entries into *out.
+cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1, int64_t n,
+                               bool check, LayoutScan* out, cudaStream_t s);
+// Writes the entries of steps [s0, s1) in stream order: into `stream` the
+// chunks step_chunk[k].. of step k, at the units that chunk_off gives (16-bit
+// column offsets if col16, else 32-bit columns; FP32 values, rounded to nearest,
+// if mixed), and if mixed the FP64 values from val64[step_entry[k]] on.
+// Padding of entries: zeros.
+struct StreamPlace {
+  const uint32_t* chunk_off;
+  const uint32_t* step_chunk;
+  const uint32_t* step_entry;  // mixed
+  unsigned char* stream;
+  double* val64;               // mixed
+};
+cudaError_t launch_layout_fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
+                               bool col16, bool mixed, cudaStream_t s);
+// dinv[i] = 1 / (sum of row i's stored entries in column i) for rows [row0, row1);
+// err set to the first row (+1) found whose diagonal is not positive.
+cudaError_t launch_jacobi_dinv(const CsrSource& src, int64_t row0, int64_t row1, double* dinv, int32_t* err,
+                               cudaStream_t s);
+
 cudaError_t launch_spmv(const DevCsr& A, const double* x, double* y, int32_t* err, cudaStream_t s);
 cudaError_t launch_dot(int64_t n, const double* x, const double* y, double* out,
                        double* partials, unsigned int* counter, int grid, cudaStream_t s);
@@ -215,6 +289,8 @@ cudaError_t launch_cluster_solve(const int32_t* row_ptr, const int32_t* col_idx,
 constexpr int32_t kSelftestSite = 99;
 // timeout_site of a single-system solve's wait for its neighbours' p
 constexpr int32_t kNeighborSite = 98;
+// timeout_site of a wait for a sum through the accumulators
+constexpr int32_t kAccSite = 96;
 // timeout_site of the synchronisation probe's barrier
 constexpr int32_t kProbeSite = 97;
 // The solves' group-wide synchronisations timed alone (cg_probe_group_sync):
@@ -223,9 +299,10 @@ constexpr int32_t kProbeSite = 97;
 // partials 2 * nblocks doubles, out nblocks doubles.
 cudaError_t launch_sync_probe(SolveCtrl* ctrl, double* partials, int iters, int mode, int nblocks,
                               unsigned long long limit_ns, double* out, cudaStream_t s);
-// Shared-memory bytes of a persistent solve CTA (FP32 ring values if mixed;
+// Shared-memory bytes of a persistent solve CTA (FP32 ring values if mixed,
+// 16- or 32-bit columns;
 // `local`: the small-share kernels, with r of the share).
-size_t solve_smem_bytes(bool mixed, bool local = false);
+size_t solve_smem_bytes(bool mixed, bool col16, bool local = false);
 // Opt a kernel in to `bytes` of dynamic shared memory with the smallest
 // carveout that holds them (once per kernel and device).
 cudaError_t ensure_smem_attr(const void* kernel, size_t bytes);

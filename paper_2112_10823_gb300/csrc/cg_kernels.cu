@@ -26,47 +26,46 @@
 #include <mutex>
 #include <set>
 #include <utility>
-#include "cg_solve.cuh"
+#include "cg_device.cuh"
 
 namespace cgk {
 
-// One system on the whole grid: CTA c is rank c of the group.  kJacobi:
-// preconditioned by M = diag(A) (P.dinv).
-template <bool kMixed, bool kJacobi, bool kSmallShare>
-__global__ void __launch_bounds__(kBlock, kCtasPerSm) cg_solve_kernel(const __grid_constant__ SolveParams P) {
+// y = A x (same partition and stream as the solve; one pass, every table read
+// once: evict-first).
+template <typename C>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+    spmv_kernel(const __grid_constant__ DevCsr A, const double* x, double* y, int32_t* err) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const RingSmem sm{smem_raw, kMixed ? 4u : 8u};  // the step loop streams FP32 values in the mixed solve
-  CtaStream cs;
-  stream_setup(sm, cs, P.A, blockIdx.x);  // the last barrier of all threads
-  if (threadIdx.x >= kConsumers) {
-    solve_producer<kMixed>(sm, cs, P);
+  using Ring = RingSmem<double, C>;
+  const Ring sm{smem_raw};
+  ring_init(sm);
+  const unsigned long long lim = 2000000000ull;
+  if (threadIdx.x >= kBlock) {
+    if (!producer(sm, A, blockIdx.x, true, lim) && threadIdx.x == kBlock) atomicExch(err, kETIMEOUT);
     return;
   }
-  // the neighbour wait at the end of a step pays off on large shares (160^3:
-  // 1.6 % faster); on small ones the group barrier is faster (64^3: 1 %, 16^3: 9 %)
-  solve_consumers<kMixed, kJacobi, kSmallShare, !kSmallShare>(sm, cs, P, blockIdx.x, &P.stream_rows);
+  const int bw = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  const int s = A.warp_step[bw], s1 = A.warp_step[bw + 1];
+  const PassIo io = pass_io(A, 1, nullptr, y, lim);
+  load_first_steps(sm, io, s, s1);
+  if (threadIdx.x == 0) sm.state()->io = io;
+  cta_sync();
+  ring_pass<Ring>(smem_raw, s, s1, x, false);
+  if ((threadIdx.x & 31) == 0 && sm.stream(threadIdx.x >> 5)->failed) {
+    atomicExch(err, kETIMEOUT);
+    *reinterpret_cast<volatile int32_t*>(sm.stop()) = 1;
+  }
 }
 
-// The product alone reads every row pointer once: always evict-first.
-__constant__ int32_t kStreamRowsAlways = 1;
-
-// y = A x (same partition and stream as the solve; one pass).
-__global__ void __launch_bounds__(kBlock, kCtasPerSm) spmv_kernel(const DevCsr A, const double* __restrict__ x,
-                                                                   double* __restrict__ y, int32_t* err) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const RingSmem sm{smem_raw};
-  CtaStream cs;
-  stream_setup(sm, cs, A, blockIdx.x);
-  const unsigned long long lim = 2000000000ull;
-  if (threadIdx.x >= kConsumers) {
-    if (threadIdx.x == kConsumers && !producer_loop<double>(sm, cs, A.val, A.col_idx, 1, lim)) atomicExch(err, kETIMEOUT);
-    return;
-  }
-  ConsumerCursor cur;
-  auto epi = [&](int i, double s, double) { y[i] = s; };
-  const bool ok = cta_and(spmv_pass<true, double, double, double>(sm, cs, cur, A, A.val, x, nullptr, epi, lim, &kStreamRowsAlways));
-  if (!ok && threadIdx.x == 0) atomicExch(err, kETIMEOUT);
-  consumers_done(sm);
+// The same of a mixed-precision handle, whose streams hold FP32 values: its FP64
+// values directly from global memory, a warp per stream.
+template <typename C>
+__global__ void __launch_bounds__(kBlock, kCtasPerSm)
+    spmv_direct_kernel(const __grid_constant__ DevCsr A, const double* x, double* y) {
+  using Ring = RingSmem<float, C>;
+  const int bw = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  direct_pass<Ring>(A, A.warp_chunk[bw].x, A.warp_entry[bw], A.warp_step[bw], A.warp_step[bw + 1], x,
+                    y);
 }
 
 // Opt a kernel in to `bytes` of dynamic shared memory, and ask for the
@@ -95,40 +94,46 @@ cudaError_t ensure_smem_attr(const void* kernel, size_t bytes) {
 }
 
 cudaError_t launch_spmv(const DevCsr& A, const double* x, double* y, int32_t* err, cudaStream_t s) {
-  constexpr size_t kSmem = ring_smem_bytes<double>();
-  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(spmv_kernel), kSmem);
+  if (A.val64 != nullptr) {
+    if (A.col16) spmv_direct_kernel<uint16_t><<<A.nblocks, kBlock, 0, s>>>(A, x, y);
+    else spmv_direct_kernel<int32_t><<<A.nblocks, kBlock, 0, s>>>(A, x, y);
+    return cudaGetLastError();
+  }
+  const size_t smem = solve_smem_bytes(false, A.col16 != 0);
+  const void* k = A.col16 ? reinterpret_cast<const void*>(spmv_kernel<uint16_t>)
+                          : reinterpret_cast<const void*>(spmv_kernel<int32_t>);
+  cudaError_t e = ensure_smem_attr(k, smem);
   if (e != cudaSuccess) return e;
-  spmv_kernel<<<A.nblocks, kBlock, kSmem, s>>>(A, x, y, err);
+  if (A.col16) spmv_kernel<uint16_t><<<A.nblocks, kThreads, smem, s>>>(A, x, y, err);
+  else spmv_kernel<int32_t><<<A.nblocks, kThreads, smem, s>>>(A, x, y, err);
   return cudaGetLastError();
 }
 
-template <bool kSmallShare>
-const void* solve_kernel_ptr_t(bool mixed, bool jacobi) {
-  if (mixed) return jacobi ? reinterpret_cast<const void*>(cg_solve_kernel<true, true, kSmallShare>)
-                           : reinterpret_cast<const void*>(cg_solve_kernel<true, false, kSmallShare>);
-  return jacobi ? reinterpret_cast<const void*>(cg_solve_kernel<false, true, kSmallShare>)
-                : reinterpret_cast<const void*>(cg_solve_kernel<false, false, kSmallShare>);
+template <bool kMixed, typename C>
+const void* solve_kernel_of(bool jacobi, bool small);  // solve_*.cu
+
+const void* solve_kernel_ptr(bool mixed, bool jacobi, bool col16, bool small) {
+  if (mixed) return col16 ? solve_kernel_of<true, uint16_t>(jacobi, small) : solve_kernel_of<true, int32_t>(jacobi, small);
+  return col16 ? solve_kernel_of<false, uint16_t>(jacobi, small) : solve_kernel_of<false, int32_t>(jacobi, small);
 }
 
-const void* solve_kernel_ptr(bool mixed, bool jacobi, bool small_share = false) {
-  return small_share ? solve_kernel_ptr_t<true>(mixed, jacobi) : solve_kernel_ptr_t<false>(mixed, jacobi);
-}
-
-size_t solve_smem_bytes(bool mixed, bool local) {
-  return mixed ? ring_smem_bytes<float>(local) : ring_smem_bytes<double>(local);
+size_t solve_smem_bytes(bool mixed, bool col16, bool local) {
+  if (mixed) return col16 ? ring_smem_bytes<float, uint16_t>(local) : ring_smem_bytes<float, int32_t>(local);
+  return col16 ? ring_smem_bytes<double, uint16_t>(local) : ring_smem_bytes<double, int32_t>(local);
 }
 
 int solve_blocks_per_sm(bool mixed, bool jacobi) {
-  int nb = 0;
-  for (const bool small : {false, true}) {  // both must fit (one CTA per SM)
-    const void* k = solve_kernel_ptr(mixed, jacobi, small);
-    const size_t smem = solve_smem_bytes(mixed, small);
-    cudaError_t e = ensure_smem_attr(k, smem);
-    int nk = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nk, k, kBlock, smem);
-    if (e != cudaSuccess) return -1;
-    nb = small ? std::min(nb, nk) : nk;
-  }
+  int nb = 1 << 20;
+  for (const bool small : {false, true})  // every variant must fit (one CTA per SM)
+    for (const bool col16 : {false, true}) {
+      const void* k = solve_kernel_ptr(mixed, jacobi, col16, small);
+      const size_t smem = solve_smem_bytes(mixed, col16, small);
+      cudaError_t e = ensure_smem_attr(k, smem);
+      int nk = 0;
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nk, k, kThreads, smem);
+      if (e != cudaSuccess) return -1;
+      nb = std::min(nb, nk);
+    }
   return nb;
 }
 
@@ -136,24 +141,23 @@ cudaError_t launch_solve(const SolveParams& P, bool mixed, cudaStream_t s) {
   void* args[] = {const_cast<SolveParams*>(&P)};
   // the small-share kernel: every CTA's rows fit its shared r, and the
   // solve runs in this one launch
-  const bool small = small_share(P.A, P.chunk_iters);
-  const void* k = solve_kernel_ptr(mixed, P.dinv != nullptr, small);
-  const size_t smem = solve_smem_bytes(mixed, small);
+  const bool small = small_share(P.A, P.chunk_iters), col16 = P.A.col16 != 0;
+  const void* k = solve_kernel_ptr(mixed, P.dinv != nullptr, col16, small);
+  const size_t smem = solve_smem_bytes(mixed, col16, small);
   cudaError_t e = ensure_smem_attr(k, smem);
   if (e != cudaSuccess) return e;
-  return cudaLaunchCooperativeKernel(k, dim3(P.A.nblocks), dim3(kBlock), args, smem, s);
+  return cudaLaunchCooperativeKernel(k, dim3(P.A.nblocks), dim3(kThreads), args, smem, s);
 }
 
 // dinv[i] = 1 / diag(A)_i (the diagonal summed over row i's entries in
 // column i, in storage order); err <- first row (+1) without a positive one.
-__global__ void jacobi_dinv_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                                   const double* __restrict__ val, int64_t n, double* __restrict__ dinv,
+__global__ void jacobi_dinv_kernel(const CsrSource src, int64_t row0, int64_t row1, double* __restrict__ dinv,
                                    int32_t* err) {
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
+  for (int64_t i = row0 + blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < row1;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     double d = 0.0;
-    for (int k = row_ptr[i]; k < row_ptr[i + 1]; ++k)
-      if (col_idx[k] == i) d += val[k];
+    for (int64_t k = src.row_ptr[i] - src.e_first; k < src.row_ptr[i + 1] - src.e_first; ++k)
+      if (src.col_idx[k] - src.base == i) d += src.val[k];
     if (d > 0.0) {
       dinv[i] = 1.0 / d;
     } else {
@@ -163,12 +167,11 @@ __global__ void jacobi_dinv_kernel(const int32_t* __restrict__ row_ptr, const in
   }
 }
 
-cudaError_t launch_jacobi_dinv(const int32_t* row_ptr, const int32_t* col_idx, const double* val, int64_t n,
-                               double* dinv, int32_t* err, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int64_t blocks = (n + 255) / 256;
-  jacobi_dinv_kernel<<<static_cast<unsigned>(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(row_ptr, col_idx, val, n,
-                                                                                        dinv, err);
+cudaError_t launch_jacobi_dinv(const CsrSource& src, int64_t row0, int64_t row1, double* dinv, int32_t* err,
+                               cudaStream_t s) {
+  if (row1 <= row0) return cudaSuccess;
+  const int64_t blocks = (row1 - row0 + 255) / 256;
+  jacobi_dinv_kernel<<<static_cast<unsigned>(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(src, row0, row1, dinv, err);
   return cudaGetLastError();
 }
 

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cg_cluster_kernel(const __
 #pragma unroll
       for (int j = 0; j < 2; ++j)
         if (j < nv) {
-          const double c = fx_combine(valid ? part[j * 16 + lane] : FxPart{0, 0, 0}, valid);
+          const double c = fx_value(fx_combine(valid ? part[j * 16 + lane] : FxPart{0, 0, 0}, valid));
           if (lane < kClusterCtas)
             cluster_st(cluster_addr(sums + (set * 2 + j) * kClusterCtas + rank, static_cast<uint32_t>(lane)), c);
         }
@@ -163,8 +163,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) cg_cluster_kernel(const __
         if (j < nv) {
           const bool valid = lane < kClusterCtas;
           const FxPart f = fx_warp(valid ? sums[(set * 2 + j) * kClusterCtas + lane] : 0.0);
-          const double tot = f.nf ? __longlong_as_double(0x7ff8000000000000ll)
-                                  : (f.e == 0 ? 0.0 : ldexp(static_cast<double>(f.m), f.e - 1074));
+          const double tot = fx_value(f);
           if (lane == 0) scal[j] = tot;
         }
     }

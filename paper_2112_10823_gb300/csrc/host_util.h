@@ -4,17 +4,29 @@
 #include <cstdint>
 #include <vector>
 #include <vector_types.h>
+#include "cg_internal.h"
 
 namespace cgh {
 
 // Row partition of the persistent kernels for `nblocks` CTAs: CTA ranges of
-// about equal cost (block_row), each split into steps (block_step, step,
-// step_mode; see cg_internal.h), plus two sentinel steps.
+// about equal cost (block_row), each split into steps (see cg_internal.h),
+// which are listed warp by warp (warp_step).  One sentinel step follows the
+// last one.  The steps' smallest columns are left 0.
+// place_steps adds the streams: the chunks of every warp (warp_chunk,
+// chunk_off), each step's place in them and the stream's size.
 struct Partition {
   std::vector<int4> step;
-  std::vector<int32_t> step_mode;
-  std::vector<int32_t> block_step;
+  std::vector<int32_t> warp_step;
   std::vector<int32_t> block_row;
+  int64_t chunks = 0;        // of all streams
+  // by place_steps
+  std::vector<int4> warp_chunk;
+  std::vector<uint32_t> chunk_off;
+  std::vector<uint32_t> step_chunk;
+  std::vector<uint32_t> warp_entry;  // mixed precision
+  std::vector<uint32_t> step_entry;
+  int64_t stream_units = 0;
+  int64_t entries = 0;       // stored, padding included
 };
 
 // Which kind of step (cgk::StepMode: one lane per row, two lanes per row, or
@@ -30,7 +42,9 @@ struct StepShape {
   bool valid() const;
 };
 
-void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, Partition& P,
+void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, bool mixed, Partition& P,
                      const StepShape& shape = StepShape());
-
+void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool mixed, Partition& P);
+// Upper bounds of stream_units and entries for either column width.
+void stream_bound(int64_t nnz, bool mixed, const Partition& P, int64_t* stream_units, int64_t* entries);
 }  // namespace cgh

@@ -1,0 +1,146 @@
+// Stream order of a matrix (cg_internal.h): what a handle or an admitted
+// system keeps of its CSR arrays, built on the device, one warp per step.
+// Both kernels are bound by the CSR arrays' bytes: the scan reads the columns
+// once; the fill reads every entry once (lanes at the stride of a row, so that
+// a warp's reads of consecutive entries of 32 rows meet again in L1) and writes
+// it once, coalesced.
+#include "cg_device.cuh"
+
+namespace cgk {
+
+namespace {
+constexpr int kLayoutBlock = 256;
+
+unsigned layout_grid(int32_t s0, int32_t s1) {
+  return static_cast<unsigned>((static_cast<int64_t>(s1 - s0) * 32 + kLayoutBlock - 1) / kLayoutBlock);
+}
+
+__device__ __forceinline__ int step_rows(const int4& d) {
+  const int mode = step_mode(d);
+  return mode == kLanePerRow ? step_lanes(d) : mode == kPairPerRow ? step_lanes(d) >> 1 : 1;
+}
+}  // namespace
+
+__global__ void __launch_bounds__(kLayoutBlock) layout_scan_kernel(const CsrSource src, int4* step, uint8_t* seg_len, int32_t* cmax,
+                                                                    int32_t s0, int32_t s1, int64_t n, int check,
+                                                                    LayoutScan* out) {
+  const int s = s0 + static_cast<int>((static_cast<int64_t>(blockIdx.x) * kLayoutBlock + threadIdx.x) >> 5);
+  if (s >= s1) return;
+  const int lane = threadIdx.x & 31;
+  const int4 d = step[s];
+  const int64_t e0 = src.row_ptr[d.x], e1 = src.row_ptr[d.x + step_rows(d)];
+  int lo = 0x7fffffff, hi = -1;
+  unsigned long long bad = 0;
+  for (int64_t k = e0 + lane; k < e1; k += 32) {
+    // (unsigned: a column below the base wraps to a large value)
+    const unsigned int c = static_cast<unsigned int>(src.col_idx[k - src.e_first]) - static_cast<unsigned int>(src.base);
+    if (check && static_cast<int64_t>(c) >= n) {
+      const unsigned long long at = ~static_cast<unsigned long long>(k);
+      bad = at > bad ? at : bad;
+    } else {
+      lo = min(lo, static_cast<int>(c));
+      hi = max(hi, static_cast<int>(c));
+    }
+  }
+  if (step_mode(d) != kLongRow) {
+    int len = 0;
+    if (lane < step_lanes(d)) {
+      const int row = d.x + (step_mode(d) == kLanePerRow ? lane : lane >> 1);
+      len = src.row_ptr[row + 1] - src.row_ptr[row];
+      if (step_mode(d) == kPairPerRow) len = (lane & 1) ? len >> 1 : (len + 1) >> 1;
+    }
+    seg_len[static_cast<size_t>(s) * 32 + lane] = static_cast<uint8_t>(len);
+  }
+  if (bad) atomicMax(&out->bad_entry, bad);
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    step[s].w = hi < 0 ? 0 : lo;
+    if (cmax != nullptr) cmax[s] = hi;
+    if (hi > lo) atomicMax(&out->span, hi - lo);
+  }
+}
+
+template <typename T, typename C>
+__global__ void __launch_bounds__(kLayoutBlock)
+    layout_fill_kernel(const CsrSource src, const int4* __restrict__ step, const StreamPlace to, int32_t s0,
+                       int32_t s1) {
+  const int s = s0 + static_cast<int>((static_cast<int64_t>(blockIdx.x) * kLayoutBlock + threadIdx.x) >> 5);
+  if (s >= s1) return;
+  const int lane = threadIdx.x & 31;
+  const unsigned int below = (1u << lane) - 1u;
+  const int4 d = step[s];
+  const int mode = step_mode(d);
+  // this lane's segment in CSR order: entries a, a + stride, ...
+  int64_t a = 0;
+  int len = 0;
+  const int stride = mode == kLongRow ? 32 : 1;
+  if (mode == kLongRow) {
+    a = src.row_ptr[d.x] + static_cast<int64_t>(lane);
+    const int64_t left = src.row_ptr[d.x + 1] - a;
+    len = left > 0 ? static_cast<int>((left + 31) >> 5) : 0;
+  } else if (lane < step_lanes(d)) {
+    const int row = d.x + (mode == kLanePerRow ? lane : lane >> 1);
+    a = src.row_ptr[row];
+    len = static_cast<int>(src.row_ptr[row + 1] - a);
+    if (mode == kPairPerRow) {
+      const int half = (len + 1) >> 1;
+      if (lane & 1) {
+        a += half;
+        len -= half;
+      } else {
+        len = half;
+      }
+    }
+  }
+  a -= src.e_first;
+  const int base = src.base + (sizeof(C) == 2 ? d.w : 0);
+  const bool padded = step_padded<C>(d);
+  const int size = step_chunk(d);
+  uint32_t chunk = to.step_chunk[s];
+  int64_t entry = sizeof(T) == 4 ? to.step_entry[s] : 0;
+  for (int u0 = 0; u0 < d.z; u0 += size, ++chunk) {
+    const int cnt = min(size, d.z - u0);
+    const int mine = padded ? cnt : max(0, min(len - u0, cnt));
+    const int tot = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(mine)));
+    unsigned char* const at = to.stream + static_cast<size_t>(to.chunk_off[chunk]) * kUnit;
+    C* const col = reinterpret_cast<C*>(at);
+    T* const val = reinterpret_cast<T*>(at + units(static_cast<int64_t>(tot) * sizeof(C)) * kUnit);
+    int pos = 0;
+    for (int k = 0; k < cnt; ++k, a += stride) {
+      const unsigned int m = __ballot_sync(0xffffffffu, k < mine);
+      if (k < mine) {
+        const bool real = u0 + k < len;
+        const int dst = pos + __popc(m & below);
+        const double v = real ? src.val[a] : 0.0;
+        col[dst] = real ? static_cast<C>(src.col_idx[a] - base) : C(0);
+        val[dst] = static_cast<T>(v);  // (round to nearest)
+        if (sizeof(T) == 4) to.val64[entry + dst] = v;
+      }
+      pos += __popc(m);
+    }
+    entry += tot;
+  }
+}
+
+cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1, int64_t n,
+                               bool check, LayoutScan* out, cudaStream_t s) {
+  if (s1 <= s0) return cudaSuccess;
+  layout_scan_kernel<<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, seg_len, cmax, s0, s1, n, check ? 1 : 0, out);
+  return cudaGetLastError();
+}
+
+template <typename T, typename C>
+static void fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1, cudaStream_t s) {
+  layout_fill_kernel<T, C><<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, to, s0, s1);
+}
+
+cudaError_t launch_layout_fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
+                               bool col16, bool mixed, cudaStream_t s) {
+  if (s1 <= s0) return cudaSuccess;
+  if (mixed) col16 ? fill<float, uint16_t>(src, step, to, s0, s1, s) : fill<float, int32_t>(src, step, to, s0, s1, s);
+  else col16 ? fill<double, uint16_t>(src, step, to, s0, s1, s) : fill<double, int32_t>(src, step, to, s0, s1, s);
+  return cudaGetLastError();
+}
+
+}  // namespace cgk
