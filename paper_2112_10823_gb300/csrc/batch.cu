@@ -510,8 +510,13 @@ void admit(cg_batch_ctx* b) {
     }
     cgh::Partition part;
     cgh::build_partition(rp, n, group, b->mixed, part, shape);
+    Layout L = layout_of(n, nnz, part, group, b->mixed, b->jacobi);
+    if (L.total > b->arena.cap()) {
+      shape.tight = true;
+      cgh::build_partition(rp, n, group, b->mixed, part, shape);
+      L = layout_of(n, nnz, part, group, b->mixed, b->jacobi);
+    }
     const int32_t nsteps = static_cast<int32_t>(part.step.size()) - 1;
-    const Layout L = layout_of(n, nnz, part, group, b->mixed, b->jacobi);
     if (L.total > b->arena.cap()) {  // (a matrix of many short steps: submit's bound allows one table less)
       std::lock_guard<std::mutex> lk(b->mu);
       b->queued.pop_front();

@@ -71,9 +71,9 @@ static int chunk_of(int64_t len, int most) {
 }
 
 static int4 make_step(int64_t row, int lanes, int mode, bool uniform, int rem, int64_t seg, int64_t entries,
-                      int chunk) {
+                      int chunk, bool tight) {
   static_assert(cgk::max_chunk<double>() < 64 && cgk::max_chunk<float>() < 64, "six bits");
-  const bool pads = (lanes < 32 || !uniform) && cgk::step_pads(seg, entries);
+  const bool pads = (lanes < 32 || !uniform) && cgk::step_pads(seg, entries, tight);
   unsigned int y = static_cast<unsigned int>(lanes) | static_cast<unsigned int>(mode) << cgk::kStepModeShift |
                    (uniform ? static_cast<unsigned int>(cgk::kStepUniform) : 0u) |
                    (pads ? static_cast<unsigned int>(cgk::kStepPadded) : 0u) |
@@ -89,7 +89,7 @@ static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end,
     const int64_t len0 = rp[row + 1] - rp[row];
     if (kind(len0) == cgk::kLongRow) {  // a warp per row
       const int rem = static_cast<int>(len0 % 32);
-      out.push_back(make_step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0, chunk));
+      out.push_back(make_step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0, chunk, shape.tight));
       ++row;
       continue;
     }
@@ -111,9 +111,10 @@ static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end,
     const int rows = static_cast<int>(row - start);
     const int64_t cnt = rp[row] - rp[start];
     if (m == cgk::kLanePerRow)
-      out.push_back(make_step(start, rows, m, minlen == maxlen, 0, maxlen, cnt, chunk));
+      out.push_back(make_step(start, rows, m, minlen == maxlen, 0, maxlen, cnt, chunk, shape.tight));
     else  // two segments per row, the first one longer by an odd entry
-      out.push_back(make_step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt, chunk));
+      out.push_back(make_step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt, chunk,
+                              shape.tight));
   }
 }
 
@@ -144,10 +145,12 @@ void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, boo
     }
   }
   P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
-  P.chunks = 0;
-  for (const int4& d : P.step)
+  P.chunks = P.padded = 0;
+  for (const int4& d : P.step) {
     if (d.z > 0) P.chunks += (d.z + chunk_size(d) - 1) / chunk_size(d);
-  P.step.push_back(make_step(n, 32, cgk::kLanePerRow, true, 0, 0, 0, chunk));  // the sentinel: no entries
+    P.padded += (d.y & cgk::kStepPadded) ? int64_t(32) * d.z : rp[d.x + rows_of(d)] - rp[d.x];
+  }
+  P.step.push_back(make_step(n, 32, cgk::kLanePerRow, true, 0, 0, 0, chunk, false));  // the sentinel: no entries
 }
 
 // Calls f(entries) for each chunk of step d, in order.
@@ -212,10 +215,11 @@ void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool m
 }
 
 void stream_bound(int64_t nnz, bool mixed, const Partition& P, int64_t* stream_units, int64_t* entries) {
-  // 32-bit columns without padding, or 16-bit ones with an eighth of it (less);
-  // at most a unit lost behind the columns and behind the values of a chunk
-  *stream_units = cgk::units((mixed ? 8 : 12) * nnz) + 2 * P.chunks;
-  *entries = nnz + nnz / 8;
+  // 32-bit columns without padding or 16-bit ones with it; at most a unit lost
+  // behind the columns and behind the values of a chunk
+  const int64_t value = mixed ? 4 : 8;
+  *stream_units = cgk::units(std::max((4 + value) * nnz, (2 + value) * P.padded)) + 2 * P.chunks;
+  *entries = P.padded;
 }
 
 }  // namespace cgh

@@ -19,6 +19,7 @@ struct Partition {
   std::vector<int32_t> warp_step;
   std::vector<int32_t> block_row;
   int64_t chunks = 0;        // of all streams
+  int64_t padded = 0;        // entries with the padding of 16-bit columns
   // by place_steps
   std::vector<int4> warp_chunk;
   std::vector<uint32_t> chunk_off;
@@ -38,6 +39,7 @@ struct Partition {
 constexpr int kShapeMaxLen = 64;
 struct StepShape {
   int8_t mode[kShapeMaxLen + 1];
+  bool tight = false;  // little padding (cgk::step_pads)
   StepShape();
   bool valid() const;
 };
