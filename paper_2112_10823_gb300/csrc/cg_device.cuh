@@ -150,6 +150,19 @@ struct FxPart {
   int32_t nf;
 };
 
+// Sum over the warp of one integer per lane (modulo 2^64), in limbs of 20, 20 and
+// 24 bits: three 32-bit reductions side by side take some 60 cycles, five rounds of
+// 64-bit shuffles 175.
+__device__ __forceinline__ long long warp_sum_int(long long m) {
+  const unsigned int l0 = static_cast<unsigned int>(m) & 0xfffffu;
+  const unsigned int l1 = static_cast<unsigned int>(m >> 20) & 0xfffffu;
+  const int l2 = static_cast<int>(m >> 40);
+  const unsigned int s0 = __reduce_add_sync(0xffffffffu, l0);
+  const unsigned int s1 = __reduce_add_sync(0xffffffffu, l1);
+  const int s2 = __reduce_add_sync(0xffffffffu, l2);
+  return (static_cast<long long>(s2) << 40) + (static_cast<long long>(s1) << 20) + s0;
+}
+
 // Sum over the warp of one double per lane, exactly, in fixed point at the
 // warp's largest exponent E (spacing 2^(E-1074), about 2^-51 of the largest
 // value; 32 values leave ample headroom).  Every lane gets the same result.
@@ -167,9 +180,7 @@ __device__ __forceinline__ FxPart fx_warp(double v) {
       m = (bits >> 63) ? -static_cast<long long>(rnd) : static_cast<long long>(rnd);
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  return FxPart{m, E, nf};
+  return FxPart{warp_sum_int(m), E, nf};
 }
 
 // Sum of up to 32 partials, one per lane (`valid` lanes), realigned to the
@@ -190,9 +201,7 @@ __device__ __forceinline__ FxPart fx_combine(FxPart p, bool valid) {
       m = p.m < 0 ? -r : r;
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  return FxPart{m, E, nf};
+  return FxPart{warp_sum_int(m), E, nf};
 }
 
 // m 2^k for a double m of magnitude below 2^64 (an integer's conversion), by its
@@ -284,9 +293,7 @@ __device__ __forceinline__ double fx_warp_sum_array(const double* src, int count
       }
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-  return fx_value(FxPart{m, E, nf});
+  return fx_value(FxPart{warp_sum_int(m), E, nf});
 }
 
 // ---- sums through accumulators
@@ -348,28 +355,14 @@ __device__ __forceinline__ void acc_words(FxPart p, int eb, unsigned long long* 
 __device__ __forceinline__ bool acc_sum(unsigned long long lo, unsigned long long hi, unsigned int count, int eb,
                                         double* sum) {
   if ((lo >> 11) & kAccCount) return false;
-  const long long high = static_cast<long long>(hi - count) >> 11;
-  const unsigned long long low = lo >> 22;
-  unsigned long long l = (static_cast<unsigned long long>(high) << 32) + low;
-  unsigned long long h = static_cast<unsigned long long>(high >> 32) + (l < low ? 1ull : 0ull);
-  const bool neg = (h >> 63) != 0;
-  if (neg) {
-    l = ~l + 1ull;
-    h = ~h + (l == 0 ? 1ull : 0ull);
-  }
-  int k = 0;
-  if (h != 0) {  // the leading 64 bits, the rest as a sticky bit
-    k = 64 - __clzll(static_cast<long long>(h));
-    const unsigned long long rest = l << (64 - k);
-    l = (h << (64 - k)) | (l >> k) | (rest != 0 ? 1ull : 0ull);
-  }
-  if (k == 0 && l < (1ull << 54)) return false;
-  const double v = __ull2double_rn(l);
+  // both parts are exact doubles, and the FMA rounds once
+  const double high = __ll2double_rn(static_cast<long long>(hi - count) >> 11);
+  const double low = __ull2double_rn(lo >> 22);
+  const double v = fma(high, 4294967296.0, low);
   const long long bits = __double_as_longlong(v);
-  const int add = k + eb - kAccUnit, e = static_cast<int>(bits >> 52) + add;
-  if (e <= 0 || e >= 2047) return false;
-  const double r = __longlong_as_double(bits + (static_cast<long long>(add) << 52));
-  *sum = neg ? -r : r;
+  const int ev = static_cast<int>((bits >> 52) & 0x7ff), e = ev + eb - kAccUnit;
+  if (ev < 1023 + 54 || e <= 0 || e >= 2047) return false;
+  *sum = __longlong_as_double(bits + (static_cast<long long>(eb - kAccUnit) << 52));
   return true;
 }
 
