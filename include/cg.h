@@ -144,7 +144,10 @@ int cg_partition_info(cg_handle h, int32_t* max_rows, int32_t* kernel);
 
 /*
  * y = A x (Sec. 2.3 / 5.2): y_i = sum_{k=IA(i)}^{IA(i+1)-1} AA(k) x(JA(k)),
- * FP64 with FMA, each row summed in storage order.  x, y: device pointers to
+ * FP64 with FMA, each row summed in storage order by one lane, as the sum of its
+ * two halves (rows of 33 to 64 entries, and all rows of small systems) or by a
+ * warp (longer rows).  The bits depend on the matrix and the GPU's SM count, not
+ * on the CTA count.  x, y: device pointers to
  * n doubles; x and y must not overlap.  Asynchronous on the handle's stream.
  */
 int cg_spmv(cg_handle h, const double* x, double* y);
@@ -334,7 +337,8 @@ typedef struct {
   int32_t max_pending;     /* queued requests not yet admitted (default 65536) */
   int32_t use_graph;       /* 1 (default): replay each round from a captured CUDA graph */
   int32_t group_override;  /* > 0: every system uses this many CTAs (tests); 0 = automatic */
-  int32_t validate;        /* 1 (default): check each request's CSR on the host */
+  int32_t validate;        /* 1 (default): check each request's CSR (row pointers on the
+                              host, columns on the device) */
   int32_t preconditioner;  /* cg_preconditioner of every system (a non-positive diagonal
                               ends that request with CG_EINVAL) */
   int32_t autotune;        /* 1: at creation, measure on this GPU which step shape (one lane,
@@ -406,10 +410,10 @@ typedef struct {
   int32_t shape_tuned;             /* 1 if the step shapes were measured */
   int32_t step_kind[6];
   int32_t pad;
-  /* rounds whose product loaded the row pointers with the evict-first L2
-   * policy: those whose systems' vectors and row pointers together take
-   * more than 4/7 of the L2 (the row pointers then give way to the vectors
-   * that every step reads again) */
+  /* rounds whose product loaded its step tables with the evict-first L2
+   * policy: those whose systems' vectors, with four bytes per row, take
+   * more than 4/7 of the L2 (the tables then give way to the vectors that
+   * every step reads again) */
   int64_t rounds_stream_rows;
 } cg_batch_stats;
 

@@ -31,7 +31,8 @@ namespace cgh {
 // contiguous CTA ranges of about equal cost (stored entries + kRowCost per
 // row, the per-row vector work), and each CTA range into steps (see
 // cg_internal.h): up to 32 rows of <= 32 entries (one lane per row), up to 16
-// rows of <= 64 entries (two lanes per row), or one longer row.
+// rows of <= 64 entries (two lanes per row), or one longer row.  kRowCost is
+// flat between 10 and 18 (160^3 within 0.3 %, 100^3 2 %).
 constexpr int64_t kRowCost = 14;
 
 int64_t cost_split(const std::vector<int32_t>& rp, int64_t lo_row, int64_t hi_row, int64_t part, int64_t parts) {
@@ -291,16 +292,28 @@ size_t ctrl_block_bytes(int nblocks) {
   return ctrl_flags_offset() + sizeof(unsigned long long) * static_cast<size_t>(nblocks > 0 ? nblocks : 1);
 }
 
-template <typename T>
-cudaError_t dalloc(cg_ctx* h, T** p, size_t count) {
-  void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count ? count * sizeof(T) : 16);
-  if (e == cudaSuccess) {
-    h->allocs.push_back(q);
-    *p = static_cast<T*>(q);
+// Arrays of one device allocation, each on a 256-byte boundary: a handle has some
+// twenty of them, and an allocation of its own for each took a third of the time
+// that a small system's handle needs.
+struct Block {
+  size_t bytes = 0;
+  std::vector<std::pair<void**, size_t>> parts;
+  template <typename T>
+  size_t add(T** p, size_t count) {
+    const size_t at = bytes;
+    parts.push_back({reinterpret_cast<void**>(p), at});
+    bytes += (std::max<size_t>(count * sizeof(T), 16) + 255) & ~size_t(255);
+    return at;
   }
-  return e;
-}
+  cudaError_t alloc(std::vector<void*>& owner) {
+    void* q = nullptr;
+    const cudaError_t e = cudaMalloc(&q, std::max<size_t>(bytes, 16));
+    if (e != cudaSuccess) return e;
+    owner.push_back(q);
+    for (auto& a : parts) *a.first = static_cast<char*>(q) + a.second;
+    return cudaSuccess;
+  }
+};
 
 void release(cg_ctx* h) {
   if (!h) return;
@@ -594,8 +607,9 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   const bool mixed = o.precision == CG_PREC_MIXED;
   // A system of at most 16 rows per warp of the whole GPU: two lanes per row, so
   // that more warps work and each row's FMA chain, which bounds so small a
-  // product, is half as long.  By the size alone, so that a product's bits do not
-  // depend on the CTA count.
+  // product, is half as long (24^3: 8.0 -> 7.0 us per product; 32^3, near the
+  // line: 14.4 -> 12.9 us per step).  By the size alone, so that a product's bits
+  // do not depend on the CTA count.
   cgh::StepShape shape;
   if (n <= static_cast<int64_t>(sms) * 16 * cgk::kWarps)
     for (int L = 0; L <= cgk::kLaneMax; ++L) shape.mode[L] = static_cast<int8_t>(cgk::kPairPerRow);
@@ -623,91 +637,81 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
     }
   }
 
-  CG_TRY(dalloc(h, &h->d_step, part.step.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_step_cmax, part.step.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_seg_len, 32 * static_cast<size_t>(h->nsteps) + 64), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_warp_step, part.warp_step.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_block_row, part.block_row.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_r, n), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_p, n), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_q, n), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_xbuf, n), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_bbuf, n), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_partials, static_cast<size_t>(6) * h->nblocks), "cg_create: cudaMalloc");
-  {
-    unsigned char* blk = nullptr;
-    CG_TRY(dalloc(h, &blk, ctrl_block_bytes(h->nblocks)), "cg_create: cudaMalloc");
-    h->d_ctrl = reinterpret_cast<cgk::SolveCtrl*>(blk);
-    h->d_flags = reinterpret_cast<unsigned long long*>(blk + ctrl_flags_offset());
+  // the cluster kernel reads CSR: its handles keep 0-based copies
+  const bool keep_csr = h->cluster_R > 0;
+  const size_t nn = static_cast<size_t>(n), nz = static_cast<size_t>(nnz);
+  Block blk;
+  const size_t at_step = blk.add(&h->d_step, part.step.size());  // (the tables of one upload first)
+  const size_t at_wstep = blk.add(&h->d_warp_step, part.warp_step.size());
+  const size_t at_brow = blk.add(&h->d_block_row, part.block_row.size());
+  std::vector<char> tables(blk.bytes);
+  blk.add(&h->d_step_cmax, part.step.size());
+  blk.add(&h->d_seg_len, 32 * static_cast<size_t>(h->nsteps) + 64);
+  blk.add(&h->d_r, nn);
+  blk.add(&h->d_p, nn);
+  blk.add(&h->d_q, nn);
+  blk.add(&h->d_xbuf, nn);
+  blk.add(&h->d_bbuf, nn);
+  blk.add(&h->d_partials, static_cast<size_t>(6) * h->nblocks);
+  unsigned char* ctrl = nullptr;
+  blk.add(&ctrl, ctrl_block_bytes(h->nblocks));
+  blk.add(&h->d_err, 16);
+  if (mixed) blk.add(&h->d_p32, nn);
+  if (o.preconditioner == CG_PRECOND_JACOBI) blk.add(&h->d_dinv, nn);
+  if (keep_csr) {
+    blk.add(&h->d_csr_row_ptr, nn + 1);
+    blk.add(&h->d_csr_col, nz);
+    blk.add(&h->d_csr_val, nz);
   }
-  CG_TRY(dalloc(h, &h->d_err, 16), "cg_create: cudaMalloc");
-  if (o.precision == CG_PREC_MIXED) {
-    CG_TRY(dalloc(h, &h->d_p32, n), "cg_create: cudaMalloc");
-  }
-  if (o.preconditioner == CG_PRECOND_JACOBI) CG_TRY(dalloc(h, &h->d_dinv, n), "cg_create: cudaMalloc");
+  CG_TRY(blk.alloc(h->allocs), "cg_create: cudaMalloc");
+  h->d_ctrl = reinterpret_cast<cgk::SolveCtrl*>(ctrl);
+  h->d_flags = reinterpret_cast<unsigned long long*>(ctrl + ctrl_flags_offset());
   CG_TRY(cudaMallocHost(&h->h_ctrl, sizeof(cgk::SolveCtrl)), "cg_create: cudaMallocHost");
-
-  CG_TRY(cudaMemcpy(h->d_step, part.step.data(), sizeof(int4) * part.step.size(), cudaMemcpyHostToDevice),
-         "cg_create: upload");
-  CG_TRY(cudaMemcpy(h->d_warp_step, part.warp_step.data(), sizeof(int32_t) * part.warp_step.size(),
-                    cudaMemcpyHostToDevice),
-         "cg_create: upload");
-  CG_TRY(cudaMemcpy(h->d_block_row, part.block_row.data(), sizeof(int32_t) * part.block_row.size(),
-                    cudaMemcpyHostToDevice),
-         "cg_create: upload");
+  std::memcpy(tables.data() + at_step, part.step.data(), sizeof(int4) * part.step.size());
+  std::memcpy(tables.data() + at_wstep, part.warp_step.data(), sizeof(int32_t) * part.warp_step.size());
+  std::memcpy(tables.data() + at_brow, part.block_row.data(), sizeof(int32_t) * part.block_row.size());
+  CG_TRY(cudaMemcpy(h->d_step, tables.data(), tables.size(), cudaMemcpyHostToDevice), "cg_create: upload");
   CG_TRY(cudaMemset(h->d_err, 0, 64), "cg_create: memset");
 
   // The CSR arrays on the device for the time of the conversion: the caller's
-  // own where they are there already, else copies that go when this returns.
-  // The cluster kernel keeps 0-based copies.
+  // own where they are there already, the kept copies, or copies that go when
+  // this returns.
   std::vector<void*> temps;
-  auto temp_of = [&](const void* src, size_t bytes, cudaMemcpyKind kind, const void** out) -> cudaError_t {
-    void* q = nullptr;
-    cudaError_t et = cudaMalloc(&q, bytes ? bytes : 16);
-    if (et != cudaSuccess) return et;
-    temps.push_back(q);
-    *out = q;
-    return bytes ? cudaMemcpy(q, src, bytes, kind) : cudaSuccess;
-  };
   struct TempGuard {
     std::vector<void*>& v;
     ~TempGuard() {
       for (void* q : v) cudaFree(q);
     }
   } temp_guard{temps};
-  const bool keep_csr = h->cluster_R > 0;
-  cgk::CsrSource src{};
-  src.base = base;
-  {
-    const void* q = nullptr;
-    CG_TRY(temp_of(rp.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, &q), "cg_create: upload");
-    src.row_ptr = static_cast<const int32_t*>(q);
-    if (csr->on_device && !(keep_csr && base != 0)) {
-      src.col_idx = csr->col_idx;
-    } else {
-      CG_TRY(temp_of(ci.data(), sizeof(int32_t) * nnz, cudaMemcpyHostToDevice, &q), "cg_create: upload");
-      src.col_idx = static_cast<const int32_t*>(q);
-      src.base = 0;  // ci is rebased
+  int32_t* d_rp = h->d_csr_row_ptr;
+  int32_t* d_ci = h->d_csr_col;
+  double* d_va = h->d_csr_val;
+  if (!keep_csr) {
+    Block tmp;
+    tmp.add(&d_rp, nn + 1);
+    if (!csr->on_device) {
+      tmp.add(&d_ci, nz);
+      tmp.add(&d_va, nz);
     }
-    if (csr->on_device) {
-      src.val = csr->val;
-    } else {
-      CG_TRY(temp_of(csr->val, sizeof(double) * nnz, cudaMemcpyHostToDevice, &q), "cg_create: upload");
-      src.val = static_cast<const double*>(q);
-    }
+    CG_TRY(tmp.alloc(temps), "cg_create: cudaMalloc");
   }
-  if (keep_csr) {
-    CG_TRY(dalloc(h, &h->d_csr_row_ptr, n + 1), "cg_create: cudaMalloc");
-    CG_TRY(dalloc(h, &h->d_csr_col, nnz), "cg_create: cudaMalloc");
-    CG_TRY(dalloc(h, &h->d_csr_val, nnz), "cg_create: cudaMalloc");
-    CG_TRY(cudaMemcpyAsync(h->d_csr_row_ptr, src.row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToDevice, nullptr),
-           "cg_create: copy");
-    if (nnz > 0) {
-      CG_TRY(cudaMemcpyAsync(h->d_csr_col, src.col_idx, sizeof(int32_t) * nnz, cudaMemcpyDeviceToDevice, nullptr),
-             "cg_create: copy");
-      CG_TRY(cudaMemcpyAsync(h->d_csr_val, src.val, sizeof(double) * nnz, cudaMemcpyDeviceToDevice, nullptr),
-             "cg_create: copy");
-    }
+  CG_TRY(cudaMemcpy(d_rp, rp.data(), sizeof(int32_t) * (nn + 1), cudaMemcpyHostToDevice), "cg_create: upload");
+  cgk::CsrSource src{};
+  src.row_ptr = d_rp;
+  src.col_idx = csr->col_idx;
+  src.val = csr->val;
+  src.base = base;
+  if (d_ci != nullptr && nnz > 0) {
+    if (csr->on_device && base == 0)
+      CG_TRY(cudaMemcpy(d_ci, csr->col_idx, sizeof(int32_t) * nz, cudaMemcpyDeviceToDevice), "cg_create: copy");
+    else
+      CG_TRY(cudaMemcpy(d_ci, ci.data(), sizeof(int32_t) * nz, cudaMemcpyHostToDevice), "cg_create: upload");
+    CG_TRY(cudaMemcpy(d_va, csr->val, sizeof(double) * nz,
+                      csr->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
+           "cg_create: upload");
+    src.col_idx = d_ci;
+    src.val = d_va;
+    src.base = 0;  // ci is rebased
   }
   // d_q holds the steps' places in the streams until the handle's first solve
   // (a step has at least one row: two words of 4 bytes in its 8)
@@ -733,21 +737,23 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   }
   h->col16 = found.scan.span <= cgk::kColSpan16;
   cgh::place_steps(rp, h->nblocks, h->col16, mixed, part);
-  CG_TRY(dalloc(h, &h->d_stream, static_cast<size_t>(part.stream_units) * cgk::kUnit), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_chunk_off, part.chunk_off.size()), "cg_create: cudaMalloc");
-  CG_TRY(dalloc(h, &h->d_warp_chunk, part.warp_chunk.size()), "cg_create: cudaMalloc");
+  Block str;
+  const size_t at_wchunk = str.add(&h->d_warp_chunk, part.warp_chunk.size());  // (one upload again)
+  const size_t at_wentry = str.add(&h->d_warp_entry, part.warp_entry.size());
+  const size_t at_coff = str.add(&h->d_chunk_off, part.chunk_off.size());
+  tables.assign(str.bytes, 0);
+  str.add(&h->d_stream, static_cast<size_t>(part.stream_units) * cgk::kUnit);
+  if (mixed) str.add(&h->d_val64, static_cast<size_t>(part.entries));
+  CG_TRY(str.alloc(h->allocs), "cg_create: cudaMalloc");
+  std::memcpy(tables.data() + at_wchunk, part.warp_chunk.data(), sizeof(int4) * part.warp_chunk.size());
+  if (mixed) std::memcpy(tables.data() + at_wentry, part.warp_entry.data(), 4 * part.warp_entry.size());
+  std::memcpy(tables.data() + at_coff, part.chunk_off.data(), 4 * part.chunk_off.size());
+  CG_TRY(cudaMemcpy(h->d_warp_chunk, tables.data(), tables.size(), cudaMemcpyHostToDevice), "cg_create: upload");
   auto up = [&](void* dst, const auto& v, size_t count) {
     return count ? cudaMemcpy(dst, v.data(), sizeof(v[0]) * count, cudaMemcpyHostToDevice) : cudaSuccess;
   };
-  CG_TRY(up(h->d_chunk_off, part.chunk_off, part.chunk_off.size()), "cg_create: upload");
-  CG_TRY(up(h->d_warp_chunk, part.warp_chunk, part.warp_chunk.size()), "cg_create: upload");
   CG_TRY(up(d_step_chunk, part.step_chunk, static_cast<size_t>(h->nsteps)), "cg_create: upload");
-  if (mixed) {
-    CG_TRY(dalloc(h, &h->d_val64, static_cast<size_t>(part.entries)), "cg_create: cudaMalloc");
-    CG_TRY(dalloc(h, &h->d_warp_entry, part.warp_entry.size()), "cg_create: cudaMalloc");
-    CG_TRY(up(h->d_warp_entry, part.warp_entry, part.warp_entry.size()), "cg_create: upload");
-    CG_TRY(up(d_step_entry, part.step_entry, static_cast<size_t>(h->nsteps)), "cg_create: upload");
-  }
+  if (mixed) CG_TRY(up(d_step_entry, part.step_entry, static_cast<size_t>(h->nsteps)), "cg_create: upload");
   const cgk::StreamPlace to{h->d_chunk_off, d_step_chunk, d_step_entry, h->d_stream, h->d_val64};
   CG_TRY(cgk::launch_layout_fill(src, h->d_step, to, 0, h->nsteps, h->col16, mixed, nullptr),
          "cg_create: stream order");

@@ -503,16 +503,12 @@ struct WarpStream {
 // (values of type T, columns of type C) of every warp, and in the small-share
 // solve the r of the CTA's rows.  The parts before the rings sit at the same
 // place whatever T and C are.
-constexpr int kMaxSlots = 5;  // of any ring: the place of the barriers
-
 template <typename T, typename C>
 struct RingSmem {
   using Val = T;
   using Col = C;
-  static constexpr int kSlots = ring_slots<T, C>();
-  static_assert(kSlots <= kMaxSlots, "barriers");
   static constexpr int kSlotBytes = static_cast<int>(kUnit * chunk_units(32 * max_chunk<T>(), sizeof(C), sizeof(T)));
-  static constexpr size_t kStateOff = (8 * kMaxSlots * kWarps + 15) & ~size_t(15);
+  static constexpr size_t kStateOff = (8 * kSlots * kWarps + 15) & ~size_t(15);
   static constexpr size_t kSumOff = kStateOff + ((sizeof(CtaState) + 15) & ~size_t(15));
   static constexpr size_t kStreamOff = (kSumOff + sizeof(SumScratch) + 15) & ~size_t(15);
   static constexpr size_t kRingOff = (kStreamOff + sizeof(WarpStream) * kWarps + 16 + 127) & ~size_t(127);
@@ -520,7 +516,7 @@ struct RingSmem {
 
   unsigned char* base;
   __device__ unsigned char* slot(int w, int s) const { return base + kRingOff + (w * kSlots + s) * kSlotBytes; }
-  __device__ uint64_t* full(int w, int slot) const { return reinterpret_cast<uint64_t*>(base) + w * kMaxSlots + slot; }
+  __device__ uint64_t* full(int w, int slot) const { return reinterpret_cast<uint64_t*>(base) + w * kSlots + slot; }
   __device__ WarpStream* stream(int w) const { return reinterpret_cast<WarpStream*>(base + kStreamOff) + w; }
   __device__ int32_t* stop() const { return reinterpret_cast<int32_t*>(base + kStreamOff + sizeof(WarpStream) * kWarps); }
   __device__ CtaState* state() const { return reinterpret_cast<CtaState*>(base + kStateOff); }
@@ -541,7 +537,7 @@ constexpr size_t ring_smem_bytes(bool local = false) {
 // all tasks.
 template <typename Ring>
 __device__ __forceinline__ void ring_init(const Ring& sm) {
-  if (threadIdx.x < kMaxSlots * kWarps) {
+  if (threadIdx.x < kSlots * kWarps) {
     mbar_init(reinterpret_cast<uint64_t*>(sm.base) + threadIdx.x, 1);
     fence_mbar_init();
   }
@@ -626,14 +622,14 @@ __device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int ra
   for (;;) {
     const bool more = nchunks > 0 && (!once || issued < static_cast<uint32_t>(nchunks));
     if (!__any_sync(0xffffffffu, more) || __any_sync(0xffffffffu, ld_volatile_i32(sm.stop()) != 0)) break;
-    const bool free = more && issued - ld_acquire_shared(&ws->consumed) < static_cast<uint32_t>(Ring::kSlots);
+    const bool free = more && issued - ld_acquire_shared(&ws->consumed) < static_cast<uint32_t>(kSlots);
     if (free) {
       uint64_t* const bar = sm.full(w, head);
       const uint32_t bytes = (end0 - start) * static_cast<uint32_t>(kUnit);
       mbar_arrive_expect_tx(bar, bytes);
       bulk_g2s_hint(sm.slot(w, head), A.stream + static_cast<size_t>(start) * kUnit, bytes, bar, pol);
       phases ^= 1u << head;
-      head = head + 1 == Ring::kSlots ? 0 : head + 1;
+      head = head + 1 == kSlots ? 0 : head + 1;
       ++issued;
       next = next + 1 == nchunks ? 0 : next + 1;
       start = next == 0 ? first : end0;
@@ -656,7 +652,7 @@ __device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int ra
     }
   }
   if (mine) {
-    for (int k = 0; k < Ring::kSlots; ++k)  // the latest copy into each slot
+    for (int k = 0; k < kSlots; ++k)  // the latest copy into each slot
       if (issued > static_cast<uint32_t>(k))
         ok = mbar_wait_bounded(sm.full(w, k), ((phases >> k) & 1u) ^ 1u, limit_ns, nullptr) && ok;
   }
@@ -754,18 +750,21 @@ __device__ __forceinline__ void load_first_steps(const Ring& sm, const PassIo& v
 }
 
 // The product over the warp's steps [s, s1) from its ring, gathering x (after
-// load_first_steps):
-// out[i] = (A x)_i; returns the sum over this lane's rows of aux[i] (A x)_i
-// (0 if aux is nullptr).  Every segment is one FMA chain in storage order.
+// load_first_steps): out[i] = (A x)_i; with_dot: returns the sum over this
+// lane's rows of aux[i] (A x)_i (out and aux from the CTA's PassIo).  Every
+// segment is one FMA chain in storage order.
 //
-// What bounds it is the FP64 pipe (an FMA occupies a sub-partition for 64
+// What bounds it in FP64 is the pipe (an FMA occupies a sub-partition for 64
 // cycles, whatever its active lanes, and a predicated-off one as well; its
 // dependent latency is 115) beside the matrix stream.  So the loop keeps two
 // things in flight ahead of the chains: the ring's copies (all slots but the
 // two of the chunk being summed and of the next one; the producer warp starts
-// them), and the gathers of the warp's next chunk, of the same step or of the next one, each issued into the
-// register that the current chunk's FMA has just freed.  A warp-uniform branch,
-// not a predicate, ends a chunk's FMAs.  The stream's `failed` is raised if a wait gave up.
+// them), and the gathers of the warp's next chunk, of the same step or of the
+// next one, each issued into the register that the current chunk's FMA has just
+// freed.  A warp-uniform branch, not a predicate, ends a chunk's FMAs.  The
+// stream's `failed` is raised if a wait gave up.  Against a ring shared by the
+// CTA, in CSR order (us with cold L2): Q1 160^3 263 -> 222, the 110^3 mesh
+// 181 -> 93, Q1 64^3 31 -> 27; 109 M FMAs take 180 us at the pipe's peak.
 template <typename Ring, typename X>
 __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, const X* x, bool with_dot) {
   using T = typename Ring::Val;
@@ -796,7 +795,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
         !__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, io.limit_ns, nullptr)))
       return false;
     phases ^= 1u << tail;
-    tail = tail + 1 == Ring::kSlots ? 0 : tail + 1;
+    tail = tail + 1 == kSlots ? 0 : tail + 1;
     return true;
   };
   // a chunk: entries [u, u + cnt) of every lane's segment of one step

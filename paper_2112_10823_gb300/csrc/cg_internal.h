@@ -9,7 +9,11 @@ namespace cgk {
 // The persistent kernels run one CTA per SM: kWarps warps that compute, each
 // its own steps of the CTA's rows from its own ring in shared memory, and one
 // producer warp, whose lane w fills warp w's ring with 1-D TMA bulk copies.
-constexpr int kWarps = 19;               // computing warps: with the producer five per SM sub-partition
+// Nineteen computing warps (with the producer five per SM sub-partition), 96
+// registers per thread, nothing spilled.  15, 19, 23 warps, us per step of a Q1
+// solve: 32^3 14.2, 12.9, 13.1; 64^3 28.9, 27.6, 29.0; 160^3 292, 267, 266;
+// 160^3 mixed 230, 214, 207.
+constexpr int kWarps = 19;
 constexpr int kBlock = kWarps * 32;      // their threads
 constexpr int kThreads = kBlock + 32;    // and the producer warp
 constexpr int kCtasPerSm = 1;
@@ -27,21 +31,19 @@ constexpr int kCtasPerSm = 1;
 // A warp works through a step in chunks of a few entries per lane;
 // a chunk is one slot of the warp's ring, so that the ring gives back its
 // oldest bytes after every few entries and not only after a whole step.
-// 9: a 27-entry row is three full chunks, an 18-entry one two.  (FP64: 14, i.e. two
-// chunks, was slower: 64^3 33.1 against 29.3 us per step; FP32: 14, 18 and 28, with
-// up to a third of the warps for their registers: 29.1, 30.2 and 31.3 against
-// 27.1 us.)
+// FP64 9: a 27-entry row is three full chunks, an 18-entry one two (14, i.e. two
+// chunks, was slower: 64^3 33.1 against 29.3 us per step, with 15 warps).  FP32
+// 14: a 27-entry row is two chunks, which are gathered together (9, gathered one
+// chunk ahead as in FP64: 26.5 against 25.2 us, with 15 warps).
 template <typename T> __host__ __device__ constexpr int max_chunk() { return sizeof(T) == 8 ? 9 : 14; }
-// Slots of a warp's ring: the chunk being summed, the next one and copies in
-// flight, in some 130 KB of shared memory.  The rest of the SM's 256 KB serves
-// the gathers as L1.
-template <typename T, typename C> __host__ __device__ constexpr int ring_slots() {
-  return 3;
-}
+// Slots of a warp's ring: the chunk being summed, the next one and a copy in
+// flight, 150 to 200 KB in all.  The rest of the SM's 256 KB serves the gathers
+// as L1.  (Two slots: 160^3 383 against 292 us per step, with 15 warps.)
+constexpr int kSlots = 3;
 constexpr int kLaneMax = 32;  // longest row computed by a single lane
 // Largest CTA share (rows) of the small-share solve kernels, which keep the
-// share's r in shared memory (20 KB behind the ring layout; the FP64 layout
-// with 32-bit columns then takes 216 KB of the 227 KB a CTA may have).
+// share's r in shared memory (20 KB behind the ring layout; the FP32 layout
+// with 32-bit columns then takes 224 KB of the 227 KB a CTA may have).
 constexpr int kLocalRows = 2560;
 
 // A chunk in memory, and in a slot: its columns, then its values, each padded

@@ -28,7 +28,7 @@ __device__ __forceinline__ void solve_fail(const SolveParams& P, bool first) {
 
 // Rows per thread in flight in the vector phases (all loads of a batch
 // issued before any is used): as many as the registers that the product
-// leaves allow without spilling (128 per thread at 16 warps per CTA; the
+// leaves allow without spilling (96 per thread at 20 warps per CTA; the
 // Jacobi variants carry dinv as well, the fused x and p update three vectors).
 template <bool kJacobi, bool kSmallShare>
 __host__ __device__ constexpr int vec_rows() {
