@@ -133,7 +133,7 @@ struct SolveCtrl {
   unsigned long long rounds;    // group-barrier rounds completed so far
   int32_t slot;                 // partial-sum slot the next group sum uses
   int32_t pad;
-  // The step sums' accumulators (group_sum_fast): two words for each of p.q, r.r
+  // The step sums' accumulators (acc_words): two words for each of p.q, r.r
   // and r.z, never cleared during a solve; their values and the exponents of the
   // last sums at the end of a launch.
   alignas(16) unsigned long long acc[3][2];
