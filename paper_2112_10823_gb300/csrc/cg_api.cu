@@ -686,7 +686,8 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   int32_t* d_rp = h->d_csr_row_ptr;
   int32_t* d_ci = h->d_csr_col;
   double* d_va = h->d_csr_val;
-  if (!keep_csr) {
+  const bool callers_rp = !keep_csr && csr->on_device && base == 0;  // (the caller's row pointers serve as they are)
+  if (!keep_csr && !callers_rp) {
     Block tmp;
     tmp.add(&d_rp, nn + 1);
     if (!csr->on_device) {
@@ -695,9 +696,10 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
     }
     CG_TRY(tmp.alloc(temps), "cg_create: cudaMalloc");
   }
-  CG_TRY(cudaMemcpy(d_rp, rp.data(), sizeof(int32_t) * (nn + 1), cudaMemcpyHostToDevice), "cg_create: upload");
+  if (!callers_rp)
+    CG_TRY(cudaMemcpy(d_rp, rp.data(), sizeof(int32_t) * (nn + 1), cudaMemcpyHostToDevice), "cg_create: upload");
   cgk::CsrSource src{};
-  src.row_ptr = d_rp;
+  src.row_ptr = callers_rp ? csr->row_ptr : d_rp;
   src.col_idx = csr->col_idx;
   src.val = csr->val;
   src.base = base;
