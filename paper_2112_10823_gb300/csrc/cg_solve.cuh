@@ -550,7 +550,9 @@ __device__ __forceinline__ void solve_task(const Ring& sm, const TaskState* cons
 
     // ---- what comes next, and the wait before the next product gathers
     const int32_t f = st->flags;
-    const bool last = (f & (kFlagDone | kFlagBreakdown)) || st->k >= P.maxit;
+    // a replacement comes before the step limit: it alone tells whether a mixed
+    // solve has converged
+    const bool last = (f & (kFlagDone | kFlagBreakdown)) || (!(f & kFlagReplace) && st->k >= P.maxit);
     const bool next_step = !last && !(f & kFlagReplace);
     bool synced;
     if constexpr (kNeighborWait)

@@ -1,0 +1,56 @@
+"""Calls at their limits, on the GPU: the step limit at the step that converges."""
+import numpy as np
+import pytest
+
+import fe_inputs as fi
+import oracle
+from gpu_util import cg_mod, handle
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-10
+
+
+def _system(N, seed):
+    A = fi.q1(N, 1.0, seed)
+    return A, oracle.spmv(A, fi.xstar(seed, A.n))
+
+
+@pytest.mark.parametrize("ctas", [3, 0])  # the large-share kernel and the small-share one
+@pytest.mark.parametrize("jacobi", [0, 1])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_step_limit_at_the_converging_step(precision, jacobi, ctas):
+    """A solve whose limit is the step that converges has converged (in mixed
+    precision the residual replacement behind that step tells), with the same
+    bits; with one step less it has not."""
+    cg = cg_mod()
+    A, b = _system(22, 81)
+    with handle(A, ctas=ctas, precision=precision, preconditioner=jacobi) as h:
+        assert h.partition_info()[1] == (cg.CG_SOLVE_KERNEL_LARGE_SHARE if ctas else cg.CG_SOLVE_KERNEL_SMALL_SHARE)
+        xs, res = [], []
+        for maxit in (10 * A.n, None, -1):
+            x = np.zeros(A.n)
+            limit = maxit if not res else res[0].iters + (maxit or 0)
+            res.append(cg.cg_solve(h, b, x, tol=TOL, maxit=limit))
+            xs.append(x)
+    assert [r.status for r in res] == [cg.CG_OK, cg.CG_OK, cg.CG_ENOTCONV], res
+    assert res[1].iters == res[0].iters == res[2].iters + 1
+    assert np.array_equal(xs[0], xs[1]) and res[1].relres == res[0].relres <= TOL
+
+
+@pytest.mark.parametrize("chunk", [0, 7])
+@pytest.mark.parametrize("jacobi", [0, 1])
+def test_step_limit_of_a_mixed_batch(jacobi, chunk):
+    """The same in a batch, alone and in a group of CTAs, in one round and in many."""
+    cg = cg_mod()
+    A, b = _system(12, 82)
+    for group in (1, 3):
+        with cg.Batch(precision=cg.CG_PREC_MIXED, preconditioner=jacobi, chunk_iters=chunk, group_override=group) as bt:
+            def solve(maxit):
+                x = np.zeros(A.n)
+                return bt.wait(bt.submit([cg.Request(A.row_ptr, A.col_idx, A.val, b, x, tol=TOL, maxit=maxit)])[0]), x
+            r0, x0 = solve(10 * A.n)
+            r1, x1 = solve(r0.iters)
+            r2, _ = solve(r0.iters - 1)
+        assert [r.status for r in (r0, r1, r2)] == [cg.CG_OK, cg.CG_OK, cg.CG_ENOTCONV], (r0, r1, r2)
+        assert r1.iters == r0.iters and np.array_equal(x0, x1)
