@@ -9,16 +9,16 @@
 namespace cgk {
 
 // A task of the computing warps or of the producer warp; false if the ring did
-// not drain in time.
+// not drain in time (a task that ended in a timeout has drained it all the same).
 template <bool kMixed, bool kJacobi, typename C>
 __device__ __noinline__ bool batch_task(unsigned char* smem, const TaskState* tk, int32_t stream_rows) {
   using T = std::conditional_t<kMixed, float, double>;
   using Ring = RingSmem<T, C>;
   const Ring sm{smem};
   if (threadIdx.x >= kBlock) {
-    const bool ok = producer(sm, tk->P.A, tk->rank, false, tk->P.wait_limit_ns);
-    if (!ok) solve_fail(tk->P, threadIdx.x == kBlock);
-    return ok;
+    const int end = producer(sm, tk->P.A, tk->rank, false, tk->P.wait_limit_ns);
+    if (end != kStreamDone) solve_fail(tk->P, threadIdx.x == kBlock);
+    return end != kStreamLost;
   }
   solve_task<kMixed, kJacobi, false, false>(sm, tk, stream_rows);
   stop_producer(sm);

@@ -588,11 +588,19 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // and all warps that wait for one are served together.  On stop every lane
 // waits for its copies in flight, so that none lands after the CTA is gone or
 // in a ring that the next task has taken over, and leaves the phases to that
-// task's warps.  Returns false (uniformly) if nothing moved for
-// limit_ns, or a copy did not arrive in that time.
+// task's warps.
+//
+// Waiting for a slot is no wait of the solve: the ring stays full through a
+// step's vector phases, both sums and a whole direct pass, each of which keeps
+// its own limit, and computing warps that give up say stop.  So it ends by
+// itself; its bound, far beyond theirs, is for a fault in this code only.
+// Returns (uniformly) kStreamDone, kStreamIdle if that bound ran out, or
+// kStreamLost if a copy did not arrive within limit_ns: then the ring cannot
+// be used again.
+enum : int { kStreamDone = 0, kStreamIdle = 1, kStreamLost = 2 };
 template <typename Ring>
-__device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int rank, bool once,
-                                         unsigned long long limit_ns) {
+__device__ __forceinline__ int producer(const Ring& sm, const DevCsr& A, int rank, bool once,
+                                        unsigned long long limit_ns) {
   const int w = threadIdx.x & 31;
   const bool mine = w < kWarps;
   WarpStream* const ws = sm.stream(mine ? w : 0);
@@ -616,7 +624,7 @@ __device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int ra
   const uint64_t pol = l2_evict_first_policy();
   uint32_t phases = ws->phases, issued = 0;
   int head = 0;
-  bool ok = true;
+  bool stalled = false, arrived = true;
   unsigned long long t0 = 0;
   uint32_t idle = 0;
   for (;;) {
@@ -644,8 +652,8 @@ __device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int ra
       if ((++idle & 255u) == 0) {
         const unsigned long long now = global_timer_ns();
         if (idle == 256u) t0 = now;
-        else if (now - t0 > limit_ns) {
-          ok = false;
+        else if (now - t0 > 4 * limit_ns + kProducerIdleNs) {
+          stalled = true;
           break;
         }
       }
@@ -654,13 +662,13 @@ __device__ __forceinline__ bool producer(const Ring& sm, const DevCsr& A, int ra
   if (mine) {
     for (int k = 0; k < kSlots; ++k)  // the latest copy into each slot
       if (issued > static_cast<uint32_t>(k))
-        ok = mbar_wait_bounded(sm.full(w, k), ((phases >> k) & 1u) ^ 1u, limit_ns, nullptr) && ok;
+        arrived = mbar_wait_bounded(sm.full(w, k), ((phases >> k) & 1u) ^ 1u, limit_ns, nullptr) && arrived;
   }
-  ok = __all_sync(0xffffffffu, ok);
+  arrived = __all_sync(0xffffffffu, arrived);
   // (no computing warp reads its phases any more: in a solve they have said
   // stop, a single pass keeps its own)
   if (!once && mine && nchunks > 0) ws->phases = phases;
-  return ok;
+  return !arrived ? kStreamLost : __any_sync(0xffffffffu, stalled) ? kStreamIdle : kStreamDone;
 }
 
 // The computing warps of a task are through (all of their threads call).

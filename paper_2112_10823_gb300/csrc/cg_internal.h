@@ -40,6 +40,8 @@ template <typename T> __host__ __device__ constexpr int max_chunk() { return siz
 // flight, 150 to 200 KB in all.  The rest of the SM's 256 KB serves the gathers
 // as L1.  (Two slots: 160^3 383 against 292 us per step, with 15 warps.)
 constexpr int kSlots = 3;
+// The producer warp's wait for a slot, beyond four waits of the computing warps.
+constexpr unsigned long long kProducerIdleNs = 60000000000ull;
 constexpr int kLaneMax = 32;  // longest row computed by a single lane
 // Largest CTA share (rows) of the small-share solve kernels, which keep the
 // share's r in shared memory (20 KB behind the ring layout; the FP32 layout
@@ -297,6 +299,9 @@ constexpr int32_t kSelftestSite = 99;
 constexpr int32_t kNeighborSite = 98;
 // timeout_site of a wait for a sum through the accumulators
 constexpr int32_t kAccSite = 96;
+// timeout_site of the matrix stream: a copy that did not arrive, or a ring that
+// stayed full
+constexpr int32_t kStreamSite = 95;
 // timeout_site of the synchronisation probe's barrier
 constexpr int32_t kProbeSite = 97;
 // The solves' group-wide synchronisations timed alone (cg_probe_group_sync):

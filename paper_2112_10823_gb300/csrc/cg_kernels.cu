@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   ring_init(sm);
   const unsigned long long lim = 2000000000ull;
   if (threadIdx.x >= kBlock) {
-    if (!producer(sm, A, blockIdx.x, true, lim) && threadIdx.x == kBlock) atomicExch(err, kETIMEOUT);
+    if (producer(sm, A, blockIdx.x, true, lim) != kStreamDone && threadIdx.x == kBlock) atomicExch(err, kETIMEOUT);
     return;
   }
   const int bw = blockIdx.x * kWarps + (threadIdx.x >> 5);

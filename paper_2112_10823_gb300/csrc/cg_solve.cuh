@@ -8,10 +8,11 @@
 namespace cgk {
 
 // Leave the solve after a failed wait: record the status (thread 0 of the
-// computing warps; lane 0 of the producer warp).
+// computing warps; lane 0 of the producer warp).  Waits on other CTAs have
+// recorded their site; the others are the matrix stream's.
 __device__ __forceinline__ void solve_fail(const SolveParams& P, bool first) {
   if (first) {
-    atomicExch(&P.ctrl->abort, 1);
+    if (atomicExch(&P.ctrl->abort, 1) == 0) atomicCAS(&P.ctrl->timeout_site, 0, kStreamSite);
     atomicExch(&P.ctrl->status, kETIMEOUT);
     atomicExch(&P.ctrl->phase, kPhaseDone);
   }

@@ -1,4 +1,5 @@
-"""Calls at their limits, on the GPU: the step limit at the step that converges."""
+"""Calls at their limits, on the GPU: the step limit at the step that converges,
+a wait limit shorter than a pass over the matrix."""
 import numpy as np
 import pytest
 
@@ -54,3 +55,30 @@ def test_step_limit_of_a_mixed_batch(jacobi, chunk):
             r2, _ = solve(r0.iters - 1)
         assert [r.status for r in (r0, r1, r2)] == [cg.CG_OK, cg.CG_OK, cg.CG_ENOTCONV], (r0, r1, r2)
         assert r1.iters == r0.iters and np.array_equal(x0, x1)
+
+
+
+def test_wait_limit_is_no_limit_on_a_pass():
+    """A mixed solve whose direct pass (one row of 2 M entries, one warp's work)
+    takes several times the wait limit, in a handle and in a batch: no wait on
+    another CTA or on a copy is that long, so nothing times out."""
+    import torch
+    cg = cg_mod()
+    n, long_row = 4096, 2 << 20
+    rp = torch.arange(n + 1, dtype=torch.int32, device="cuda")
+    rp[1:] += long_row - 1
+    ci = torch.cat([torch.arange(long_row, dtype=torch.int32, device="cuda") % 1024,
+                    torch.arange(1, n, dtype=torch.int32, device="cuda")])
+    va = torch.ones(ci.numel(), dtype=torch.float64, device="cuda")
+    b = torch.ones(n, dtype=torch.float64, device="cuda")
+    mixed = cg.CG_PREC_MIXED
+    with cg.Batch(precision=mixed, group_override=1, wait_limit_ms=1, validate=False) as bt:
+        reqs = [cg.Request(rp, ci, va, b, torch.zeros_like(b), tol=TOL, maxit=1) for _ in range(3)]
+        systems = [_system(8, 90 + i) for i in range(3)]
+        reqs += [cg.Request(A.row_ptr, A.col_idx, A.val, c, np.zeros(A.n), tol=TOL) for A, c in systems]
+        res = bt.wait_all(bt.submit(reqs), 60000)
+        assert bt.stats()["last_round_ms"] > 4  # two passes of the long row
+    assert [r.status for r in res] == 3 * [cg.CG_ENOTCONV] + 3 * [cg.CG_OK], res
+    with cg.cg_create(rp, ci, va, precision=mixed, ctas=1, wait_limit_ms=1) as h:
+        r = cg.cg_solve(h, b, torch.zeros_like(b), tol=TOL, maxit=1)
+    assert r.status == cg.CG_ENOTCONV, r
