@@ -318,7 +318,7 @@ bool load_structure(const cg_request& r, bool validate, std::vector<int32_t>& rp
   const int base = r.csr.index_base;
   rp.resize(static_cast<size_t>(n) + 1);
   if (r.csr.on_device) {
-    if (cudaMemcpy(rp.data(), r.csr.row_ptr, 4 * (n + 1), cudaMemcpyDeviceToHost) != cudaSuccess) {
+    if (cudaMemcpy(rp.data(), r.csr.row_ptr, 4 * (n + 1), cudaMemcpyDefault) != cudaSuccess) {
       cudaGetLastError();
       bad = "copy of row_ptr failed";
       return false;
@@ -386,7 +386,7 @@ struct Dev {
 };
 
 // Device buffer for the columns and values of at least `least` entries of a
-// request's host arrays: kStageEntries, or what one CTA's share needs if that is
+// request's arrays that are not on this device: kStageEntries, or what one CTA's share needs if that is
 // more; half as much, and so on, where memory is short.
 constexpr int64_t kStageEntries = int64_t(4) << 20;
 cudaError_t reserve_stage(cg_batch_ctx* b, int64_t least) {
@@ -424,15 +424,16 @@ void finish_without_device(cg_batch_ctx* b, Job* j, int status) {
 // to back (the host prepares the next system while the previous one's work
 // runs); the small host arrays are staged in pinned memory that stays
 // untouched until the end of the pass.  The stream order of a system needs
-// one read-back, the column scan's: systems whose arrays are on the device
-// share one for the whole pass; those with host arrays, which go through one
-// staging buffer, have one each.
+// one read-back, the column scan's: systems whose arrays are on this device
+// share one for the whole pass; those with other arrays (the host's, another
+// GPU's), which go through one staging buffer, have one each.
 void admit(cg_batch_ctx* b) {
   struct Staged {
     Job* j;
     Layout L;
     std::vector<int32_t> rp;
     cgh::Partition part;
+    bool in_place;
     cudaError_t e;
   };
   std::vector<Staged> staged;
@@ -588,10 +589,13 @@ void admit(cg_batch_ctx* b) {
     step(cudaMemsetAsync(b->d_ctrl + slot, 0, sizeof(cgk::SolveCtrl), s));
     step(cudaMemsetAsync(b->d_scan + slot, 0, sizeof(cgk::LayoutScan), s));
     cgk::CsrSource src{d.at<int32_t>(L.r), r.csr.col_idx, r.csr.val, 0, r.csr.index_base};
-    if (e == cudaSuccess && r.csr.on_device) {
+    // (the row pointers, and a matrix without entries, are there already)
+    const bool in_place = r.csr.on_device && (nnz == 0 || (cgh::readable_in_place(r.csr.col_idx, b->device) &&
+                                                           cgh::readable_in_place(r.csr.val, b->device)));
+    if (e == cudaSuccess && in_place) {
       step(scan(d, src, slot, 0, nsteps, n));
     } else if (e == cudaSuccess) {
-      // host arrays: in runs of CTA shares (consecutive rows) that fit the staging
+      // arrays elsewhere: in runs of CTA shares (consecutive rows) that fit the staging
       // buffer, scanned, read back, and uploaded again to be filled (once, if a
       // single run holds them all)
       auto first_entry = [&](int c) -> int64_t { return rp[part.block_row[c]]; };
@@ -612,8 +616,9 @@ void admit(cg_batch_ctx* b) {
         src.col_idx = c;
         src.val = v;
         if (cnt == 0) return;
-        step(cudaMemcpyAsync(c, r.csr.col_idx + e0, 4 * cnt, cudaMemcpyHostToDevice, s));
-        if (values) step(cudaMemcpyAsync(v, r.csr.val + e0, 8 * cnt, cudaMemcpyHostToDevice, s));
+        const cudaMemcpyKind k = r.csr.on_device ? cudaMemcpyDefault : cudaMemcpyHostToDevice;
+        step(cudaMemcpyAsync(c, r.csr.col_idx + e0, 4 * cnt, k, s));
+        if (values) step(cudaMemcpyAsync(v, r.csr.val + e0, 8 * cnt, k, s));
       };
       const bool single = e == cudaSuccess && run_end(0) == group;
       for (int c0 = 0, c1; e == cudaSuccess && c0 < group; c0 = c1) {
@@ -631,7 +636,7 @@ void admit(cg_batch_ctx* b) {
       }
     }
     j->d_x = d.at<double>(L.x);
-    staged.push_back({j, L, std::move(rp), std::move(part), e});
+    staged.push_back({j, L, std::move(rp), std::move(part), in_place, e});
   }
   if (staged.empty()) return;
   cudaError_t es = cudaMemcpyAsync(b->h_scan, b->d_scan, sizeof(cgk::LayoutScan) * b->max_systems,
@@ -646,7 +651,7 @@ void admit(cg_batch_ctx* b) {
     };
     const Dev d{b->d_arena + st.j->off, st.L};
     const cg_request& r = st.j->req;
-    if (r.csr.on_device) {
+    if (st.in_place) {
       const cgk::CsrSource src{d.at<int32_t>(st.L.r), r.csr.col_idx, r.csr.val, 0, r.csr.index_base};
       step(place(d, st.rp, st.part, slot));
       if (st.e == cudaSuccess) step(fill(d, src, slot, 0, b->h_sys[slot].A.nsteps, 0, r.n));

@@ -560,11 +560,11 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   } while (0)
 
   if (csr->on_device) {
-    CG_TRY(cudaMemcpy(rp.data(), csr->row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost),
+    CG_TRY(cudaMemcpy(rp.data(), csr->row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyDefault),
            "cg_create: copy of row_ptr");
     if (need_cols_on_host && nnz > 0) {
       ci.resize(static_cast<size_t>(nnz));
-      CG_TRY(cudaMemcpy(ci.data(), csr->col_idx, sizeof(int32_t) * nnz, cudaMemcpyDeviceToHost),
+      CG_TRY(cudaMemcpy(ci.data(), csr->col_idx, sizeof(int32_t) * nnz, cudaMemcpyDefault),
              "cg_create: copy of col_idx");
     }
   }
@@ -686,11 +686,14 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   int32_t* d_rp = h->d_csr_row_ptr;
   int32_t* d_ci = h->d_csr_col;
   double* d_va = h->d_csr_val;
-  const bool callers_rp = !keep_csr && csr->on_device && base == 0;  // (the caller's row pointers serve as they are)
+  const bool in_place = csr->on_device && cgh::readable_in_place(csr->row_ptr, h->device) &&
+                        (nnz == 0 || (cgh::readable_in_place(csr->col_idx, h->device) &&
+                                      cgh::readable_in_place(csr->val, h->device)));
+  const bool callers_rp = !keep_csr && in_place && base == 0;  // (the caller's row pointers serve as they are)
   if (!keep_csr && !callers_rp) {
     Block tmp;
     tmp.add(&d_rp, nn + 1);
-    if (!csr->on_device) {
+    if (!in_place) {
       tmp.add(&d_ci, nz);
       tmp.add(&d_va, nz);
     }
@@ -705,11 +708,10 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   src.base = base;
   if (d_ci != nullptr && nnz > 0) {
     if (csr->on_device && base == 0)
-      CG_TRY(cudaMemcpy(d_ci, csr->col_idx, sizeof(int32_t) * nz, cudaMemcpyDeviceToDevice), "cg_create: copy");
+      CG_TRY(cudaMemcpy(d_ci, csr->col_idx, sizeof(int32_t) * nz, cudaMemcpyDefault), "cg_create: copy");
     else
       CG_TRY(cudaMemcpy(d_ci, ci.data(), sizeof(int32_t) * nz, cudaMemcpyHostToDevice), "cg_create: upload");
-    CG_TRY(cudaMemcpy(d_va, csr->val, sizeof(double) * nz,
-                      csr->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
+    CG_TRY(cudaMemcpy(d_va, csr->val, sizeof(double) * nz, csr->on_device ? cudaMemcpyDefault : cudaMemcpyHostToDevice),
            "cg_create: upload");
     src.col_idx = d_ci;
     src.val = d_va;

@@ -49,4 +49,15 @@ void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, boo
 void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool mixed, Partition& P);
 // Upper bounds of stream_units and entries for either column width.
 void stream_bound(int64_t nnz, bool mixed, const Partition& P, int64_t* stream_units, int64_t* entries);
+
+// Whether kernels on `device` may read p in place: its own or managed memory.
+// Another GPU's memory can be copied, but not always read by a kernel.
+inline bool readable_in_place(const void* p, int device) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+}
 }  // namespace cgh

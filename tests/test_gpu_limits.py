@@ -82,3 +82,44 @@ def test_wait_limit_is_no_limit_on_a_pass():
     with cg.cg_create(rp, ci, va, precision=mixed, ctas=1, wait_limit_ms=1) as h:
         r = cg.cg_solve(h, b, torch.zeros_like(b), tol=TOL, maxit=1)
     assert r.status == cg.CG_ENOTCONV, r
+
+
+@pytest.mark.parametrize("base", [0, 1])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_device_arrays_that_are_not_this_gpus(precision, base):
+    """Arrays declared to be on the device that are not this GPU's own memory
+    (here pinned host memory; another GPU's is another case) are copied, not read
+    in place: the bits of the same arrays on this GPU, from a handle and a batch,
+    in several runs through the batch's staging buffer."""
+    import ctypes
+    import torch
+    from paper_2112_10823_gb300 import _binding as bd
+    cg = cg_mod()
+    A, b = _system(60, 83)
+    assert A.nnz > (4 << 20)
+    ref = np.zeros(A.n)
+    with handle(A, precision=precision) as h:
+        cg.cg_solve(h, b, ref, tol=TOL)
+    rp, ci, va = (torch.from_numpy(a).pin_memory() for a in (A.row_ptr + np.int32(base), A.col_idx + np.int32(base), A.val))
+    csr = bd.cg_csr(rp.data_ptr(), ci.data_ptr(), va.data_ptr(), base, 1)
+    o = bd.cg_opts()
+    bd.lib.cg_opts_default(ctypes.byref(o))
+    o.precision = precision
+    out = ctypes.c_void_p(0)
+    assert bd.lib.cg_create(ctypes.byref(out), ctypes.byref(csr), A.n, A.nnz, ctypes.byref(o)) == cg.CG_OK
+    x = np.zeros(A.n)
+    it, rr = ctypes.c_int64(0), ctypes.c_double(0)
+    assert bd.lib.cg_solve(out, b.ctypes.data, x.ctypes.data, TOL, 10 * A.n, ctypes.byref(it), ctypes.byref(rr)) == cg.CG_OK
+    bd.lib.cg_destroy(out)
+    assert np.array_equal(x, ref)
+    xs = [np.zeros(A.n), np.zeros(A.n)]
+    with cg.Batch(precision=precision, group_override=8) as bt:
+        r = bt.wait(bt.submit([cg.Request(A.row_ptr, A.col_idx, A.val, b, xs[0], tol=TOL)])[0])
+        req = bd.cg_request()
+        req.csr, req.n, req.nnz = csr, A.n, A.nnz
+        req.b, req.x, req.tol, req.maxit = b.ctypes.data, xs[1].ctypes.data, TOL, 10 * A.n
+        t = ctypes.c_uint64(0)
+        assert bd.lib.cg_batch_submit(bt._b, ctypes.byref(req), 1, ctypes.byref(t)) == cg.CG_OK
+        r2 = bt.wait(t.value)
+    assert r.status == r2.status == cg.CG_OK and r.iters == r2.iters
+    assert np.array_equal(xs[0], xs[1])
