@@ -329,7 +329,10 @@ typedef struct {
   int32_t device;          /* CUDA device ordinal; -1 = the current device */
   int32_t precision;       /* cg_precision of every system of the batch */
   int64_t budget_bytes;    /* device memory for resident systems (matrices, vectors,
-                              partition tables); 0 = half of the free memory at creation */
+                              partition tables); 0 = half of the free memory at creation.
+                              Beside it, for requests with host arrays: a staging buffer of
+                              48 MB (less where memory is short; 12 bytes per entry of the
+                              longest row if that is more) */
   int32_t max_systems;     /* resident systems at most (default 1024) */
   int32_t chunk_iters;     /* steps per system per round; 0 = until the system ends */
   int32_t replace_every;   /* CG_PREC_MIXED residual-replacement period (default 50) */

@@ -386,8 +386,9 @@ struct Dev {
 };
 
 // Device buffer for the columns and values of at least `least` entries of a
-// request's arrays that are not on this device: kStageEntries, or what one CTA's share needs if that is
-// more; half as much, and so on, where memory is short.
+// request's arrays that are not on this device: kStageEntries (48 MB), or half as
+// much, and so on, where memory is short; more only for a step (a row) that needs
+// more.
 constexpr int64_t kStageEntries = int64_t(4) << 20;
 cudaError_t reserve_stage(cg_batch_ctx* b, int64_t least) {
   if (b->stage_entries >= least && b->d_stage != nullptr) return cudaSuccess;
@@ -452,15 +453,18 @@ void admit(cg_batch_ctx* b) {
     std::memcpy(q, src, bytes);
     return cudaMemcpyAsync(dst, q, bytes, cudaMemcpyHostToDevice, s);
   };
-  // of a system's steps [k0, k1) or rows [r0, r1), whose entries src holds
-  auto scan = [&](const Dev& d, const cgk::CsrSource& src, int slot, int32_t k0, int32_t k1, int64_t n) {
-    return cgk::launch_layout_scan(src, d.at<int4>(d.L.step), d.at<uint8_t>(d.L.len), nullptr, k0, k1, n, b->validate, b->d_scan + slot, s);
+  // of the rows [r0, r1) of a system, whose entries src holds and whose steps are
+  // among [k0, k1)
+  auto scan = [&](const Dev& d, const cgk::CsrSource& src, int slot, int32_t k0, int32_t k1, int32_t r0, int32_t r1,
+                  int64_t n) {
+    return cgk::launch_layout_scan(src, d.at<int4>(d.L.step), d.at<uint8_t>(d.L.len), nullptr, k0, k1, r0, r1, n,
+                                   b->validate, b->d_scan + slot, s);
   };
-  auto fill = [&](const Dev& d, const cgk::CsrSource& src, int slot, int32_t k0, int32_t k1, int64_t r0, int64_t r1) {
+  auto fill = [&](const Dev& d, const cgk::CsrSource& src, int slot, int32_t k0, int32_t k1, int32_t r0, int32_t r1) {
     const cgk::DevCsr& A = b->h_sys[slot].A;
     const cgk::StreamPlace to{A.chunk_off, d.at<uint32_t>(d.L.q), d.at<uint32_t>(d.L.q) + A.nsteps,
                               d.at<unsigned char>(d.L.stream), b->mixed ? d.at<double>(d.L.val64) : nullptr};
-    cudaError_t e = cgk::launch_layout_fill(src, A.step, to, k0, k1, A.col16 != 0, b->mixed, s);
+    cudaError_t e = cgk::launch_layout_fill(src, A.step, to, k0, k1, r0, r1, A.col16 != 0, b->mixed, s);
     if (e == cudaSuccess && b->jacobi)
       e = cgk::launch_jacobi_dinv(src, r0, r1, d.at<double>(d.L.dinv), b->d_admit_err + slot, s);
     return e;
@@ -593,23 +597,25 @@ void admit(cg_batch_ctx* b) {
     const bool in_place = r.csr.on_device && (nnz == 0 || (cgh::readable_in_place(r.csr.col_idx, b->device) &&
                                                            cgh::readable_in_place(r.csr.val, b->device)));
     if (e == cudaSuccess && in_place) {
-      step(scan(d, src, slot, 0, nsteps, n));
+      step(scan(d, src, slot, 0, nsteps, 0, static_cast<int32_t>(n), n));
     } else if (e == cudaSuccess) {
-      // arrays elsewhere: in runs of CTA shares (consecutive rows) that fit the staging
+      // arrays elsewhere: in runs of steps (consecutive rows) that fit the staging
       // buffer, scanned, read back, and uploaded again to be filled (once, if a
       // single run holds them all)
-      auto first_entry = [&](int c) -> int64_t { return rp[part.block_row[c]]; };
-      auto first_step = [&](int c) { return part.warp_step[static_cast<size_t>(c) * cgk::kWarps]; };
+      std::vector<int32_t> cut;  // the rows at which steps begin
+      cut.reserve(static_cast<size_t>(nsteps) + 1);
+      for (const int4& t : part.step) cut.push_back(t.x);  // (the sentinel's: n)
+      std::sort(cut.begin(), cut.end());
       int64_t most = 1;
-      for (int c = 0; c < group; ++c) most = std::max(most, first_entry(c + 1) - first_entry(c));
+      for (int k = 0; k < nsteps; ++k) most = std::max<int64_t>(most, rp[cut[k + 1]] - rp[cut[k]]);
       step(reserve_stage(b, most));
-      auto run_end = [&](int c0) {
-        int c1 = c0 + 1;
-        while (c1 < group && first_entry(c1 + 1) - first_entry(c0) <= b->stage_entries) ++c1;
-        return c1;
+      auto run_end = [&](int k0) {
+        int k1 = k0 + 1;
+        while (k1 < nsteps && rp[cut[k1 + 1]] - rp[cut[k0]] <= b->stage_entries) ++k1;
+        return k1;
       };
-      auto stage = [&](int c0, int c1, bool values) {
-        const int64_t e0 = first_entry(c0), cnt = first_entry(c1) - e0;
+      auto stage = [&](int32_t r0, int32_t r1, bool values) {
+        const int64_t e0 = rp[r0], cnt = rp[r1] - e0;
         double* const v = reinterpret_cast<double*>(b->d_stage);
         int32_t* const c = reinterpret_cast<int32_t*>(v + b->stage_entries);
         src.e_first = e0;
@@ -620,19 +626,27 @@ void admit(cg_batch_ctx* b) {
         step(cudaMemcpyAsync(c, r.csr.col_idx + e0, 4 * cnt, k, s));
         if (values) step(cudaMemcpyAsync(v, r.csr.val + e0, 8 * cnt, k, s));
       };
-      const bool single = e == cudaSuccess && run_end(0) == group;
-      for (int c0 = 0, c1; e == cudaSuccess && c0 < group; c0 = c1) {
-        c1 = run_end(c0);
-        stage(c0, c1, single);
-        step(scan(d, src, slot, first_step(c0), first_step(c1), n));
+      // the steps of the CTAs that hold rows [r0, r1)
+      auto first_step = [&](int32_t row, bool end) {
+        const auto& br = part.block_row;
+        const size_t c = static_cast<size_t>(std::upper_bound(br.begin(), br.end() - 1, row) - br.begin()) - (end ? 0 : 1);
+        return part.warp_step[c * cgk::kWarps];
+      };
+      const bool single = e == cudaSuccess && run_end(0) == nsteps;
+      for (int k0 = 0, k1; e == cudaSuccess && k0 < nsteps; k0 = k1) {
+        k1 = run_end(k0);
+        const int32_t r0 = cut[k0], r1 = cut[k1];
+        stage(r0, r1, single);
+        step(scan(d, src, slot, first_step(r0, false), first_step(r1 - 1, true), r0, r1, n));
       }
       step(cudaMemcpyAsync(b->h_scan + slot, b->d_scan + slot, sizeof(cgk::LayoutScan), cudaMemcpyDeviceToHost, s));
       step(cudaStreamSynchronize(s));
       if (e == cudaSuccess && b->h_scan[slot].bad_entry == 0) step(place(d, rp, part, slot));
-      for (int c0 = 0, c1; e == cudaSuccess && c0 < group && b->h_scan[slot].bad_entry == 0; c0 = c1) {
-        c1 = run_end(c0);
-        if (!single) stage(c0, c1, true);
-        step(fill(d, src, slot, first_step(c0), first_step(c1), part.block_row[c0], part.block_row[c1]));
+      for (int k0 = 0, k1; e == cudaSuccess && k0 < nsteps && b->h_scan[slot].bad_entry == 0; k0 = k1) {
+        k1 = run_end(k0);
+        const int32_t r0 = cut[k0], r1 = cut[k1];
+        if (!single) stage(r0, r1, true);
+        step(fill(d, src, slot, first_step(r0, false), first_step(r1 - 1, true), r0, r1));
       }
     }
     j->d_x = d.at<double>(L.x);
@@ -654,7 +668,7 @@ void admit(cg_batch_ctx* b) {
     if (st.in_place) {
       const cgk::CsrSource src{d.at<int32_t>(st.L.r), r.csr.col_idx, r.csr.val, 0, r.csr.index_base};
       step(place(d, st.rp, st.part, slot));
-      if (st.e == cudaSuccess) step(fill(d, src, slot, 0, b->h_sys[slot].A.nsteps, 0, r.n));
+      if (st.e == cudaSuccess) step(fill(d, src, slot, 0, b->h_sys[slot].A.nsteps, 0, static_cast<int32_t>(r.n)));
     }
     if (b->jacobi)
       step(cudaMemcpyAsync(b->h_admit_err + slot, b->d_admit_err + slot, sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -723,7 +723,8 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   uint32_t* const d_step_chunk = reinterpret_cast<uint32_t*>(h->d_q);
   uint32_t* const d_step_entry = d_step_chunk + h->nsteps;
   cgk::LayoutScan* const d_scan = reinterpret_cast<cgk::LayoutScan*>(h->d_err + 4);
-  CG_TRY(cgk::launch_layout_scan(src, h->d_step, h->d_seg_len, h->d_step_cmax, 0, h->nsteps, n, false, d_scan, nullptr),
+  CG_TRY(cgk::launch_layout_scan(src, h->d_step, h->d_seg_len, h->d_step_cmax, 0, h->nsteps, 0, static_cast<int32_t>(n), n,
+                                 false, d_scan, nullptr),
          "cg_create: column scan");
   if (o.preconditioner == CG_PRECOND_JACOBI)
     CG_TRY(cgk::launch_jacobi_dinv(src, 0, n, h->d_dinv, h->d_err, nullptr),
@@ -759,7 +760,7 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   CG_TRY(up(d_step_chunk, part.step_chunk, static_cast<size_t>(h->nsteps)), "cg_create: upload");
   if (mixed) CG_TRY(up(d_step_entry, part.step_entry, static_cast<size_t>(h->nsteps)), "cg_create: upload");
   const cgk::StreamPlace to{h->d_chunk_off, d_step_chunk, d_step_entry, h->d_stream, h->d_val64};
-  CG_TRY(cgk::launch_layout_fill(src, h->d_step, to, 0, h->nsteps, h->col16, mixed, nullptr),
+  CG_TRY(cgk::launch_layout_fill(src, h->d_step, to, 0, h->nsteps, 0, static_cast<int32_t>(n), h->col16, mixed, nullptr),
          "cg_create: stream order");
   CG_TRY(cudaDeviceSynchronize(), "cg_create: synchronize");
 #undef CG_TRY

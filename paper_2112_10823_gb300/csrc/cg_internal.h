@@ -230,12 +230,12 @@ struct LayoutScan {
   int32_t pad;
   unsigned long long bad_entry;  // ~entry (so that a maximum finds the first), 0: none
 };
-// For steps [s0, s1): the lanes' segment lengths into seg_len[], the smallest
+// For the steps among [s0, s1) that begin in rows [row0, row1): the lanes' segment lengths into seg_len[], the smallest
 // column into step[].w (0 for a step without entries), the largest into cmax[]
 // (if not nullptr; -1 without entries), span and bad entries into *out.
-cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1, int64_t n,
-                               bool check, LayoutScan* out, cudaStream_t s);
-// Writes the entries of steps [s0, s1) in stream order: into `stream` the
+cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1,
+                               int32_t row0, int32_t row1, int64_t n, bool check, LayoutScan* out, cudaStream_t s);
+// Writes the entries of the same steps in stream order: into `stream` the
 // chunks step_chunk[k].. of step k, at the units that chunk_off gives (16-bit
 // column offsets if col16, else 32-bit columns; FP32 values, rounded to nearest,
 // if mixed), and if mixed the FP64 values from val64[step_entry[k]] on.
@@ -248,7 +248,7 @@ struct StreamPlace {
   double* val64;               // mixed
 };
 cudaError_t launch_layout_fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
-                               bool col16, bool mixed, cudaStream_t s);
+                               int32_t row0, int32_t row1, bool col16, bool mixed, cudaStream_t s);
 // dinv[i] = 1 / (sum of row i's stored entries in column i) for rows [row0, row1);
 // err set to the first row (+1) found whose diagonal is not positive.
 cudaError_t launch_jacobi_dinv(const CsrSource& src, int64_t row0, int64_t row1, double* dinv, int32_t* err,

@@ -21,13 +21,14 @@ __device__ __forceinline__ int step_rows(const int4& d) {
 }
 }  // namespace
 
-__global__ void __launch_bounds__(kLayoutBlock) layout_scan_kernel(const CsrSource src, int4* step, uint8_t* seg_len, int32_t* cmax,
-                                                                    int32_t s0, int32_t s1, int64_t n, int check,
-                                                                    LayoutScan* out) {
+__global__ void __launch_bounds__(kLayoutBlock)
+    layout_scan_kernel(const CsrSource src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1,
+                       int32_t row0, int32_t row1, int64_t n, int check, LayoutScan* out) {
   const int s = s0 + static_cast<int>((static_cast<int64_t>(blockIdx.x) * kLayoutBlock + threadIdx.x) >> 5);
   if (s >= s1) return;
   const int lane = threadIdx.x & 31;
   const int4 d = step[s];
+  if (d.x < row0 || d.x >= row1) return;
   const int64_t e0 = src.row_ptr[d.x], e1 = src.row_ptr[d.x + step_rows(d)];
   int lo = 0x7fffffff, hi = -1;
   unsigned long long bad = 0;
@@ -64,12 +65,13 @@ __global__ void __launch_bounds__(kLayoutBlock) layout_scan_kernel(const CsrSour
 template <typename T, typename C>
 __global__ void __launch_bounds__(kLayoutBlock)
     layout_fill_kernel(const CsrSource src, const int4* __restrict__ step, const StreamPlace to, int32_t s0,
-                       int32_t s1) {
+                       int32_t s1, int32_t row0, int32_t row1) {
   const int s = s0 + static_cast<int>((static_cast<int64_t>(blockIdx.x) * kLayoutBlock + threadIdx.x) >> 5);
   if (s >= s1) return;
   const int lane = threadIdx.x & 31;
   const unsigned int below = (1u << lane) - 1u;
   const int4 d = step[s];
+  if (d.x < row0 || d.x >= row1) return;
   const int mode = step_mode(d);
   // this lane's segment in CSR order: entries a, a + stride, ...
   int64_t a = 0;
@@ -123,23 +125,20 @@ __global__ void __launch_bounds__(kLayoutBlock)
   }
 }
 
-cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1, int64_t n,
-                               bool check, LayoutScan* out, cudaStream_t s) {
+cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_len, int32_t* cmax, int32_t s0, int32_t s1,
+                               int32_t row0, int32_t row1, int64_t n, bool check, LayoutScan* out, cudaStream_t s) {
   if (s1 <= s0) return cudaSuccess;
-  layout_scan_kernel<<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, seg_len, cmax, s0, s1, n, check ? 1 : 0, out);
+  layout_scan_kernel<<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, seg_len, cmax, s0, s1, row0, row1, n,
+                                                                 check ? 1 : 0, out);
   return cudaGetLastError();
 }
 
-template <typename T, typename C>
-static void fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1, cudaStream_t s) {
-  layout_fill_kernel<T, C><<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, to, s0, s1);
-}
-
 cudaError_t launch_layout_fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
-                               bool col16, bool mixed, cudaStream_t s) {
+                               int32_t row0, int32_t row1, bool col16, bool mixed, cudaStream_t s) {
   if (s1 <= s0) return cudaSuccess;
-  if (mixed) col16 ? fill<float, uint16_t>(src, step, to, s0, s1, s) : fill<float, int32_t>(src, step, to, s0, s1, s);
-  else col16 ? fill<double, uint16_t>(src, step, to, s0, s1, s) : fill<double, int32_t>(src, step, to, s0, s1, s);
+  auto fill = [&](auto kernel) { kernel<<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, to, s0, s1, row0, row1); };
+  if (mixed) col16 ? fill(layout_fill_kernel<float, uint16_t>) : fill(layout_fill_kernel<float, int32_t>);
+  else col16 ? fill(layout_fill_kernel<double, uint16_t>) : fill(layout_fill_kernel<double, int32_t>);
   return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
 """Calls at their limits, on the GPU: the step limit at the step that converges,
-a wait limit shorter than a pass over the matrix."""
+a wait limit shorter than a pass over the matrix, a budget near the card's memory."""
 import numpy as np
 import pytest
 
@@ -123,3 +123,24 @@ def test_device_arrays_that_are_not_this_gpus(precision, base):
         r2 = bt.wait(t.value)
     assert r.status == r2.status == cg.CG_OK and r.iters == r2.iters
     assert np.array_equal(xs[0], xs[1])
+
+
+def test_host_arrays_beside_a_budget_near_the_cards_memory():
+    """With 200 MB left beside the budget, a one-CTA request with host arrays of
+    more than that is admitted as before, through a small staging buffer, with the
+    bits of device arrays."""
+    import torch
+    cg = cg_mod()
+    A = fi.q1(100, 1.0, 84)
+    assert 12 * A.nnz > (250 << 20)
+    b = np.ones(A.n)
+    dev = [torch.from_numpy(a).cuda() for a in (A.row_ptr, A.col_idx, A.val, b, np.zeros(A.n))]
+    x = np.zeros(A.n)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    with cg.Batch(group_override=1, budget_bytes=free - (200 << 20)) as bt:
+        rd = bt.wait(bt.submit([cg.Request(*dev, tol=TOL, maxit=3)])[0], 60000)
+        rh = bt.wait(bt.submit([cg.Request(A.row_ptr, A.col_idx, A.val, b, x, tol=TOL, maxit=3)])[0], 60000)
+    assert rd.status == rh.status == cg.CG_ENOTCONV, (rd, rh)
+    assert np.array_equal(x, dev[4].cpu().numpy())
