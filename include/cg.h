@@ -330,7 +330,9 @@ typedef struct {
   int32_t precision;       /* cg_precision of every system of the batch */
   int64_t budget_bytes;    /* device memory for resident systems (matrices, vectors,
                               partition tables); 0 = half of the free memory at creation.
-                              Beside it, for requests with host arrays: a staging buffer of
+                              Beside it: the tables of a system that submit accepts but
+                              that needs a little more than the budget (long rows, many
+                              CTAs), and for requests with host arrays a staging buffer of
                               48 MB (less where memory is short; 12 bytes per entry of the
                               longest row if that is more) */
   int32_t max_systems;     /* resident systems at most (default 1024) */

@@ -132,10 +132,12 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Upper bound of a system's device footprint (before its partition is known:
-// at most one step per row).
+// What a request has to fit the budget by: its matrix (12 bytes per entry, 16 in
+// mixed precision), its vectors and 24 bytes per row.  A system's own layout is
+// usually smaller; where it is not (long rows, whose steps are a row each; many
+// CTAs), what lies beyond the budget is allocated for that request alone.
 constexpr int64_t kPadEntries = 8;
-size_t footprint_bound(int64_t n, int64_t nnz, bool mixed, bool jacobi, int nblocks) {
+size_t footprint(int64_t n, int64_t nnz, bool mixed, bool jacobi, int nblocks) {
   const size_t pad = kPadEntries;
   size_t b = 0;
   b += align_up(4 * (n + 1));
@@ -157,6 +159,7 @@ struct Job {
   JobState state = kQueued;
   int slot = -1;
   size_t off = 0, bytes = 0;   // arena block
+  char* d_extra = nullptr;     // what of the layout lies beyond the arena's size
   int group = 1;
   double* d_x = nullptr;
   double bytes_step = 0.0;
@@ -338,33 +341,29 @@ bool load_structure(const cg_request& r, bool validate, std::vector<int32_t>& rp
   return true;
 }
 
-// A job's device layout inside its arena block: room for the matrix in either
-// column width.  Until the solve starts, r holds the row pointers and q the
-// steps' places in the streams (8 bytes per row at most).
+// A job's device layout: room for the matrix in either column width.  Until the
+// solve starts, r holds the row pointers and q the steps' places in the streams
+// (8 bytes per row at most).  Offsets from `cap` (the arena's size) on lie in the
+// job's extra block; no array lies across.
 struct Layout {
   size_t len, stream, val64, step, coff, wchunk, wentry, wstep, brow, b, x, r, p, q, p32, dinv, part, total;
 };
 
-Layout layout_of(int64_t n, int64_t nnz, const cgh::Partition& part, int group, bool mixed, bool jacobi) {
+Layout layout_of(int64_t n, int64_t nnz, const cgh::Partition& part, int group, bool mixed, bool jacobi, size_t cap) {
   int64_t stream_units = 0, entries = 0;
   cgh::stream_bound(nnz, mixed, part, &stream_units, &entries);
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) {
+    bytes = align_up(bytes);
+    if (o < cap && o + bytes > cap) o = cap;
     const size_t at = o;
-    o += align_up(bytes);
+    o += bytes;
     return at;
   };
   const size_t warps = static_cast<size_t>(group) * cgk::kWarps;
-  L.len = take(32 * part.step.size());
   L.stream = take(static_cast<size_t>(stream_units) * cgk::kUnit);
   L.val64 = mixed ? take(8 * static_cast<size_t>(entries)) : 0;
-  L.step = take(sizeof(int4) * part.step.size());
-  L.coff = take(4 * (static_cast<size_t>(part.chunks) + 1));
-  L.wchunk = take(sizeof(int4) * warps);
-  L.wentry = mixed ? take(4 * warps) : 0;
-  L.wstep = take(4 * (warps + 1));
-  L.brow = take(4 * (static_cast<size_t>(group) + 1));
   L.b = take(8 * n);
   L.x = take(8 * n);
   L.r = take(8 * n);
@@ -373,17 +372,33 @@ Layout layout_of(int64_t n, int64_t nnz, const cgh::Partition& part, int group, 
   L.p32 = mixed ? take(4 * n) : 0;
   L.dinv = jacobi ? take(8 * n) : 0;
   L.part = take(sizeof(double) * 6 * group);
+  L.len = take(32 * part.step.size());
+  L.step = take(sizeof(int4) * part.step.size());
+  L.coff = take(4 * (static_cast<size_t>(part.chunks) + 1));
+  L.wchunk = take(sizeof(int4) * warps);
+  L.wentry = mixed ? take(4 * warps) : 0;
+  L.wstep = take(4 * (warps + 1));
+  L.brow = take(4 * (static_cast<size_t>(group) + 1));
   L.total = o;
   return L;
 }
 
-// A system's arrays in its arena block.
+// A system's arrays in its arena block and, from `cap` on, in its extra one.
 struct Dev {
   char* base;
+  char* extra;
+  size_t cap;
   const Layout& L;
   template <typename T>
-  T* at(size_t o) const { return reinterpret_cast<T*>(base + o); }
+  T* at(size_t o) const { return reinterpret_cast<T*>(o < cap ? base + o : extra + (o - cap)); }
 };
+
+// The job's device memory is free again (b->mu held).
+void release_memory(cg_batch_ctx* b, Job* j) {
+  b->arena.release(j->off, j->bytes);
+  if (j->d_extra) cudaFree(j->d_extra);
+  j->d_extra = nullptr;
+}
 
 // Device buffer for the columns and values of at least `least` entries of a
 // request's arrays that are not on this device: kStageEntries (48 MB), or half as
@@ -515,37 +530,37 @@ void admit(cg_batch_ctx* b) {
     }
     cgh::Partition part;
     cgh::build_partition(rp, n, group, b->mixed, part, shape);
-    Layout L = layout_of(n, nnz, part, group, b->mixed, b->jacobi);
-    if (L.total > b->arena.cap()) {
+    const size_t cap = b->arena.cap();
+    Layout L = layout_of(n, nnz, part, group, b->mixed, b->jacobi, cap);
+    if (L.total > cap) {
       shape.tight = true;
       cgh::build_partition(rp, n, group, b->mixed, part, shape);
-      L = layout_of(n, nnz, part, group, b->mixed, b->jacobi);
+      L = layout_of(n, nnz, part, group, b->mixed, b->jacobi, cap);
     }
     const int32_t nsteps = static_cast<int32_t>(part.step.size()) - 1;
-    if (L.total > b->arena.cap()) {  // (a matrix of many short steps: submit's bound allows one table less)
-      std::lock_guard<std::mutex> lk(b->mu);
-      b->queued.pop_front();
-      finish_without_device(b, j, CG_ENOMEM);
-      b->err = "request " + std::to_string(j->ticket) + " needs more memory than the budget";
-      b->cv_done.notify_all();
-      continue;
-    }
+    const size_t bytes = std::min(L.total, cap);
     size_t off = 0;
     int slot = -1;
     {
       std::lock_guard<std::mutex> lk(b->mu);
-      if (!b->arena.alloc(L.total, off)) break;  // wait for memory (arrival order is kept)
+      if (!b->arena.alloc(bytes, off)) break;  // wait for memory (arrival order is kept)
       slot = b->free_slots.back();
       b->free_slots.pop_back();
       b->queued.pop_front();
     }
     j->slot = slot;
     j->off = off;
-    j->bytes = L.total;
+    j->bytes = bytes;
     j->group = group;
     j->bytes_step = bytes_per_step(n, nnz, b->mixed);
     j->steps_est = est_steps(b->model, n);
-    const Dev d{b->d_arena + off, L};
+    cudaError_t e = L.total > cap ? cudaMalloc(&j->d_extra, L.total - cap) : cudaSuccess;
+    if (e != cudaSuccess) {
+      j->d_extra = nullptr;
+      staged.push_back({j, L, std::move(rp), std::move(part), false, e});
+      continue;
+    }
+    const Dev d{b->d_arena + off, j->d_extra, cap, L};
     cgk::SolveParams& P = b->h_sys[slot];  // pinned; copied once the matrix has its place
     std::memset(&P, 0, sizeof(P));
     P.A.stream = d.at<unsigned char>(L.stream);
@@ -578,7 +593,6 @@ void admit(cg_batch_ctx* b) {
     P.group = group;
     P.chunk_iters = b->chunk_iters;
     P.dinv = b->jacobi ? d.at<double>(L.dinv) : nullptr;
-    cudaError_t e = cudaSuccess;
     auto step = [&](cudaError_t x) {
       if (e == cudaSuccess) e = x;
     };
@@ -663,7 +677,7 @@ void admit(cg_batch_ctx* b) {
     auto step = [&](cudaError_t x) {
       if (st.e == cudaSuccess) st.e = x;
     };
-    const Dev d{b->d_arena + st.j->off, st.L};
+    const Dev d{b->d_arena + st.j->off, st.j->d_extra, b->arena.cap(), st.L};
     const cg_request& r = st.j->req;
     if (st.in_place) {
       const cgk::CsrSource src{d.at<int32_t>(st.L.r), r.csr.col_idx, r.csr.val, 0, r.csr.index_base};
@@ -679,7 +693,7 @@ void admit(cg_batch_ctx* b) {
   // a request that cannot become resident: its memory and slot are free again
   auto give_up = [&](Job* j, int status, const std::string& why) {
     std::lock_guard<std::mutex> lk(b->mu);
-    b->arena.release(j->off, j->bytes);
+    release_memory(b, j);
     b->free_slots.push_back(j->slot);
     j->slot = -1;
     finish_without_device(b, j, status);
@@ -801,7 +815,7 @@ void retire(cg_batch_ctx* b, const std::vector<Job*>& in_round) {
     j->res.done = 1;
     j->res.done_ms = t;
     j->state = kFinished;
-    b->arena.release(j->off, j->bytes);
+    release_memory(b, j);
     b->free_slots.push_back(j->slot);
     j->slot = -1;
     ++b->completed;
@@ -833,7 +847,7 @@ void worker_main(cg_batch_ctx* b) {
         std::lock_guard<std::mutex> lk(b->mu);
         b->err = cuda_msg(e, "round launch");
         for (Job* j : in_round) {
-          b->arena.release(j->off, j->bytes);
+          release_memory(b, j);
           b->free_slots.push_back(j->slot);
           j->slot = -1;
           finish_without_device(b, j, CG_ECUDA);
@@ -877,6 +891,8 @@ void worker_main(cg_batch_ctx* b) {
 void release_all(cg_batch_ctx* b) {
   if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
   if (b->graph) cudaGraphDestroy(b->graph);
+  for (auto& j : b->jobs)
+    if (j.second->d_extra) cudaFree(j.second->d_extra);
   if (b->d_arena) cudaFree(b->d_arena);
   if (b->d_sys) cudaFree(b->d_sys);
   if (b->d_ctrl) cudaFree(b->d_ctrl);
@@ -938,10 +954,12 @@ void stencil27(int m, std::vector<int32_t>& rp, std::vector<int32_t>& ci, std::v
 double time_per_step(cg_batch_ctx* b, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                      const std::vector<double>& va, int copies, int group, int steps) {
   const int64_t n = static_cast<int64_t>(rp.size()) - 1, nnz = static_cast<int64_t>(ci.size());
-  if (copies <= 0 || static_cast<size_t>(copies) * footprint_bound(n, nnz, b->mixed, b->jacobi, b->nblocks) >
-                         b->arena.cap() ||
-      copies > b->max_systems)
-    return -1.0;
+  const size_t cap = b->arena.cap();
+  cgh::Partition part;
+  cgh::build_partition(rp, n, group, b->mixed, part, b->shape);
+  const size_t each = std::max(footprint(n, nnz, b->mixed, b->jacobi, b->nblocks),
+                               layout_of(n, nnz, part, group, b->mixed, b->jacobi, cap).total);
+  if (copies <= 0 || static_cast<size_t>(copies) * each > cap || copies > b->max_systems) return -1.0;
   std::vector<double> bv(static_cast<size_t>(n), 1.0);
   std::vector<std::vector<double>> xs(static_cast<size_t>(copies), std::vector<double>(static_cast<size_t>(n)));
   std::vector<cg_request> reqs(static_cast<size_t>(copies));
@@ -1262,7 +1280,7 @@ int cg_batch_submit(cg_batch b, const cg_request* reqs, int32_t count, uint64_t*
     std::string why;
     if (!request_ok(reqs[i], why))
       return bfail(b, CG_EINVAL, "cg_batch_submit: request " + std::to_string(i) + ": " + why);
-    const size_t need = footprint_bound(reqs[i].n, reqs[i].nnz, b->mixed, b->jacobi, b->nblocks);
+    const size_t need = footprint(reqs[i].n, reqs[i].nnz, b->mixed, b->jacobi, b->nblocks);
     if (need > b->arena.cap())
       return bfail(b, CG_ENOMEM, "cg_batch_submit: request " + std::to_string(i) + " needs up to " +
                                      std::to_string(need) + " bytes, more than the budget of " +

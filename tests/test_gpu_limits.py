@@ -1,5 +1,8 @@
 """Calls at their limits, on the GPU: the step limit at the step that converges,
-a wait limit shorter than a pass over the matrix, a budget near the card's memory."""
+a wait limit shorter than a pass over the matrix, the smallest budget that takes a
+request and one near the card's memory."""
+import re
+
 import numpy as np
 import pytest
 
@@ -123,6 +126,47 @@ def test_device_arrays_that_are_not_this_gpus(precision, base):
         r2 = bt.wait(t.value)
     assert r.status == r2.status == cg.CG_OK and r.iters == r2.iters
     assert np.array_equal(xs[0], xs[1])
+
+
+def _banded(n, length, seed):
+    """Symmetric, diagonally dominant; `length` (odd) entries in an inner row."""
+    import scipy.sparse as sp
+    rng = np.random.default_rng(seed)
+    h = length // 2
+    S = sp.diags([rng.uniform(-1, 0, n - d) for d in range(1, h + 1)], range(1, h + 1), shape=(n, n))
+    S = S + S.T
+    S = (S + sp.diags(np.asarray(abs(S).sum(axis=1)).ravel() + 1.0)).tocsr()
+    S.sort_indices()
+    return fi.CSR(S.indptr.astype(np.int32), S.indices.astype(np.int32), S.data.astype(np.float64), n)
+
+
+@pytest.mark.parametrize("host", [True, False])
+@pytest.mark.parametrize("precision,jacobi", [(0, 0), (1, 0), (1, 1)])
+@pytest.mark.parametrize("n,length,opts", [(20000, 65, {}), (5000, 97, {}), (300, 7, {"step_shape": 3}),
+                                           (20000, 3, {"step_shape": 3}), (500, 5, {"group_override": 1 << 20})])
+def test_smallest_accepted_budget_takes_the_request(n, length, opts, precision, jacobi, host):
+    """A budget of exactly the bytes that submit asks for takes a request whose
+    steps are single rows, or whose CTAs' tables outweigh the matrix; with the bits
+    of an ample budget."""
+    import torch
+    cg = cg_mod()
+    A = _banded(n, length, n)
+    b = oracle.spmv(A, fi.xstar(4, n))
+
+    def solved(budget):
+        arrays = [A.row_ptr, A.col_idx, A.val, b, np.zeros(n)]
+        if not host:
+            arrays = [torch.from_numpy(a).cuda() for a in arrays]
+        with cg.Batch(precision=precision, preconditioner=jacobi, budget_bytes=budget, **opts) as bt:
+            r = bt.wait(bt.submit([cg.Request(*arrays, tol=TOL)])[0], 60000)
+            assert bt.stats()["bytes_in_use"] == 0
+        assert r.done and r.status == cg.CG_OK, r
+        return arrays[4] if host else arrays[4].cpu().numpy()
+
+    with pytest.raises(cg.CGError) as refused:
+        solved(4096)
+    need = int(re.search(r"needs up to (\d+) bytes", str(refused.value)).group(1))
+    assert np.array_equal(solved(need), solved(1 << 30))
 
 
 def test_host_arrays_beside_a_budget_near_the_cards_memory():
