@@ -25,9 +25,10 @@ constexpr int kCtasPerSm = 1;
 // of a CTA goes to computing warp k modulo their number.
 //
 // The handle stores the matrix as one stream per warp: the entries of the
-// warp's steps in the order in which the warp consumes them.  Within a step
-// that is entry u of every lane's segment, in lane order, then entry u + 1, and
-// so on: one shared-memory read per entry and warp, free of bank conflicts.
+// warp's steps in the order in which the warp consumes them.  Within a chunk
+// (below) that is entry u of every lane's segment, in lane order, then entry
+// u + 1, and so on, free of bank conflicts in shared memory; or, where the lanes'
+// segments differ in length and are not padded, lane after lane.
 // A warp works through a step in chunks of a few entries per lane;
 // a chunk is one slot of the warp's ring, so that the ring gives back its
 // oldest bytes after every few entries and not only after a whole step.
@@ -80,10 +81,10 @@ constexpr int64_t kColSpan16 = 65535;
 // With 16-bit columns, a step whose lanes differ in length, or that fills only
 // some lanes, is padded to the longest segment in all 32 lanes where that adds
 // at most half (`tight`, where memory is short: an eighth): an entry's place is
-// then a constant offset.  Other steps hold their entries only, placed by
-// counting the lanes before them, with two votes per entry.  Padding is never
-// multiplied.  (At most an eighth, a quarter, a half, all of it: product of the
-// 110^3 mesh 95, 88, 84, 83 us; step of Q1 64^3 mixed 21.0, 20.9, 19.6, 19.6 us.)
+// then a constant offset.  Other steps hold their entries only (chunk_place).
+// Padding is never multiplied.  (At most an eighth, a quarter, a half, all of it,
+// when the other steps still cost two votes per entry: product of the 110^3 mesh
+// 95, 88, 84, 83 us; step of Q1 64^3 mixed 21.0, 20.9, 19.6, 19.6 us.)
 constexpr bool step_pads(int64_t longest, int64_t entries, bool tight) {
   return tight ? 8 * 32 * longest <= 9 * entries : 2 * 32 * longest <= 3 * entries;
 }

@@ -69,7 +69,6 @@ __global__ void __launch_bounds__(kLayoutBlock)
   const int s = s0 + static_cast<int>((static_cast<int64_t>(blockIdx.x) * kLayoutBlock + threadIdx.x) >> 5);
   if (s >= s1) return;
   const int lane = threadIdx.x & 31;
-  const unsigned int below = (1u << lane) - 1u;
   const int4 d = step[s];
   if (d.x < row0 || d.x >= row1) return;
   const int mode = step_mode(d);
@@ -104,24 +103,20 @@ __global__ void __launch_bounds__(kLayoutBlock)
   for (int u0 = 0; u0 < d.z; u0 += size, ++chunk) {
     const int cnt = min(size, d.z - u0);
     const int mine = padded ? cnt : max(0, min(len - u0, cnt));
-    const int tot = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(mine)));
+    const ChunkPlace place = chunk_place<C>(d, u0, cnt, len, lane);
     unsigned char* const at = to.stream + static_cast<size_t>(to.chunk_off[chunk]) * kUnit;
     C* const col = reinterpret_cast<C*>(at);
-    T* const val = reinterpret_cast<T*>(at + units(static_cast<int64_t>(tot) * sizeof(C)) * kUnit);
-    int pos = 0;
-    for (int k = 0; k < cnt; ++k, a += stride) {
-      const unsigned int m = __ballot_sync(0xffffffffu, k < mine);
+    T* const val = reinterpret_cast<T*>(at + units(static_cast<int64_t>(place.tot) * sizeof(C)) * kUnit);
+    for (int k = 0, dst = place.base; k < cnt; ++k, a += stride, dst += place.stride) {
       if (k < mine) {
         const bool real = u0 + k < len;
-        const int dst = pos + __popc(m & below);
         const double v = real ? src.val[a] : 0.0;
         col[dst] = real ? static_cast<C>(src.col_idx[a] - base) : C(0);
         val[dst] = static_cast<T>(v);  // (round to nearest)
         if (sizeof(T) == 4) to.val64[entry + dst] = v;
       }
-      pos += __popc(m);
     }
-    entry += tot;
+    entry += place.tot;
   }
 }
 
