@@ -249,6 +249,8 @@ struct cg_ctx {
   uint32_t* d_chunk_off = nullptr;
   int4* d_warp_chunk = nullptr;
   uint32_t* d_warp_entry = nullptr;
+  uint32_t* d_step_chunk = nullptr;  // mixed precision
+  uint32_t* d_step_entry = nullptr;
   int32_t* d_warp_step = nullptr;
   int32_t* d_block_row = nullptr;
   // the CSR arrays (0-based), kept for the cluster kernel only
@@ -346,6 +348,8 @@ cgk::DevCsr dev_view(const cg_ctx* h) {
   A.chunk_off = h->d_chunk_off;
   A.warp_chunk = h->d_warp_chunk;
   A.warp_entry = h->d_warp_entry;
+  A.step_chunk = h->d_step_chunk;
+  A.step_entry = h->d_step_entry;
   A.warp_step = h->d_warp_step;
   A.block_row = h->d_block_row;
   A.n = static_cast<int32_t>(h->n);
@@ -717,11 +721,6 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
     src.val = d_va;
     src.base = 0;  // ci is rebased
   }
-  // d_q holds the steps' places in the streams until the handle's first solve
-  // (a step has at least one row: two words of 4 bytes in its 8)
-  static_assert(sizeof(double) >= 2 * sizeof(uint32_t), "step_chunk and step_entry fit q");
-  uint32_t* const d_step_chunk = reinterpret_cast<uint32_t*>(h->d_q);
-  uint32_t* const d_step_entry = d_step_chunk + h->nsteps;
   cgk::LayoutScan* const d_scan = reinterpret_cast<cgk::LayoutScan*>(h->d_err + 4);
   CG_TRY(cgk::launch_layout_scan(src, h->d_step, h->d_seg_len, h->d_step_cmax, 0, h->nsteps, 0, static_cast<int32_t>(n), n,
                                  false, d_scan, nullptr),
@@ -746,6 +745,8 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   const size_t at_wchunk = str.add(&h->d_warp_chunk, part.warp_chunk.size());  // (one upload again)
   const size_t at_wentry = str.add(&h->d_warp_entry, part.warp_entry.size());
   const size_t at_coff = str.add(&h->d_chunk_off, part.chunk_off.size());
+  const size_t steps = mixed ? static_cast<size_t>(h->nsteps) : 0;
+  const size_t at_schunk = str.add(&h->d_step_chunk, steps), at_sentry = str.add(&h->d_step_entry, steps);
   tables.assign(str.bytes, 0);
   str.add(&h->d_stream, static_cast<size_t>(part.stream_units) * cgk::kUnit);
   if (mixed) str.add(&h->d_val64, static_cast<size_t>(part.entries));
@@ -753,13 +754,20 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   std::memcpy(tables.data() + at_wchunk, part.warp_chunk.data(), sizeof(int4) * part.warp_chunk.size());
   if (mixed) std::memcpy(tables.data() + at_wentry, part.warp_entry.data(), 4 * part.warp_entry.size());
   std::memcpy(tables.data() + at_coff, part.chunk_off.data(), 4 * part.chunk_off.size());
+  // in FP64 the steps' places in the streams serve the conversion only: q holds
+  // them until the handle's first solve (a step has at least one row)
+  static_assert(sizeof(double) >= sizeof(uint32_t), "step_chunk fits q");
+  uint32_t* d_step_chunk = reinterpret_cast<uint32_t*>(h->d_q);
+  if (mixed) {
+    d_step_chunk = h->d_step_chunk;
+    std::memcpy(tables.data() + at_schunk, part.step_chunk.data(), 4 * steps);
+    std::memcpy(tables.data() + at_sentry, part.step_entry.data(), 4 * steps);
+  } else if (h->nsteps > 0) {
+    CG_TRY(cudaMemcpy(d_step_chunk, part.step_chunk.data(), 4 * static_cast<size_t>(h->nsteps), cudaMemcpyHostToDevice),
+           "cg_create: upload");
+  }
   CG_TRY(cudaMemcpy(h->d_warp_chunk, tables.data(), tables.size(), cudaMemcpyHostToDevice), "cg_create: upload");
-  auto up = [&](void* dst, const auto& v, size_t count) {
-    return count ? cudaMemcpy(dst, v.data(), sizeof(v[0]) * count, cudaMemcpyHostToDevice) : cudaSuccess;
-  };
-  CG_TRY(up(d_step_chunk, part.step_chunk, static_cast<size_t>(h->nsteps)), "cg_create: upload");
-  if (mixed) CG_TRY(up(d_step_entry, part.step_entry, static_cast<size_t>(h->nsteps)), "cg_create: upload");
-  const cgk::StreamPlace to{h->d_chunk_off, d_step_chunk, d_step_entry, h->d_stream, h->d_val64};
+  const cgk::StreamPlace to{h->d_chunk_off, d_step_chunk, h->d_step_entry, h->d_stream, h->d_val64};
   CG_TRY(cgk::launch_layout_fill(src, h->d_step, to, 0, h->nsteps, 0, static_cast<int32_t>(n), h->col16, mixed, nullptr),
          "cg_create: stream order");
   CG_TRY(cudaDeviceSynchronize(), "cg_create: synchronize");

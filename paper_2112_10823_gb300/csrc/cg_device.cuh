@@ -1058,52 +1058,78 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
 }
 
 // out = A x in FP64 over the warp's steps [s, s1), read directly from global memory in
-// stream order: the passes outside a solve's step loop (its setup, the final
-// true residual, the mixed solve's residual replacements) take it, which leaves
-// the ring's contents alone.
+// stream order, from chunk `chunk` and (mixed) entry `entry` on: the passes outside a
+// mixed solve's step loop (its setup, the final true residual, the residual
+// replacements), which leaves the ring's contents alone, and a mixed handle's
+// product.  Latency bounds it: a step's chain would be its chunk's offset, columns,
+// x, FMAs, chunk after chunk.  So 32 chunk offsets are loaded at once, and a batch's
+// columns while the batch before waits for its x.
 template <typename Ring>
-__device__ __forceinline__ void direct_pass(const DevCsr& A, int chunk, int64_t entry, int s,
-                                         int s1, const double* x, double* out) {
+__device__ __forceinline__ void direct_pass(const DevCsr& A, uint32_t chunk, int64_t entry, int s, int s1,
+                                            const double* x, double* out) {
   using T = typename Ring::Val;
   using C = typename Ring::Col;
-  constexpr int kU = 9;  // entries per lane in flight
+  constexpr int kU = 7;  // entries per lane and batch (half an FP32 chunk)
   const int lane = fresh_tid() & 31;
   for (; s < s1; ++s) {
     const int4 d = A.step[s];
     const int seg = lane_segment(d, A.seg_len[static_cast<size_t>(s) * 32 + lane], lane);
     const double* const xb = sizeof(C) == 2 ? x + d.w : x;
-    const int size = step_chunk(d);
-    double acc = 0.0;
-    for (int u = 0; u < d.z; u += size, ++chunk) {
-      const int cnt = min(size, d.z - u), len = max(0, min(seg - u, cnt));
-      const ChunkPlace place = chunk_place<C>(d, u, cnt, seg, lane);
-      const unsigned char* const at = A.stream + static_cast<size_t>(A.chunk_off[chunk]) * kUnit;
-      const C* cp = reinterpret_cast<const C*>(at) + place.base;
-      const double* vp;
-      if constexpr (sizeof(T) == 4) vp = A.val64 + entry;
-      else vp = reinterpret_cast<const double*>(at + ((place.tot * static_cast<int>(sizeof(C)) + kUnit - 1) & ~(kUnit - 1)));
-      vp += place.base;
-      for (int k0 = 0; k0 < cnt; k0 += kU) {
-        double a[kU], g[kU];
-#pragma unroll
-        for (int k = 0; k < kU; ++k) a[k] = g[k] = 0.0;  // (not live before: no spills)
-#pragma unroll
-        for (int k = 0; k < kU; ++k) {
-          if (k0 + k < len) {
-            a[k] = __ldcs(vp);
-            g[k] = xb[__ldcs(cp)];
-          }
-          vp += place.stride;
-          cp += place.stride;
-        }
-#pragma unroll
-        for (int k = 0; k < kU; ++k) {
-          if (k0 + k >= cnt) break;
-          if (k0 + k < len) acc = fma(a[k], g[k], acc);
-        }
+    const int size = step_chunk(d), nchunks = size > 0 ? (d.z + size - 1) / size : 0;
+    uint32_t off = lane < nchunks ? A.chunk_off[chunk + lane] : 0;
+    // the batch after the one at hand: chunk j of the step, entries [k, ..) of it
+    int j = 0, k = 0, cnt = 0;
+    ChunkPlace place{0, 0, 0};
+    const C* cp = nullptr;
+    const double* vp = nullptr;
+    int c[kU] = {};
+    // columns of the next batch; returns how many of its entries this lane has
+    auto load = [&]() -> int {
+      const int u = j * size;
+      if (k == 0) {
+        if (j > 0 && (j & 31) == 0) off = j + lane < nchunks ? A.chunk_off[chunk + j + lane] : 0;
+        cnt = min(size, d.z - u);
+        place = chunk_place<C>(d, u, cnt, seg, lane);
+        const unsigned char* const at = A.stream + static_cast<size_t>(__shfl_sync(0xffffffffu, off, j & 31)) * kUnit;
+        cp = reinterpret_cast<const C*>(at) + place.base;
+        if constexpr (sizeof(T) == 4) vp = A.val64 + entry + place.base;
+        else
+          vp = reinterpret_cast<const double*>(at + ((place.tot * static_cast<int>(sizeof(C)) + kUnit - 1) & ~(kUnit - 1))) +
+               place.base;
+        entry += place.tot;
       }
-      entry += place.tot;
+      const int len = max(0, min(min(seg - u, cnt) - k, kU));
+#pragma unroll
+      for (int i = 0; i < kU; ++i, cp += place.stride)
+        if (i < len) c[i] = static_cast<int>(__ldcs(cp));
+      return len;
+    };
+    double acc = 0.0;
+    int len = nchunks > 0 ? load() : 0;
+    while (j < nchunks) {
+      double a[kU], g[kU];
+#pragma unroll
+      for (int i = 0; i < kU; ++i) a[i] = g[i] = 0.0;  // (not live before: no spills)
+#pragma unroll
+      for (int i = 0; i < kU; ++i, vp += place.stride)
+        if (i < len) {
+          a[i] = __ldcs(vp);
+          g[i] = xb[c[i]];
+        }
+      const int now = len, most = cnt - k;  // (most: warp-uniform)
+      k += kU;
+      if (k >= cnt) {
+        k = 0;
+        ++j;
+      }
+      if (j < nchunks) len = load();
+#pragma unroll
+      for (int i = 0; i < kU; ++i) {
+        if (i >= most) break;  // (a predicated-off FMA would take the pipe's time)
+        if (i < now) acc = fma(a[i], g[i], acc);
+      }
     }
+    chunk += static_cast<uint32_t>(nchunks);
     const double tot = combine_lanes(step_mode(d), acc);
     const int i = result_row(d, lane);
     if (i >= 0) out[i] = tot;

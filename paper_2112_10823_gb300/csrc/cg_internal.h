@@ -100,6 +100,8 @@ struct DevCsr {
   const int4* warp_chunk;     // [nblocks * kWarps] each warp's stream: first chunk, number of chunks,
                               // start and end of the first one (units)
   const uint32_t* warp_entry; // mixed precision: [nblocks * kWarps] its first entry in val64
+  const uint32_t* step_chunk; // mixed precision, a handle's: [nsteps] first chunk of each step,
+  const uint32_t* step_entry; // [nsteps] and its first entry in val64
   const int32_t* warp_step;   // [nblocks * kWarps + 1] first step of each warp (stream by stream)
   const int32_t* block_row;   // [nblocks + 1] first row of each CTA (vector phases)
   int32_t n;

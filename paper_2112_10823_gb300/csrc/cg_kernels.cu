@@ -58,13 +58,21 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 }
 
 // The same of a mixed-precision handle, whose streams hold FP32 values: its FP64
-// values directly from global memory, a warp per stream.
+// values directly from global memory, a warp per step.  What bounds it is the
+// latency of a step's chain (step, columns, x, FMAs), so as many warps as 64
+// registers allow (32 per SM) work on steps of their own, in small blocks, whose
+// warps give way to the next steps at once (blocks of 64, 128, 256 threads: Q1
+// 160^3 232, 238, 250 us; 48 registers spill: 267).  Q1 64^3 20.8 us, 160^3 232;
+// the former CSR ring 25.0 and 239, a warp per stream (19 per SM) 27.1 and 350.
+constexpr int kDirectThreads = 64, kDirectBlocks = 16;
+
 template <typename C>
-__global__ void __launch_bounds__(kBlock, kCtasPerSm)
+__global__ void __launch_bounds__(kDirectThreads, kDirectBlocks)
     spmv_direct_kernel(const __grid_constant__ DevCsr A, const double* x, double* y) {
   using Ring = RingSmem<float, C>;
-  const int bw = blockIdx.x * kWarps + (threadIdx.x >> 5);
-  direct_pass<Ring>(A, A.warp_chunk[bw].x, A.warp_entry[bw], A.warp_step[bw], A.warp_step[bw + 1], x,
+  const int64_t s = (static_cast<int64_t>(blockIdx.x) * kDirectThreads + threadIdx.x) >> 5;
+  if (s >= A.nsteps) return;
+  direct_pass<Ring>(A, A.step_chunk[s], A.step_entry[s], static_cast<int>(s), static_cast<int>(s) + 1, x,
                     y);
 }
 
@@ -95,8 +103,9 @@ cudaError_t ensure_smem_attr(const void* kernel, size_t bytes) {
 
 cudaError_t launch_spmv(const DevCsr& A, const double* x, double* y, int32_t* err, cudaStream_t s) {
   if (A.val64 != nullptr) {
-    if (A.col16) spmv_direct_kernel<uint16_t><<<A.nblocks, kBlock, 0, s>>>(A, x, y);
-    else spmv_direct_kernel<int32_t><<<A.nblocks, kBlock, 0, s>>>(A, x, y);
+    const unsigned blocks = static_cast<unsigned>((static_cast<int64_t>(A.nsteps) * 32 + kDirectThreads - 1) / kDirectThreads);
+    if (A.col16) spmv_direct_kernel<uint16_t><<<blocks, kDirectThreads, 0, s>>>(A, x, y);
+    else spmv_direct_kernel<int32_t><<<blocks, kDirectThreads, 0, s>>>(A, x, y);
     return cudaGetLastError();
   }
   const size_t smem = solve_smem_bytes(false, A.col16 != 0);
