@@ -479,7 +479,7 @@ void admit(cg_batch_ctx* b) {
     const cgk::DevCsr& A = b->h_sys[slot].A;
     const cgk::StreamPlace to{A.chunk_off, d.at<uint32_t>(d.L.q), d.at<uint32_t>(d.L.q) + A.nsteps,
                               d.at<unsigned char>(d.L.stream), b->mixed ? d.at<double>(d.L.val64) : nullptr};
-    cudaError_t e = cgk::launch_layout_fill(src, A.step, to, k0, k1, r0, r1, A.col16 != 0, b->mixed, s);
+    cudaError_t e = cgk::launch_layout_fill(src, d.at<int4>(d.L.step), to, k0, k1, r0, r1, A.col16 != 0, b->mixed, s);
     if (e == cudaSuccess && b->jacobi)
       e = cgk::launch_jacobi_dinv(src, r0, r1, d.at<double>(d.L.dinv), b->d_admit_err + slot, s);
     return e;

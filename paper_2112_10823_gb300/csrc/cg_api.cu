@@ -63,34 +63,25 @@ bool StepShape::valid() const {
   return true;
 }
 
-// A segment of `len` entries split evenly over as few chunks as it takes: the
-// entries of one chunk.
-static int chunk_of(int64_t len, int most) {
-  if (len <= 0) return 0;
-  const int64_t parts = (len + most - 1) / most;
-  return static_cast<int>((len + parts - 1) / parts);
-}
-
+// (the chunk size is left to place_steps)
 static int4 make_step(int64_t row, int lanes, int mode, bool uniform, int rem, int64_t seg, int64_t entries,
-                      int chunk, bool tight) {
-  static_assert(cgk::max_chunk<double>() < 64 && cgk::max_chunk<float>() < 64, "six bits");
+                      bool tight) {
   const bool pads = (lanes < 32 || !uniform) && cgk::step_pads(seg, entries, tight);
   unsigned int y = static_cast<unsigned int>(lanes) | static_cast<unsigned int>(mode) << cgk::kStepModeShift |
                    (uniform ? static_cast<unsigned int>(cgk::kStepUniform) : 0u) |
                    (pads ? static_cast<unsigned int>(cgk::kStepPadded) : 0u) |
-                   static_cast<unsigned int>(rem) << cgk::kStepRemShift |
-                   static_cast<unsigned int>(chunk_of(seg, chunk)) << cgk::kStepChunkShift;
+                   static_cast<unsigned int>(rem) << cgk::kStepRemShift;
   return make_int4(static_cast<int>(row), static_cast<int>(y), static_cast<int>(seg), 0);
 }
 
-static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end, int chunk, const StepShape& shape,
+static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end, const StepShape& shape,
                        std::vector<int4>& out) {
   auto kind = [&](int64_t len) -> int { return len > kShapeMaxLen ? cgk::kLongRow : shape.mode[len]; };
   while (row < end) {
     const int64_t len0 = rp[row + 1] - rp[row];
     if (kind(len0) == cgk::kLongRow) {  // a warp per row
       const int rem = static_cast<int>(len0 % 32);
-      out.push_back(make_step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0, chunk, shape.tight));
+      out.push_back(make_step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0, shape.tight));
       ++row;
       continue;
     }
@@ -112,9 +103,9 @@ static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end,
     const int rows = static_cast<int>(row - start);
     const int64_t cnt = rp[row] - rp[start];
     if (m == cgk::kLanePerRow)
-      out.push_back(make_step(start, rows, m, minlen == maxlen, 0, maxlen, cnt, chunk, shape.tight));
+      out.push_back(make_step(start, rows, m, minlen == maxlen, 0, maxlen, cnt, shape.tight));
     else  // two segments per row, the first one longer by an odd entry
-      out.push_back(make_step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt, chunk,
+      out.push_back(make_step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt,
                               shape.tight));
   }
 }
@@ -125,12 +116,11 @@ static int64_t rows_of(const int4& d) {
   return mode == cgk::kLanePerRow ? lanes : mode == cgk::kPairPerRow ? lanes / 2 : 1;
 }
 
-// Entries per lane of a chunk of step d.
-static int64_t chunk_size(const int4& d) { return (d.y >> cgk::kStepChunkShift) & 63; }
-
 void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, bool mixed, Partition& P,
                      const StepShape& shape) {
-  const int chunk = mixed ? cgk::max_chunk<float>() : cgk::max_chunk<double>();
+  // (the column width is not known yet: 32-bit columns have the smaller chunks)
+  const int chunk = cgk::max_chunk(mixed, false);
+  static_assert(cgk::max_chunk(true, false) <= cgk::max_chunk(true, true), "an upper bound of the chunks");
   P.step.clear();
   P.block_row.assign(static_cast<size_t>(nblocks) + 1, 0);
   for (int b = 0; b <= nblocks; ++b) P.block_row[b] = static_cast<int32_t>(cost_split(rp, 0, n, b, nblocks));
@@ -139,7 +129,7 @@ void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, boo
   std::vector<int4> rows;  // a CTA's steps in row order
   for (int b = 0; b < nblocks; ++b) {
     rows.clear();
-    warp_steps(rp, P.block_row[b], P.block_row[b + 1], chunk, shape, rows);
+    warp_steps(rp, P.block_row[b], P.block_row[b + 1], shape, rows);
     for (int w = 0; w < cgk::kWarps; ++w) {
       P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
       for (size_t k = static_cast<size_t>(w); k < rows.size(); k += cgk::kWarps) P.step.push_back(rows[k]);
@@ -148,16 +138,16 @@ void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, boo
   P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
   P.chunks = P.padded = 0;
   for (const int4& d : P.step) {
-    if (d.z > 0) P.chunks += (d.z + chunk_size(d) - 1) / chunk_size(d);
+    P.chunks += (d.z + chunk - 1) / chunk;
     P.padded += (d.y & cgk::kStepPadded) ? int64_t(32) * d.z : rp[d.x + rows_of(d)] - rp[d.x];
   }
-  P.step.push_back(make_step(n, 32, cgk::kLanePerRow, true, 0, 0, 0, chunk, false));  // the sentinel: no entries
+  P.step.push_back(make_step(n, 32, cgk::kLanePerRow, true, 0, 0, 0, false));  // the sentinel: no entries
 }
 
-// Calls f(entries) for each chunk of step d, in order.
+// Calls f(entries) for each chunk (of at most `most` entries per lane) of step d, in order.
 template <typename F>
-static void for_chunks(const std::vector<int32_t>& rp, const int4& d, bool col16, F&& f) {
-  const int64_t size = chunk_size(d), lanes = d.y & 0xff, seg = d.z;
+static void for_chunks(const std::vector<int32_t>& rp, const int4& d, bool col16, int most, F&& f) {
+  const int64_t size = cgk::chunk_of(d.z, most), lanes = d.y & 0xff, seg = d.z;
   const int mode = (d.y >> cgk::kStepModeShift) & 3;
   const bool padded = col16 && (d.y & cgk::kStepPadded), uniform = (d.y & cgk::kStepUniform) != 0;
   for (int64_t u = 0; u < seg; u += size) {  // (size > 0 when seg is)
@@ -197,7 +187,7 @@ void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool m
     for (int k = P.warp_step[bw]; k < P.warp_step[bw + 1]; ++k) {
       P.step_chunk[k] = static_cast<uint32_t>(P.chunk_off.size());
       if (mixed) P.step_entry[k] = static_cast<uint32_t>(entry);
-      for_chunks(rp, P.step[k], col16, [&](int64_t cnt) {
+      for_chunks(rp, P.step[k], col16, cgk::max_chunk(mixed, col16), [&](int64_t cnt) {
         P.chunk_off.push_back(static_cast<uint32_t>(at));
         at += cgk::chunk_units(cnt, col16 ? 2 : 4, mixed ? 4 : 8);
         entry += cnt;

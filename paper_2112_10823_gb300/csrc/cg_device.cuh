@@ -507,7 +507,8 @@ template <typename T, typename C>
 struct RingSmem {
   using Val = T;
   using Col = C;
-  static constexpr int kSlotBytes = static_cast<int>(kUnit * chunk_units(32 * max_chunk<T>(), sizeof(C), sizeof(T)));
+  static constexpr int kChunk = max_chunk(sizeof(T) == 4, sizeof(C) == 2);
+  static constexpr int kSlotBytes = static_cast<int>(kUnit * chunk_units(32 * kChunk, sizeof(C), sizeof(T)));
   static constexpr size_t kStateOff = (8 * kSlots * kWarps + 15) & ~size_t(15);
   static constexpr size_t kSumOff = kStateOff + ((sizeof(CtaState) + 15) & ~size_t(15));
   static constexpr size_t kStreamOff = (kSumOff + sizeof(SumScratch) + 15) & ~size_t(15);
@@ -683,7 +684,7 @@ __device__ __forceinline__ void stop_producer(const Ring& sm) {
 __device__ __forceinline__ int step_lanes(const int4& d) { return d.y & 0xff; }
 __device__ __forceinline__ int step_mode(const int4& d) { return (d.y >> kStepModeShift) & 3; }
 
-__device__ __forceinline__ int step_chunk(const int4& d) { return (d.y >> kStepChunkShift) & 63; }
+__device__ __forceinline__ int step_chunk(const int4& d) { return (d.y >> kStepChunkShift) & kStepChunkMask; }
 
 // Whether step d is stored padded (with columns of type C).
 template <typename C>
@@ -809,7 +810,7 @@ template <typename Ring, typename X>
 __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, const X* x, bool with_dot) {
   using T = typename Ring::Val;
   using C = typename Ring::Col;
-  constexpr int kU = max_chunk<T>();
+  constexpr int kU = Ring::kChunk;
   const Ring sm{smem};
   const PassIo& io = sm.state()->io;
   const int tid = fresh_tid(), w = tid >> 5, lane = tid & 31;

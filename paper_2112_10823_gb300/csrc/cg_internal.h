@@ -36,7 +36,16 @@ constexpr int kCtasPerSm = 1;
 // chunks, was slower: 64^3 33.1 against 29.3 us per step, with 15 warps).  FP32
 // 14: a 27-entry row is two chunks, which are gathered together (9, gathered one
 // chunk ahead as in FP64: 26.5 against 25.2 us, with 15 warps).
-template <typename T> __host__ __device__ constexpr int max_chunk() { return sizeof(T) == 8 ? 9 : 14; }
+// FP32 with 32-bit columns 11: the rings then leave 92 KB of L1 instead of 28, and
+// scattered gathers have one L1 line each (110^3 mesh in random numbering, chunks of
+// 9, 10, 11, 12, 14: 145, 144, 144, 155, 250 us per step; in its own numbering 84,
+// 84, 84, 87, 115; rows of 1 to 32 entries 31.0, 31.5, 26.1, 27.1, 27.0).
+__host__ __device__ constexpr int max_chunk(bool mixed, bool col16) { return !mixed ? 9 : col16 ? 14 : 11; }
+// A segment of `len` entries split evenly over as few chunks of at most `most` as
+// it takes: the entries of one chunk.
+__host__ __device__ constexpr int chunk_of(int len, int most) {
+  return len <= 0 ? 0 : (len + (len + most - 1) / most - 1) / ((len + most - 1) / most);
+}
 // Slots of a warp's ring: the chunk being summed, the next one and a copy in
 // flight, 150 to 200 KB in all.  The rest of the SM's 256 KB serves the gathers
 // as L1.  (Two slots: 160^3 383 against 292 us per step, with 15 warps.)
@@ -45,8 +54,8 @@ constexpr int kSlots = 3;
 constexpr unsigned long long kProducerIdleNs = 60000000000ull;
 constexpr int kLaneMax = 32;  // longest row computed by a single lane
 // Largest CTA share (rows) of the small-share solve kernels, which keep the
-// share's r in shared memory (20 KB behind the ring layout; the FP32 layout
-// with 32-bit columns then takes 224 KB of the 227 KB a CTA may have).
+// share's r in shared memory (20 KB behind the ring layout; the FP64 layout
+// with 32-bit columns then takes 221 KB of the 227 KB a CTA may have).
 constexpr int kLocalRows = 2560;
 
 // A chunk in memory, and in a slot: its columns, then its values, each padded
@@ -74,6 +83,7 @@ constexpr int kStepUniform = 1 << 10;
 constexpr int kStepPadded = 1 << 11;
 constexpr int kStepRemShift = 16;
 constexpr int kStepChunkShift = 24;
+constexpr int kStepChunkMask = 63;
 // Columns are stored as 16-bit offsets from their step's smallest column when
 // every step of the matrix spans at most this much, and as 32-bit columns
 // otherwise.
@@ -242,7 +252,8 @@ cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_le
 // chunks step_chunk[k].. of step k, at the units that chunk_off gives (16-bit
 // column offsets if col16, else 32-bit columns; FP32 values, rounded to nearest,
 // if mixed), and if mixed the FP64 values from val64[step_entry[k]] on.
-// Padding of entries: zeros.
+// Padding of entries: zeros.  Sets the steps' chunk sizes to those of the column
+// width (max_chunk).
 struct StreamPlace {
   const uint32_t* chunk_off;
   const uint32_t* step_chunk;
@@ -250,7 +261,7 @@ struct StreamPlace {
   unsigned char* stream;
   double* val64;               // mixed
 };
-cudaError_t launch_layout_fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
+cudaError_t launch_layout_fill(const CsrSource& src, int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
                                int32_t row0, int32_t row1, bool col16, bool mixed, cudaStream_t s);
 // dinv[i] = 1 / (sum of row i's stored entries in column i) for rows [row0, row1);
 // err set to the first row (+1) found whose diagonal is not positive.

@@ -18,7 +18,7 @@ struct Partition {
   std::vector<int4> step;
   std::vector<int32_t> warp_step;
   std::vector<int32_t> block_row;
-  int64_t chunks = 0;        // of all streams
+  int64_t chunks = 0;        // of all streams (at most)
   int64_t padded = 0;        // entries with the padding of 16-bit columns
   // by place_steps
   std::vector<int4> warp_chunk;

@@ -64,13 +64,16 @@ __global__ void __launch_bounds__(kLayoutBlock)
 
 template <typename T, typename C>
 __global__ void __launch_bounds__(kLayoutBlock)
-    layout_fill_kernel(const CsrSource src, const int4* __restrict__ step, const StreamPlace to, int32_t s0,
+    layout_fill_kernel(const CsrSource src, int4* __restrict__ step, const StreamPlace to, int32_t s0,
                        int32_t s1, int32_t row0, int32_t row1) {
   const int s = s0 + static_cast<int>((static_cast<int64_t>(blockIdx.x) * kLayoutBlock + threadIdx.x) >> 5);
   if (s >= s1) return;
   const int lane = threadIdx.x & 31;
-  const int4 d = step[s];
+  int4 d = step[s];
   if (d.x < row0 || d.x >= row1) return;
+  const int size = chunk_of(d.z, max_chunk(sizeof(T) == 4, sizeof(C) == 2));
+  d.y = (d.y & ~(kStepChunkMask << kStepChunkShift)) | size << kStepChunkShift;
+  if (lane == 0) step[s].y = d.y;
   const int mode = step_mode(d);
   // this lane's segment in CSR order: entries a, a + stride, ...
   int64_t a = 0;
@@ -97,7 +100,6 @@ __global__ void __launch_bounds__(kLayoutBlock)
   a -= src.e_first;
   const int base = src.base + (sizeof(C) == 2 ? d.w : 0);
   const bool padded = step_padded<C>(d);
-  const int size = step_chunk(d);
   uint32_t chunk = to.step_chunk[s];
   int64_t entry = sizeof(T) == 4 ? to.step_entry[s] : 0;
   for (int u0 = 0; u0 < d.z; u0 += size, ++chunk) {
@@ -128,7 +130,7 @@ cudaError_t launch_layout_scan(const CsrSource& src, int4* step, uint8_t* seg_le
   return cudaGetLastError();
 }
 
-cudaError_t launch_layout_fill(const CsrSource& src, const int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
+cudaError_t launch_layout_fill(const CsrSource& src, int4* step, const StreamPlace& to, int32_t s0, int32_t s1,
                                int32_t row0, int32_t row1, bool col16, bool mixed, cudaStream_t s) {
   if (s1 <= s0) return cudaSuccess;
   auto fill = [&](auto kernel) { kernel<<<layout_grid(s0, s1), kLayoutBlock, 0, s>>>(src, step, to, s0, s1, row0, row1); };
