@@ -5,7 +5,9 @@
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
+#include <initializer_list>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -74,14 +76,45 @@ static int4 make_step(int64_t row, int lanes, int mode, bool uniform, int rem, i
   return make_int4(static_cast<int>(row), static_cast<int>(y), static_cast<int>(seg), 0);
 }
 
-static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end, const StepShape& shape,
-                       std::vector<int4>& out) {
+// The steps of rows [row, end) in row order into out[] (room for a step per row);
+// returns their number and adds up P.chunks and P.padded.
+static size_t warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end, const StepShape& shape, bool mixed,
+                         int4* out, Partition& P) {
+  // (the column width is not known yet: 32-bit columns have the smaller chunks)
+  constexpr int kChunk64 = cgk::max_chunk(false, false), kChunk32 = cgk::max_chunk(true, false);
+  static_assert(kChunk32 <= cgk::max_chunk(true, true), "an upper bound of the chunks");
+  size_t count = 0;
+  int64_t chunks = 0, padded = 0;
+  auto step = [&](int64_t first, int lanes, int mode, bool uniform, int rem, int64_t seg, int64_t entries) {
+    const int4 d = make_step(first, lanes, mode, uniform, rem, seg, entries, shape.tight);
+    out[count++] = d;
+    chunks += mixed ? (seg + kChunk32 - 1) / kChunk32 : (seg + kChunk64 - 1) / kChunk64;
+    padded += (d.y & cgk::kStepPadded) ? 32 * seg : entries;
+  };
   auto kind = [&](int64_t len) -> int { return len > kShapeMaxLen ? cgk::kLongRow : shape.mode[len]; };
+  int short_rows = -1;  // rows of up to this many entries are all of one lane
+  while (short_rows < kShapeMaxLen && shape.mode[short_rows + 1] == cgk::kLanePerRow) ++short_rows;
   while (row < end) {
+    // 32 such rows are a step (the usual case, in loops that the compiler vectorises:
+    // 4.1 M rows 10.1 ms row by row, 1.9 so)
+    if (row + 32 <= end && rp[row + 1] - rp[row] <= short_rows) {
+      const int32_t* const at = rp.data() + row;
+      int32_t longest = 0, shortest = INT32_MAX;
+      for (int k = 0; k < 32; ++k) {
+        const int32_t len = at[k + 1] - at[k];
+        longest = longest > len ? longest : len;
+        shortest = shortest < len ? shortest : len;
+      }
+      if (longest <= short_rows) {
+        step(row, 32, cgk::kLanePerRow, shortest == longest, 0, longest, at[32] - at[0]);
+        row += 32;
+        continue;
+      }
+    }
     const int64_t len0 = rp[row + 1] - rp[row];
     if (kind(len0) == cgk::kLongRow) {  // a warp per row
       const int rem = static_cast<int>(len0 % 32);
-      out.push_back(make_step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0, shape.tight));
+      step(row, 32, cgk::kLongRow, rem == 0, rem, (len0 + 31) / 32, len0);
       ++row;
       continue;
     }
@@ -103,11 +136,13 @@ static void warp_steps(const std::vector<int32_t>& rp, int64_t row, int64_t end,
     const int rows = static_cast<int>(row - start);
     const int64_t cnt = rp[row] - rp[start];
     if (m == cgk::kLanePerRow)
-      out.push_back(make_step(start, rows, m, minlen == maxlen, 0, maxlen, cnt, shape.tight));
+      step(start, rows, m, minlen == maxlen, 0, maxlen, cnt);
     else  // two segments per row, the first one longer by an odd entry
-      out.push_back(make_step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt,
-                              shape.tight));
+      step(start, 2 * rows, m, minlen == maxlen && maxlen % 2 == 0, 0, (maxlen + 1) / 2, cnt);
   }
+  P.chunks += chunks;
+  P.padded += padded;
+  return count;
 }
 
 // Rows of step k of P.
@@ -118,91 +153,104 @@ static int64_t rows_of(const int4& d) {
 
 void build_partition(const std::vector<int32_t>& rp, int64_t n, int nblocks, bool mixed, Partition& P,
                      const StepShape& shape) {
-  // (the column width is not known yet: 32-bit columns have the smaller chunks)
-  const int chunk = cgk::max_chunk(mixed, false);
-  static_assert(cgk::max_chunk(true, false) <= cgk::max_chunk(true, true), "an upper bound of the chunks");
   P.step.clear();
   P.block_row.assign(static_cast<size_t>(nblocks) + 1, 0);
   for (int b = 0; b <= nblocks; ++b) P.block_row[b] = static_cast<int32_t>(cost_split(rp, 0, n, b, nblocks));
   P.block_row[nblocks] = static_cast<int32_t>(n);
   P.warp_step.clear();
-  std::vector<int4> rows;  // a CTA's steps in row order
+  P.chunks = P.padded = 0;
+  int32_t most_rows = 1;
+  for (int b = 0; b < nblocks; ++b) most_rows = std::max(most_rows, P.block_row[b + 1] - P.block_row[b]);
+  std::unique_ptr<int4[]> rows(new int4[static_cast<size_t>(most_rows)]);  // a CTA's steps in row order (not cleared)
   for (int b = 0; b < nblocks; ++b) {
-    rows.clear();
-    warp_steps(rp, P.block_row[b], P.block_row[b + 1], shape, rows);
+    const size_t count = warp_steps(rp, P.block_row[b], P.block_row[b + 1], shape, mixed, rows.get(), P);
+    if (b == 0) P.step.reserve((count + count / 8 + 1) * static_cast<size_t>(nblocks));  // (CTAs are alike)
     for (int w = 0; w < cgk::kWarps; ++w) {
       P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
-      for (size_t k = static_cast<size_t>(w); k < rows.size(); k += cgk::kWarps) P.step.push_back(rows[k]);
+      for (size_t k = static_cast<size_t>(w); k < count; k += cgk::kWarps) P.step.push_back(rows[k]);
     }
   }
   P.warp_step.push_back(static_cast<int32_t>(P.step.size()));
-  P.chunks = P.padded = 0;
-  for (const int4& d : P.step) {
-    P.chunks += (d.z + chunk - 1) / chunk;
-    P.padded += (d.y & cgk::kStepPadded) ? int64_t(32) * d.z : rp[d.x + rows_of(d)] - rp[d.x];
-  }
   P.step.push_back(make_step(n, 32, cgk::kLanePerRow, true, 0, 0, 0, false));  // the sentinel: no entries
 }
 
-// Calls f(entries) for each chunk (of at most `most` entries per lane) of step d, in order.
-template <typename F>
-static void for_chunks(const std::vector<int32_t>& rp, const int4& d, bool col16, int most, F&& f) {
-  const int64_t size = cgk::chunk_of(d.z, most), lanes = d.y & 0xff, seg = d.z;
+// Calls f(entries) for each chunk of step d, in order.
+template <bool kCol16, bool kMixed, typename F>
+static void for_chunks(const std::vector<int32_t>& rp, const int4& d, F&& f) {
+  const int size = cgk::chunk_of(d.z, cgk::max_chunk(kMixed, kCol16)), lanes = d.y & 0xff, seg = d.z;
   const int mode = (d.y >> cgk::kStepModeShift) & 3;
-  const bool padded = col16 && (d.y & cgk::kStepPadded), uniform = (d.y & cgk::kStepUniform) != 0;
-  for (int64_t u = 0; u < seg; u += size) {  // (size > 0 when seg is)
-    const int64_t cnt = std::min(size, seg - u);
-    if (padded) {
-      f(32 * cnt);
-    } else if (uniform) {
-      f(lanes * cnt);
-    } else if (mode == cgk::kLongRow) {  // all lanes but in the last, partial stride
-      const int64_t rem = (d.y >> cgk::kStepRemShift) & 0x3f;
+  const bool padded = kCol16 && (d.y & cgk::kStepPadded);
+  if (padded || (d.y & cgk::kStepUniform)) {
+    const int64_t each = padded ? 32 : lanes;
+    for (int u = 0; u < seg; u += size) f(each * std::min(size, seg - u));  // (size > 0 when seg is)
+  } else if (mode == cgk::kLongRow) {  // all lanes but in the last, partial stride
+    const int rem = (d.y >> cgk::kStepRemShift) & 0x3f;
+    for (int u = 0; u < seg; u += size) {
+      const int64_t cnt = std::min(size, seg - u);
       f(u + cnt == seg ? 32 * (cnt - 1) + rem : 32 * cnt);
+    }
+  } else {
+    int32_t len[32] = {};
+    const int rows = static_cast<int>(rows_of(d));
+    const int32_t* const at = rp.data() + d.x;
+    if (mode == cgk::kLanePerRow) {
+      for (int i = 0; i < rows; ++i) len[i] = at[i + 1] - at[i];
     } else {
-      int64_t tot = 0;
-      const int64_t rows = rows_of(d);
-      for (int64_t i = d.x; i < d.x + rows; ++i) {
-        const int64_t len = rp[i + 1] - rp[i];
-        auto part = [&](int64_t l) { return std::max<int64_t>(0, std::min(l - u, cnt)); };
-        tot += mode == cgk::kLanePerRow ? part(len) : part((len + 1) / 2) + part(len / 2);
+      for (int i = 0; i < rows; ++i) {
+        len[i] = (at[i + 1] - at[i] + 1) / 2;
+        len[16 + i] = (at[i + 1] - at[i]) / 2;
+      }
+    }
+    for (int u = 0; u < seg; u += size) {
+      const int cnt = std::min(size, seg - u);
+      int tot = 0;
+      for (int i = 0; i < 32; ++i) {
+        const int left = len[i] - u < cnt ? len[i] - u : cnt;
+        tot += left > 0 ? left : 0;
       }
       f(tot);
     }
   }
 }
 
-void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool mixed, Partition& P) {
+template <bool kCol16, bool kMixed>
+static void place(const std::vector<int32_t>& rp, int nblocks, Partition& P) {
   const size_t warps = static_cast<size_t>(nblocks) * cgk::kWarps;
   P.step_chunk.assign(P.step.size(), 0);
-  P.step_entry.assign(mixed ? P.step.size() : 0, 0);
+  P.step_entry.assign(kMixed ? P.step.size() : 0, 0);
   P.warp_chunk.assign(warps, int4{0, 0, 0, 0});
-  P.warp_entry.assign(mixed ? warps : 0, 0);
-  P.chunk_off.clear();
-  P.chunk_off.reserve(static_cast<size_t>(P.chunks) + 1);
+  P.warp_entry.assign(kMixed ? warps : 0, 0);
+  P.chunk_off.resize(static_cast<size_t>(P.chunks) + 1);
   int64_t at = 0, entry = 0;
+  size_t chunk = 0;
   for (size_t bw = 0; bw < warps; ++bw) {
-    const size_t c0 = P.chunk_off.size();
-    if (mixed) P.warp_entry[bw] = static_cast<uint32_t>(entry);
+    const size_t c0 = chunk;
+    if (kMixed) P.warp_entry[bw] = static_cast<uint32_t>(entry);
     for (int k = P.warp_step[bw]; k < P.warp_step[bw + 1]; ++k) {
-      P.step_chunk[k] = static_cast<uint32_t>(P.chunk_off.size());
-      if (mixed) P.step_entry[k] = static_cast<uint32_t>(entry);
-      for_chunks(rp, P.step[k], col16, cgk::max_chunk(mixed, col16), [&](int64_t cnt) {
-        P.chunk_off.push_back(static_cast<uint32_t>(at));
-        at += cgk::chunk_units(cnt, col16 ? 2 : 4, mixed ? 4 : 8);
+      P.step_chunk[k] = static_cast<uint32_t>(chunk);
+      if (kMixed) P.step_entry[k] = static_cast<uint32_t>(entry);
+      for_chunks<kCol16, kMixed>(rp, P.step[k], [&](int64_t cnt) {
+        P.chunk_off[chunk++] = static_cast<uint32_t>(at);
+        at += cgk::chunk_units(cnt, kCol16 ? 2 : 4, kMixed ? 4 : 8);
         entry += cnt;
       });
     }
     P.warp_chunk[bw].x = static_cast<int32_t>(c0);
-    P.warp_chunk[bw].y = static_cast<int32_t>(P.chunk_off.size() - c0);
+    P.warp_chunk[bw].y = static_cast<int32_t>(chunk - c0);
   }
-  P.chunk_off.push_back(static_cast<uint32_t>(at));
+  P.chunk_off[chunk] = static_cast<uint32_t>(at);
+  P.chunk_off.resize(chunk + 1);
   for (int4& c : P.warp_chunk) {
     c.z = static_cast<int32_t>(P.chunk_off[static_cast<size_t>(c.x)]);
     c.w = static_cast<int32_t>(P.chunk_off[static_cast<size_t>(c.x) + (c.y > 0)]);
   }
   P.stream_units = at;
   P.entries = entry;
+}
+
+void place_steps(const std::vector<int32_t>& rp, int nblocks, bool col16, bool mixed, Partition& P) {
+  if (mixed) col16 ? place<true, true>(rp, nblocks, P) : place<false, true>(rp, nblocks, P);
+  else col16 ? place<true, false>(rp, nblocks, P) : place<false, false>(rp, nblocks, P);
 }
 
 void stream_bound(int64_t nnz, bool mixed, const Partition& P, int64_t* stream_units, int64_t* entries) {
@@ -306,6 +354,34 @@ struct Block {
     return cudaSuccess;
   }
 };
+
+// Uploads host arrays into consecutive parts of a Block, `at` bytes behind base:
+// small ones in one copy, large ones as they are (assembling them would cost more
+// than the copies).
+struct Table {
+  size_t at;
+  const void* src;
+  size_t bytes;
+};
+cudaError_t upload(void* base, std::initializer_list<Table> parts) {
+  size_t total = 0;
+  for (const Table& t : parts) total = std::max(total, t.at + t.bytes);
+  cudaError_t e = cudaSuccess;
+  if (total <= (size_t(256) << 10)) {
+    std::vector<char> all(total);
+    for (const Table& t : parts)
+      if (t.bytes) std::memcpy(all.data() + t.at, t.src, t.bytes);
+    return total ? cudaMemcpy(base, all.data(), total, cudaMemcpyHostToDevice) : e;
+  }
+  for (const Table& t : parts)
+    if (e == cudaSuccess && t.bytes)
+      e = cudaMemcpy(static_cast<char*>(base) + t.at, t.src, t.bytes, cudaMemcpyHostToDevice);
+  return e;
+}
+template <typename T>
+Table table(size_t at, const std::vector<T>& v) {
+  return Table{at, v.data(), sizeof(T) * v.size()};
+}
 
 void release(cg_ctx* h) {
   if (!h) return;
@@ -638,7 +714,6 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   const size_t at_step = blk.add(&h->d_step, part.step.size());  // (the tables of one upload first)
   const size_t at_wstep = blk.add(&h->d_warp_step, part.warp_step.size());
   const size_t at_brow = blk.add(&h->d_block_row, part.block_row.size());
-  std::vector<char> tables(blk.bytes);
   blk.add(&h->d_step_cmax, part.step.size());
   blk.add(&h->d_seg_len, 32 * static_cast<size_t>(h->nsteps) + 64);
   blk.add(&h->d_r, nn);
@@ -657,14 +732,33 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
     blk.add(&h->d_csr_col, nz);
     blk.add(&h->d_csr_val, nz);
   }
+  // The streams, whose size the scan tells: with the rest where their bound is
+  // small (an allocation of more than a megabyte takes 100 us, and 50 to free)
+  int64_t most_units = 0, most_entries = 0;
+  cgh::stream_bound(nnz, mixed, part, &most_units, &most_entries);
+  const size_t most = static_cast<size_t>(most_units) * cgk::kUnit + sizeof(double) * static_cast<size_t>(mixed ? most_entries : 0);
+  const bool one_block = most <= (size_t(16) << 20);
+  Block str;
+  Block& sb = one_block ? blk : str;
+  const size_t warps = static_cast<size_t>(h->nblocks) * cgk::kWarps, steps = mixed ? static_cast<size_t>(h->nsteps) : 0;
+  size_t at_wchunk = 0, at_wentry = 0, at_coff = 0, at_schunk = 0, at_sentry = 0;
+  auto add_streams = [&](size_t chunks, int64_t units, int64_t entries) {
+    at_wchunk = sb.add(&h->d_warp_chunk, warps);
+    at_wentry = sb.add(&h->d_warp_entry, mixed ? warps : 0) - at_wchunk;
+    at_schunk = sb.add(&h->d_step_chunk, steps) - at_wchunk;
+    at_sentry = sb.add(&h->d_step_entry, steps) - at_wchunk;
+    at_coff = sb.add(&h->d_chunk_off, chunks + 1) - at_wchunk;
+    sb.add(&h->d_stream, static_cast<size_t>(units) * cgk::kUnit);
+    if (mixed) sb.add(&h->d_val64, static_cast<size_t>(entries));
+    at_wchunk = 0;
+  };
+  if (one_block) add_streams(static_cast<size_t>(part.chunks), most_units, most_entries);
   CG_TRY(blk.alloc(h->allocs), "cg_create: cudaMalloc");
   h->d_ctrl = reinterpret_cast<cgk::SolveCtrl*>(ctrl);
   h->d_flags = reinterpret_cast<unsigned long long*>(ctrl + ctrl_flags_offset());
   CG_TRY(cudaMallocHost(&h->h_ctrl, sizeof(cgk::SolveCtrl)), "cg_create: cudaMallocHost");
-  std::memcpy(tables.data() + at_step, part.step.data(), sizeof(int4) * part.step.size());
-  std::memcpy(tables.data() + at_wstep, part.warp_step.data(), sizeof(int32_t) * part.warp_step.size());
-  std::memcpy(tables.data() + at_brow, part.block_row.data(), sizeof(int32_t) * part.block_row.size());
-  CG_TRY(cudaMemcpy(h->d_step, tables.data(), tables.size(), cudaMemcpyHostToDevice), "cg_create: upload");
+  CG_TRY(upload(h->d_step, {table(at_step, part.step), table(at_wstep, part.warp_step), table(at_brow, part.block_row)}),
+         "cg_create: upload");
   CG_TRY(cudaMemset(h->d_err, 0, 64), "cg_create: memset");
 
   // The CSR arrays on the device for the time of the conversion: the caller's
@@ -731,32 +825,22 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   }
   h->col16 = found.scan.span <= cgk::kColSpan16;
   cgh::place_steps(rp, h->nblocks, h->col16, mixed, part);
-  Block str;
-  const size_t at_wchunk = str.add(&h->d_warp_chunk, part.warp_chunk.size());  // (one upload again)
-  const size_t at_wentry = str.add(&h->d_warp_entry, part.warp_entry.size());
-  const size_t at_coff = str.add(&h->d_chunk_off, part.chunk_off.size());
-  const size_t steps = mixed ? static_cast<size_t>(h->nsteps) : 0;
-  const size_t at_schunk = str.add(&h->d_step_chunk, steps), at_sentry = str.add(&h->d_step_entry, steps);
-  tables.assign(str.bytes, 0);
-  str.add(&h->d_stream, static_cast<size_t>(part.stream_units) * cgk::kUnit);
-  if (mixed) str.add(&h->d_val64, static_cast<size_t>(part.entries));
-  CG_TRY(str.alloc(h->allocs), "cg_create: cudaMalloc");
-  std::memcpy(tables.data() + at_wchunk, part.warp_chunk.data(), sizeof(int4) * part.warp_chunk.size());
-  if (mixed) std::memcpy(tables.data() + at_wentry, part.warp_entry.data(), 4 * part.warp_entry.size());
-  std::memcpy(tables.data() + at_coff, part.chunk_off.data(), 4 * part.chunk_off.size());
+  if (!one_block) {
+    add_streams(part.chunk_off.size() - 1, part.stream_units, part.entries);
+    CG_TRY(str.alloc(h->allocs), "cg_create: cudaMalloc");
+  }
   // in FP64 the steps' places in the streams serve the conversion only: q holds
   // them until the handle's first solve (a step has at least one row)
   static_assert(sizeof(double) >= sizeof(uint32_t), "step_chunk fits q");
-  uint32_t* d_step_chunk = reinterpret_cast<uint32_t*>(h->d_q);
-  if (mixed) {
-    d_step_chunk = h->d_step_chunk;
-    std::memcpy(tables.data() + at_schunk, part.step_chunk.data(), 4 * steps);
-    std::memcpy(tables.data() + at_sentry, part.step_entry.data(), 4 * steps);
-  } else if (h->nsteps > 0) {
-    CG_TRY(cudaMemcpy(d_step_chunk, part.step_chunk.data(), 4 * static_cast<size_t>(h->nsteps), cudaMemcpyHostToDevice),
-           "cg_create: upload");
-  }
-  CG_TRY(cudaMemcpy(h->d_warp_chunk, tables.data(), tables.size(), cudaMemcpyHostToDevice), "cg_create: upload");
+  uint32_t* const d_step_chunk = mixed ? h->d_step_chunk : reinterpret_cast<uint32_t*>(h->d_q);
+  part.step_chunk.resize(static_cast<size_t>(h->nsteps));  // (no sentinel)
+  part.step_entry.resize(steps);
+  if (!mixed) CG_TRY(upload(d_step_chunk, {table(0, part.step_chunk)}), "cg_create: upload");
+  part.step_chunk.resize(steps);
+  CG_TRY(upload(h->d_warp_chunk, {table(at_wchunk, part.warp_chunk), table(at_wentry, part.warp_entry),
+                                  table(at_schunk, part.step_chunk), table(at_sentry, part.step_entry),
+                                  table(at_coff, part.chunk_off)}),
+         "cg_create: upload");
   const cgk::StreamPlace to{h->d_chunk_off, d_step_chunk, h->d_step_entry, h->d_stream, h->d_val64};
   CG_TRY(cgk::launch_layout_fill(src, h->d_step, to, 0, h->nsteps, 0, static_cast<int32_t>(n), h->col16, mixed, nullptr),
          "cg_create: stream order");
