@@ -218,8 +218,9 @@ int cg_probe_fp64_peak(int32_t device, double* gflops);
  * solve kernels' block, runs `iters` group barriers (*barrier_us: the
  * barrier a solve step ends with) and then `iters` group sums
  * (*sum_us: a CTA value published, the barrier, the group's values summed
- * exactly in fixed point, as for alpha and beta), each between CTA barriers
- * as in a step; the results are microseconds per barrier and per sum (CUDA
+ * exactly in fixed point: the general form of the solves' sums; those of alpha
+ * and beta usually go through accumulators, at about half of it), each between
+ * CTA barriers as in a step; the results are microseconds per barrier and per sum (CUDA
  * events, one warm-up launch first).  device < 0: the current device.
  * iters in [1, 10^6] (2*10^4 takes about 0.1 s).  Returns CG_ETIMEOUT if a
  * wait gave up (2 s), CG_EINVAL for bad arguments.

@@ -675,13 +675,14 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
 
   Partition part;
   const bool mixed = o.precision == CG_PREC_MIXED;
-  // A system of at most 16 rows per warp of the whole GPU: two lanes per row, so
-  // that more warps work and each row's FMA chain, which bounds so small a
-  // product, is half as long (24^3: 8.0 -> 7.0 us per product; 32^3, near the
-  // line: 14.4 -> 12.9 us per step).  By the size alone, so that a product's bits
-  // do not depend on the CTA count.
+  // A system of at most 12 rows per warp of the whole GPU with rows long enough:
+  // two lanes per row, so that more warps work and each row's FMA chain, which
+  // bounds so small a product, is half as long (whole-grid step with one lane, with
+  // two, us: Q1 16^3 11.9, 10.7; 24^3 11.9, 11.0; 32^3 12.5, 12.2; beyond the line
+  // 35^3 12.9, 13.6, its mesh 13.5, 15.1; rows of 7 entries 32^3 10.1, 10.4).  By the
+  // matrix alone, so that a product's bits do not depend on the CTA count.
   cgh::StepShape shape;
-  if (n <= static_cast<int64_t>(sms) * 16 * cgk::kWarps)
+  if (n <= static_cast<int64_t>(sms) * 12 * cgk::kWarps && nnz >= 12 * n)
     for (int L = 0; L <= cgk::kLaneMax; ++L) shape.mode[L] = static_cast<int8_t>(cgk::kPairPerRow);
   build_partition(rp, n, h->nblocks, mixed, part, shape);
   h->nsteps = static_cast<int>(part.step.size()) - 1;

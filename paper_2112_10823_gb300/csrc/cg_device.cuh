@@ -74,8 +74,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-
-
 __device__ __forceinline__ int ld_volatile_i32(const int32_t* p) {
   return *reinterpret_cast<const volatile int32_t*>(p);
 }
@@ -311,10 +309,15 @@ __device__ __forceinline__ double fx_warp_sum_array(const double* src, int count
 //
 // The integers' unit is set by the last sum of the same kind, of biased exponent
 // eb: 2^(eb - 1085), i.e. that sum was about 2^62 units.  A CTA's value is
-// rounded to a unit (152 of them: 2^-54 of a sum as large as the last).  Values
-// of up to 2^73 units go in (growth by 2^11), split in a signed high part (53
-// bits) and 32 low bits; anything else, or a sum that came out below 2^54 units
-// (its precision would suffer), makes every CTA take the general form instead.
+// rounded to a unit: 152 roundings of half a unit are at most 2^-55.7 of a sum as
+// large as the last, and 2^-47.7 of the smallest one accepted, 2^54 units (a sum
+// that fell by 2^8).  The general form rounds the CTAs' values to 2^-51 of the
+// largest of them: at most 2^-44.7 of a sum that one CTA dominates, and some 2^-52
+// of one with even shares, so a sum of even shares that fell by 20 times or more
+// from one step to the next is the one case in which this form is the coarser.
+// Values of up to 2^73 units go in (growth by 2^11), split in a signed high part
+// (53 bits) and 32 low bits; anything else, or a sum below 2^54 units, makes every
+// CTA take the general form instead.
 // Low word: 42 bits of low parts, 11 of CTAs that could not add theirs, 11 of
 // arrivals; high word: 53 bits of high parts, 11 of arrivals.
 constexpr int kAccUnit = 1085;
@@ -435,9 +438,6 @@ __device__ __forceinline__ bool group_barrier_t0(SolveCtrl* ctrl, unsigned long 
 
 // ------------------------------------------------------ streamed CSR product
 
-// Per-CTA state of a solve, in shared memory: written by thread 0 (between
-// CTA barriers), read by all.  Keeping it out of registers leaves the
-// product in the step loop the registers it needs.
 // What a product reads and writes besides the warp's ring.  In shared memory and
 // read where it is used: the product's registers hold what it gathers.
 struct PassIo {
@@ -454,6 +454,9 @@ __device__ __forceinline__ PassIo pass_io(const DevCsr& A, int32_t stream_rows, 
   return PassIo{A.step, A.seg_len, aux, out, limit_ns, A.nsteps, stream_rows};
 }
 
+// Per-CTA state of a solve, in shared memory: written by thread 0 (between
+// CTA barriers), read by all.  Keeping it out of registers leaves the
+// product in the step loop the registers it needs.
 struct CtaState {
   PassIo io;
   double rho;                  // r.z (r.r without a preconditioner)
@@ -804,8 +807,8 @@ __device__ __forceinline__ void load_first_steps(const Ring& sm, const PassIo& v
 // next one, each issued into the register that the current chunk's FMA has just
 // freed.  A warp-uniform branch, not a predicate, ends a chunk's FMAs.  The
 // stream's `failed` is raised if a wait gave up.  Against a ring shared by the
-// CTA, in CSR order (us with cold L2): Q1 160^3 263 -> 222, the 110^3 mesh
-// 181 -> 93, Q1 64^3 31 -> 27; 109 M FMAs take 180 us at the pipe's peak.
+// CTA, in CSR order (us, calls back to back): Q1 160^3 240 -> 204, the 110^3 mesh
+// 169 -> 81, Q1 64^3 25 -> 19; 109 M FMAs take 176 us at the pipe's peak.
 template <typename Ring, typename X>
 __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, const X* x, bool with_dot) {
   using T = typename Ring::Val;

@@ -12,8 +12,9 @@
 // from the same deterministic sums, so no host synchronisation happens per
 // step and every CTA takes the same branch.  Each CTA owns a fixed range of
 // rows (a run of product steps) for all phases, so only the two sums and the
-// gather of p need synchronisation across the CTAs that share the system:
-// three group barriers per step.  A single-system solve uses the whole grid
+// gather of p need synchronisation across the CTAs that share the system: two
+// sums through accumulators (or the group barrier, see acc_words) and one barrier
+// or neighbour wait per step.  A single-system solve uses the whole grid
 // as one group; a batched solve gives each system its own group of CTAs (one
 // CTA for most systems) and lets CTAs take systems from a queue.
 //
@@ -207,8 +208,9 @@ cudaError_t launch_wait_timeout_selftest(SolveCtrl* ctrl, unsigned long long lim
 // barriers as in a solve step, warp 0 of every CTA either meets the others at
 // the group barrier (mode 0: group_barrier_t0), or runs a group sum (mode 1:
 // publishes the CTA's value in one of two alternating slots, meets the others
-// at the barrier, and sums the group's values exactly with
-// fx_warp_sum_array, as group_sum in the solve does).  The waits are the
+// at the barrier, and sums the group's values exactly with fx_warp_sum_array: the
+// general form of the solves' group_sum; the sums of a step usually go through
+// the accumulators, which it does not time).  The waits are the
 // solves' bounded ones: a wait that gives up raises ctrl->abort, after which
 // every CTA stops.  out[rank] keeps the sums live.
 __global__ void __launch_bounds__(kBlock, kCtasPerSm)

@@ -201,8 +201,11 @@ __device__ __forceinline__ void solve_task(const Ring& sm, const TaskState* cons
   // p is written (release pattern as in the group barrier) and waits until
   // the CTAs that own the columns its rows reach (ranks dep_lo..dep_hi) have
   // published the same step: the next product gathers p only from them.
-  // Reusing p in place is safe: a CTA overwrites its p only after the r.r
-  // barrier of the step, which every CTA reaches after its product.
+  // Reusing p in place is safe: a CTA overwrites its p only once it has the step's
+  // r.r, i.e. every CTA's arrival at that sum, and a CTA arrives only after its
+  // p.q, whose value depends on every p that its product has gathered.  Those loads
+  // have returned before the arrival is even computed, so no fence is needed
+  // between them (in the general form of the sums the barrier has its fences).
   auto neighbor_sync = [&]() -> bool {
     cta_sync();
     if (warp == 0) {

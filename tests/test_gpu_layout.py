@@ -149,3 +149,28 @@ def test_batch_layout_from_host_and_device_and_at_the_budget(mixed):
         solved(1 << 20, False)
     need = int(re.search(r"needs up to (\d+) bytes", str(refused.value)).group(1))
     assert np.array_equal(xh, solved(need, False))
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("span", [300, 10 ** 6])
+@pytest.mark.parametrize("kind", ["even", "edges", "uneven", "pairs", "long"])
+def test_ring_product_of_every_step_form(kind, span, precision):
+    """The product of a solve's steps, which in mixed precision is the FP32 ring's:
+    one step from x = 0 with integers (products and sums exact in FP32, dot products
+    in FP64) gives x = (b.b / b.Ab) b to the last bit."""
+    cg = cg_mod()
+    for n, ctas in ((533, 0), (1500, 3), (1500, 0), (70000, 0), (70000, 7)):
+        if span > 65535 and n < 70000:
+            continue
+        A = _matrix(kind, n, span, 2 * n + len(kind))
+        rng = np.random.default_rng(6)
+        b = rng.integers(1, 21, n) * rng.choice([-1.0, 1.0], n)
+        gamma = float(b @ oracle.spmv(A, b))
+        assert gamma != 0.0
+        if gamma < 0:
+            A = fi.CSR(A.row_ptr, A.col_idx, -A.val, n)
+        x = np.zeros(n)
+        with handle(A, ctas=ctas, precision=precision) as h:
+            res = cg.cg_solve(h, b, x, tol=0.0, maxit=1)
+        assert res.status == cg.CG_ENOTCONV and res.iters == 1, (n, ctas, res)
+        assert np.array_equal(x, (float(b @ b) / abs(gamma)) * b), (n, ctas)
