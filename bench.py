@@ -103,11 +103,19 @@ def peaks():
 
 # ----------------------------------------------------------------- counters
 
+def col_bytes(n: int) -> int:
+    """Bytes per stored column of an N^3 grid system: 16-bit offsets where a
+    step (32 consecutive rows) spans at most 65535 columns, else 32-bit columns."""
+    N = round(n ** (1 / 3))
+    return 2 if 2 * (N * N + N + 1) + 31 <= 65535 else 4
+
+
 def algorithmic_bytes_per_iter(n: int, nnz: int) -> int:
-    """One FP64 CG step: the CSR product (12 B per entry + 4 B per row
-    pointer) plus 88 B per row of vector traffic (p gather 8, q write 8;
-    x, r read+write 32, p, q read 16; r read 8, p read+write 16)."""
-    return 12 * nnz + 4 * (n + 1) + 88 * n
+    """One FP64 CG step: the matrix as it is stored (values and columns, 10 or
+    12 B per entry, and 2 B per row of step tables) plus 88 B per row of vector
+    traffic (p gather 8, q write 8; x, r read+write 32, p, q read 16; r read 8,
+    p read+write 16)."""
+    return (8 + col_bytes(n)) * nnz + 2 * n + 88 * n
 
 
 def flops_per_iter(n: int, nnz: int) -> int:
@@ -115,17 +123,17 @@ def flops_per_iter(n: int, nnz: int) -> int:
 
 
 def mixed_bytes_per_iter(n: int, nnz: int) -> int:
-    """One mixed-precision CG step: FP32 values and column indices (8 B per
-    entry), row pointers, and 96 B per row (p32 gather 4, p read 8 and q
+    """One mixed-precision CG step: FP32 values and columns (6 or 8 B per
+    entry), step tables, and 96 B per row (p32 gather 4, p read 8 and q
     write 8 for the FP64 p.q; x, r read+write 32 and p, q read 16; r read 8,
     p read+write 16, p32 write 4)."""
-    return 8 * nnz + 4 * (n + 1) + 96 * n
+    return (4 + col_bytes(n)) * nnz + 2 * n + 96 * n
 
 
 def replacement_bytes(n: int, nnz: int) -> int:
-    """One FP64 residual replacement r = b - A x: the FP64 product (12 B per
-    entry, row pointers, x gather 8) plus b read 8 and r write 8 per row."""
-    return 12 * nnz + 4 * (n + 1) + 24 * n
+    """One FP64 residual replacement r = b - A x: the FP64 product (10 or 12 B
+    per entry, step tables, x gather 8) plus b read 8 and r write 8 per row."""
+    return (8 + col_bytes(n)) * nnz + 2 * n + 24 * n
 
 
 def replacements(iters: int, every: int) -> int:
@@ -152,13 +160,13 @@ def solve_flops(n: int, nnz: int, iters: int, mixed: bool, every: int = 50, jaco
 
 def l2_resident(n: int, nnz: int, mixed: bool) -> bool:
     """Whether the matrix and the vectors of a solve fit in the 126.5 MiB L2."""
-    mat = (8 if mixed else 12) * nnz + 4 * (n + 1)
+    mat = ((4 if mixed else 8) + col_bytes(n)) * nnz + 2 * n
     return mat + 48 * n < 100 * 2**20
 
 
 def spmv_bytes(n: int, nnz: int) -> int:
-    """y = A x: values and columns (12 B per entry), row pointers, x read once, y written."""
-    return 12 * nnz + 4 * (n + 1) + 16 * n
+    """y = A x: values and columns (10 or 12 B per entry), step tables, x read once, y written."""
+    return (8 + col_bytes(n)) * nnz + 2 * n + 16 * n
 
 
 def source_sha() -> str:
@@ -574,13 +582,17 @@ def blas1_record(cg, dev, stream, flush, hbm_peak):
     return out
 
 
+def col_type(n: int) -> str:
+    return "unsigned short" if col_bytes(n) == 2 else "int"
+
+
 def solve_kernel_name(cg, h, mixed: bool, jac: bool) -> str:
     kind = h.partition_info()[1]
     if kind == cg.CG_SOLVE_KERNEL_CLUSTER:
         return "cg_cluster_kernel"
     small = kind == cg.CG_SOLVE_KERNEL_SMALL_SHARE
     return (f"cg_solve_kernel<{'true' if mixed else 'false'}, {'true' if jac else 'false'}, "
-            f"{'true' if small else 'false'}>")
+            f"{'true' if small else 'false'}, {col_type(h.n)}>")
 
 
 def roofline(n, nnz, iters, launch_s, mixed, jac, kname, workload, hbm_peak, hbm_src, fp64_peak, fp64_src):
@@ -774,8 +786,8 @@ def run_ours(args):
         "roofline": roof,
         "accuracy": accuracy,
         "spmv": {"gbs": spmv_gbs, "frac": spmv_gbs / hbm_peak, "ms": spmv_ms, "bytes": spmv_bytes(n, nnz),
-                 "l2": "flushed before every call", "precision": "fp64", "kernel": "spmv_kernel",
-                 "traffic": recorded_traffic("spmv_kernel", f"{args.matrix}_{args.grid}")},
+                 "l2": "flushed before every call", "precision": "fp64", "kernel": f"spmv_kernel<{col_type(n)}>",
+                 "traffic": recorded_traffic(f"spmv_kernel<{col_type(n)}>", f"{args.matrix}_{args.grid}")},
         "blas1": blas1,
         "energy": {"joules_per_solve": joules, "avg_watts": watts, "idle_watts": idle_watts,
                    "joules_per_solve_above_idle": (joules - idle_watts * tl / len(lat)
@@ -839,15 +851,16 @@ def run_variants(args, cg, A, xs, x64, dev, stream, energy, hbm, fp64, fp64_line
         ms = spmv_alone(cg, h, xd, y, stream, flush)
         gbs = spmv_bytes(A64.n, A64.nnz) / (ms * 1e-3) / 1e9
         rec["spmv"] = {"gbs": gbs, "frac": gbs / hbm[0], "ms": ms, "bytes": spmv_bytes(A64.n, A64.nnz),
-                       "l2": "flushed before every call (the 87.6 MB product barely exceeds L2)"}
+                       "l2": "flushed before every call"}
         h.close()
-        # the three group-wide synchronisations of a small-share step (two
-        # sums, one barrier), timed alone on the whole grid
+        # the group barrier and the group sum in its general form, timed alone on
+        # the whole grid: what a step (two sums, one barrier) would spend on them if
+        # its sums did not go through the accumulators
         bar_us, sum_us = cg.cg_probe_group_sync(dev.index or 0, 20000)
         step_us = 1000.0 * rec["ms_per_solve"] / rec["iters"]
         rec["sync_probe"] = {"barrier_us": bar_us, "sum_us": sum_us, "per_step_us": 2 * sum_us + bar_us,
                              "step_us": step_us, "share_of_step": (2 * sum_us + bar_us) / step_us,
-                             "source": "cg_probe_group_sync (the solves' group barrier and group sum, one CTA "
+                             "source": "cg_probe_group_sync (the solves' group barrier and general group sum, one CTA "
                                        "per SM, 20000 of each)"}
         return rec
 
