@@ -145,9 +145,9 @@ int cg_partition_info(cg_handle h, int32_t* max_rows, int32_t* kernel);
 /*
  * y = A x (Sec. 2.3 / 5.2): y_i = sum_{k=IA(i)}^{IA(i+1)-1} AA(k) x(JA(k)),
  * FP64 with FMA, each row summed in storage order by one lane, as the sum of its
- * two halves (rows of 33 to 64 entries, and all rows of small systems) or by a
- * warp (longer rows).  The bits depend on the matrix and the GPU's SM count, not
- * on the CTA count.  x, y: device pointers to
+ * two halves (rows of 33 to 64 entries, and all rows of small systems of 12 entries
+ * per row and more) or by a warp (longer rows).  The bits depend on the matrix and
+ * the GPU's SM count, not on the CTA count.  x, y: device pointers to
  * n doubles; x and y must not overlap.  Asynchronous on the handle's stream.
  */
 int cg_spmv(cg_handle h, const double* x, double* y);

@@ -163,6 +163,7 @@ struct Job {
   int group = 1;
   double* d_x = nullptr;
   double bytes_step = 0.0;
+  int64_t stream_bytes = 0;
   double steps_est = 0.0;
 };
 
@@ -553,6 +554,7 @@ void admit(cg_batch_ctx* b) {
     j->bytes = bytes;
     j->group = group;
     j->bytes_step = bytes_per_step(n, nnz, b->mixed);
+    j->stream_bytes = (b->mixed ? 8 : 12) * nnz;  // (at most, but for padding)
     j->steps_est = est_steps(b->model, n);
     cudaError_t e = L.total > cap ? cudaMalloc(&j->d_extra, L.total - cap) : cudaSuccess;
     if (e != cudaSuccess) {
@@ -780,9 +782,13 @@ std::vector<Job*> build_queue(cg_batch_ctx* b, const std::vector<Job*>& res) {
   }
   b->h_queue->ntasks = nt;
   // the systems of a round run side by side: their vectors share the L2
-  int64_t reused = 0;
-  for (const Job* j : in_round) reused += cgk::step_reused_bytes(j->req.n, b->mixed, b->jacobi);
+  int64_t reused = 0, streams = 0;
+  for (const Job* j : in_round) {
+    reused += cgk::step_reused_bytes(j->req.n, b->mixed, b->jacobi);
+    streams += j->stream_bytes;
+  }
   b->h_queue->stream_rows = cgk::stream_row_tables(reused, b->l2_bytes) ? 1 : 0;
+  b->h_queue->keep = cgk::streams_stay(streams, reused, b->l2_bytes) ? 1 : 0;
   return in_round;
 }
 

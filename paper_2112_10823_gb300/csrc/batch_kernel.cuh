@@ -11,12 +11,12 @@ namespace cgk {
 // A task of the computing warps or of the producer warp; false if the ring did
 // not drain in time (a task that ended in a timeout has drained it all the same).
 template <bool kMixed, bool kJacobi, typename C>
-__device__ __noinline__ bool batch_task(unsigned char* smem, const TaskState* tk, int32_t stream_rows) {
+__device__ __noinline__ bool batch_task(unsigned char* smem, const TaskState* tk, int32_t stream_rows, int32_t keep) {
   using T = std::conditional_t<kMixed, float, double>;
   using Ring = RingSmem<T, C>;
   const Ring sm{smem};
   if (threadIdx.x >= kBlock) {
-    const int end = producer(sm, tk->P.A, tk->rank, false, tk->P.wait_limit_ns);
+    const int end = producer(sm, tk->P.A, tk->rank, false, keep != 0, tk->P.wait_limit_ns);
     if (end != kStreamDone) solve_fail(tk->P, threadIdx.x == kBlock);
     return end != kStreamLost;
   }
@@ -48,9 +48,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     const BatchTask tk = B.queue->task[t];
     ring_reset(RingSmem<T, int32_t>{smem_raw});
     task_load(&task, B.sys[tk.sys], tk.rank);
-    const int32_t stream_rows = B.queue->stream_rows;
-    const bool drained = task.P.A.col16 ? batch_task<kMixed, kJacobi, uint16_t>(smem_raw, &task, stream_rows)
-                                   : batch_task<kMixed, kJacobi, int32_t>(smem_raw, &task, stream_rows);
+    const int32_t stream_rows = B.queue->stream_rows, keep = B.queue->keep;
+    const bool drained = task.P.A.col16 ? batch_task<kMixed, kJacobi, uint16_t>(smem_raw, &task, stream_rows, keep)
+                                       : batch_task<kMixed, kJacobi, int32_t>(smem_raw, &task, stream_rows, keep);
     if (!__syncthreads_and(drained)) break;
   }
 }

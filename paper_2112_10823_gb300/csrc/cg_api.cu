@@ -278,6 +278,7 @@ struct cg_ctx {
   int cluster_R = 0;  // > 0: cg_solve runs the cluster kernel, R rows and E entries per CTA
   int cluster_E = 0;
   bool col16 = false;  // columns stored as 16-bit offsets
+  int64_t stream_bytes = 0;
   // device memory owned by the handle: the matrix in stream order
   unsigned char* d_stream = nullptr;
   double* d_val64 = nullptr;
@@ -424,7 +425,7 @@ cgk::DevCsr dev_view(const cg_ctx* h) {
   A.max_rows = h->max_rows;
   A.nnz = h->nnz;
   A.col16 = h->col16 ? 1 : 0;
-  A.pad = 0;
+  A.keep = 0;
   return A;
 }
 
@@ -826,6 +827,7 @@ int cg_create(cg_handle* out, const cg_csr* csr, int64_t n, int64_t nnz, const c
   }
   h->col16 = found.scan.span <= cgk::kColSpan16;
   cgh::place_steps(rp, h->nblocks, h->col16, mixed, part);
+  h->stream_bytes = part.stream_units * cgk::kUnit;
   if (!one_block) {
     add_streams(part.chunk_off.size() - 1, part.stream_units, part.entries);
     CG_TRY(str.alloc(h->allocs), "cg_create: cudaMalloc");
@@ -881,7 +883,11 @@ int cg_spmv(cg_handle h, const double* x, double* y) {
   if (h->n == 0) return CG_OK;
   if (!x || !y) return fail(h, CG_EINVAL, "cg_spmv: NULL vector");
   DeviceGuard g(h->device);
-  cudaError_t e = cgk::launch_spmv(dev_view(h), x, y, h->d_err, h->stream);
+  cgk::DevCsr A = dev_view(h);
+  // (a mixed handle's product reads the columns and FP64 values)
+  const int64_t matrix = h->precision == CG_PREC_MIXED ? 12 * h->nnz : h->stream_bytes;
+  A.keep = cgk::streams_stay(matrix, 16 * h->n, l2_bytes(h->device)) ? 1 : 0;
+  cudaError_t e = cgk::launch_spmv(A, x, y, h->d_err, h->stream);
   return e == cudaSuccess ? CG_OK : cuda_fail(h, e, "cg_spmv: launch");
 }
 
@@ -1075,8 +1081,9 @@ int cg_solve(cg_handle h, const double* b, double* x, double tol, int64_t maxit,
   P.replace_every = h->replace_every;
   P.wait_limit_ns = h->wait_limit_ns;
   P.group = h->nblocks;
-  P.stream_rows = cgk::stream_row_tables(
-      cgk::step_reused_bytes(h->n, h->precision == CG_PREC_MIXED, h->d_dinv != nullptr), l2_bytes(h->device));
+  const int64_t reused = cgk::step_reused_bytes(h->n, h->precision == CG_PREC_MIXED, h->d_dinv != nullptr);
+  P.stream_rows = cgk::stream_row_tables(reused, l2_bytes(h->device));
+  P.A.keep = cgk::streams_stay(h->stream_bytes, reused, l2_bytes(h->device)) ? 1 : 0;
   P.chunk_iters = 0;
   P.dinv = h->d_dinv;
   P.flags = h->nblocks > 1 ? h->d_flags : nullptr;

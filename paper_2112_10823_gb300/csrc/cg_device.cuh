@@ -586,8 +586,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 }
 
 // The producer warp of CTA `rank`: lane w copies the chunks of warp w's stream,
-// pass after pass (`once`: one pass), into its ring as the warp gives slots
-// back, until the computing warps say stop.  One lane per warp: a copy takes
+// pass after pass (`once`: one pass; `keep`: with the L2's default policy, else
+// evict-first), into its ring as the warp gives slots back, until the computing warps say stop.  One lane per warp: a copy takes
 // some thirty instructions, which are no part of any computing warp's chain,
 // and all warps that wait for one are served together.  On stop every lane
 // waits for its copies in flight, so that none lands after the CTA is gone or
@@ -603,7 +603,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // be used again.
 enum : int { kStreamDone = 0, kStreamIdle = 1, kStreamLost = 2 };
 template <typename Ring>
-__device__ __forceinline__ int producer(const Ring& sm, const DevCsr& A, int rank, bool once,
+__device__ __forceinline__ int producer(const Ring& sm, const DevCsr& A, int rank, bool once, bool keep,
                                         unsigned long long limit_ns) {
   const int w = threadIdx.x & 31;
   const bool mine = w < kWarps;
@@ -639,7 +639,9 @@ __device__ __forceinline__ int producer(const Ring& sm, const DevCsr& A, int ran
       uint64_t* const bar = sm.full(w, head);
       const uint32_t bytes = (end0 - start) * static_cast<uint32_t>(kUnit);
       mbar_arrive_expect_tx(bar, bytes);
-      bulk_g2s_hint(sm.slot(w, head), A.stream + static_cast<size_t>(start) * kUnit, bytes, bar, pol);
+      const unsigned char* const from = A.stream + static_cast<size_t>(start) * kUnit;
+      if (keep) bulk_g2s(sm.slot(w, head), from, bytes, bar);
+      else bulk_g2s_hint(sm.slot(w, head), from, bytes, bar, pol);
       phases ^= 1u << head;
       head = head + 1 == kSlots ? 0 : head + 1;
       ++issued;
@@ -1065,15 +1067,16 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
 // stream order, from chunk `chunk` and (mixed) entry `entry` on: the passes outside a
 // mixed solve's step loop (its setup, the final true residual, the residual
 // replacements), which leaves the ring's contents alone, and a mixed handle's
-// product.  Latency bounds it: a step's chain would be its chunk's offset, columns,
+// product (kKeep: loads with the L2's default policy).  Latency bounds it: a step's chain would be its chunk's offset, columns,
 // x, FMAs, chunk after chunk.  So 32 chunk offsets are loaded at once, and a batch's
 // columns while the batch before waits for its x.
-template <typename Ring>
+template <typename Ring, bool kKeep = false>
 __device__ __forceinline__ void direct_pass(const DevCsr& A, uint32_t chunk, int64_t entry, int s, int s1,
                                             const double* x, double* out) {
   using T = typename Ring::Val;
   using C = typename Ring::Col;
   constexpr int kU = 7;  // entries per lane and batch (half an FP32 chunk)
+  auto ld = [](const auto* at) { return kKeep ? __ldg(at) : __ldcs(at); };
   const int lane = fresh_tid() & 31;
   for (; s < s1; ++s) {
     const int4 d = A.step[s];
@@ -1105,7 +1108,7 @@ __device__ __forceinline__ void direct_pass(const DevCsr& A, uint32_t chunk, int
       const int len = max(0, min(min(seg - u, cnt) - k, kU));
 #pragma unroll
       for (int i = 0; i < kU; ++i, cp += place.stride)
-        if (i < len) c[i] = static_cast<int>(__ldcs(cp));
+        if (i < len) c[i] = static_cast<int>(ld(cp));
       return len;
     };
     double acc = 0.0;
@@ -1117,7 +1120,7 @@ __device__ __forceinline__ void direct_pass(const DevCsr& A, uint32_t chunk, int
 #pragma unroll
       for (int i = 0; i < kU; ++i, vp += place.stride)
         if (i < len) {
-          a[i] = __ldcs(vp);
+          a[i] = ld(vp);
           g[i] = xb[c[i]];
         }
       const int now = len, most = cnt - k;  // (most: warp-uniform)

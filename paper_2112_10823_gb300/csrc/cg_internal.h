@@ -10,9 +10,10 @@ namespace cgk {
 // its own steps of the CTA's rows from its own ring in shared memory, and one
 // producer warp, whose lane w fills warp w's ring with 1-D TMA bulk copies.
 // Nineteen computing warps (with the producer five per SM sub-partition), 96
-// registers per thread, nothing spilled.  15, 19, 23 warps, us per step of a Q1
-// solve: 32^3 14.2, 12.9, 13.1; 64^3 28.9, 27.6, 29.0; 160^3 292, 267, 266;
-// 160^3 mixed 230, 214, 207.
+// registers per thread (at most 8 bytes spilled, in mixed precision).  15, 19, 23
+// warps, us per step of a Q1 solve: 32^3 14.2, 12.9, 13.1; 64^3 28.9, 27.6, 29.0;
+// 160^3 292, 267, 266; 160^3 mixed 230, 214, 207 (before the uneven chunks went
+// lane after lane).
 constexpr int kWarps = 19;
 constexpr int kBlock = kWarps * 32;      // their threads
 constexpr int kThreads = kBlock + 32;    // and the producer warp
@@ -120,7 +121,7 @@ struct DevCsr {
   int32_t max_rows;           // most rows in one CTA's range (host side; 0 if unknown)
   int64_t nnz;
   int32_t col16;              // 1: 16-bit column offsets
-  int32_t pad;
+  int32_t keep;               // 1: the streams stay in the L2 (streams_stay)
 };
 
 // Whether a solve of A in one launch (chunk_iters <= 0) runs the small-share
@@ -193,6 +194,8 @@ struct BatchTask {
 struct BatchQueue {
   int32_t ntasks;
   int32_t stream_rows;          // row tables evict-first in this launch (stream_row_tables)
+  int32_t keep;                 // the streams stay in the L2 (streams_stay)
+  int32_t pad;
   BatchTask task[1];            // ntasks entries (allocated to capacity)
 };
 struct BatchParams {
@@ -216,6 +219,16 @@ inline int64_t step_reused_bytes(int64_t n, bool mixed, bool jacobi) {
 // to give up.
 inline bool stream_row_tables(int64_t reused_bytes, int64_t l2_bytes) {
   return l2_bytes > 0 && 7 * reused_bytes > 4 * l2_bytes;
+}
+
+// Whether the matrix streams are read with the L2's default policy instead of
+// evict-first: when they and the bytes that the running steps read again take at
+// most 3/4 of the L2, and so stay there.  Evict-first then only costs energy (Q1
+// 64^3, FP64 step 14.1 -> 10.6 mJ at the same 25 us, mixed 9.4 -> 7.8); where they do
+// not fit, it keeps the vectors in (72^3 35.5 us with it, 35.8 without; 90^3 53.9,
+// 58.8; 160^3 274, 283).
+inline bool streams_stay(int64_t stream_bytes, int64_t reused_bytes, int64_t l2_bytes) {
+  return 4 * (stream_bytes + reused_bytes) <= 3 * l2_bytes;
 }
 
 // Status codes (same values as include/cg.h).

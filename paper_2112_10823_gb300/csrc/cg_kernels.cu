@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   ring_init(sm);
   const unsigned long long lim = 2000000000ull;
   if (threadIdx.x >= kBlock) {
-    if (producer(sm, A, blockIdx.x, true, lim) != kStreamDone && threadIdx.x == kBlock) atomicExch(err, kETIMEOUT);
+    if (producer(sm, A, blockIdx.x, true, A.keep != 0, lim) != kStreamDone && threadIdx.x == kBlock) atomicExch(err, kETIMEOUT);
     return;
   }
   const int bw = blockIdx.x * kWarps + (threadIdx.x >> 5);
@@ -67,13 +67,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 // the former CSR ring 25.0 and 239, a warp per stream (19 per SM) 27.1 and 350.
 constexpr int kDirectThreads = 64, kDirectBlocks = 16;
 
-template <typename C>
+template <typename C, bool kKeep>
 __global__ void __launch_bounds__(kDirectThreads, kDirectBlocks)
     spmv_direct_kernel(const __grid_constant__ DevCsr A, const double* x, double* y) {
   using Ring = RingSmem<float, C>;
   const int64_t s = (static_cast<int64_t>(blockIdx.x) * kDirectThreads + threadIdx.x) >> 5;
   if (s >= A.nsteps) return;
-  direct_pass<Ring>(A, A.step_chunk[s], A.step_entry[s], static_cast<int>(s), static_cast<int>(s) + 1, x,
+  direct_pass<Ring, kKeep>(A, A.step_chunk[s], A.step_entry[s], static_cast<int>(s), static_cast<int>(s) + 1, x,
                     y);
 }
 
@@ -105,8 +105,9 @@ cudaError_t ensure_smem_attr(const void* kernel, size_t bytes) {
 cudaError_t launch_spmv(const DevCsr& A, const double* x, double* y, int32_t* err, cudaStream_t s) {
   if (A.val64 != nullptr) {
     const unsigned blocks = static_cast<unsigned>((static_cast<int64_t>(A.nsteps) * 32 + kDirectThreads - 1) / kDirectThreads);
-    if (A.col16) spmv_direct_kernel<uint16_t><<<blocks, kDirectThreads, 0, s>>>(A, x, y);
-    else spmv_direct_kernel<int32_t><<<blocks, kDirectThreads, 0, s>>>(A, x, y);
+    auto run = [&](auto kernel) { kernel<<<blocks, kDirectThreads, 0, s>>>(A, x, y); };
+    if (A.keep) A.col16 ? run(spmv_direct_kernel<uint16_t, true>) : run(spmv_direct_kernel<int32_t, true>);
+    else A.col16 ? run(spmv_direct_kernel<uint16_t, false>) : run(spmv_direct_kernel<int32_t, false>);
     return cudaGetLastError();
   }
   const size_t smem = solve_smem_bytes(false, A.col16 != 0);

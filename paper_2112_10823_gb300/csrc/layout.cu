@@ -1,9 +1,10 @@
 // Stream order of a matrix (cg_internal.h): what a handle or an admitted
 // system keeps of its CSR arrays, built on the device, one warp per step.
-// Both kernels are bound by the CSR arrays' bytes: the scan reads the columns
-// once; the fill reads every entry once (lanes at the stride of a row, so that
-// a warp's reads of consecutive entries of 32 rows meet again in L1) and writes
-// it once, coalesced.
+// Both kernels are bound by the CSR arrays' bytes and, with few or long steps, by
+// latency: the scan reads the columns once, eight loads of a lane under way; the fill
+// reads every entry once (lanes at the stride of a row, so that a warp's reads of
+// consecutive entries of 32 rows meet again in L1; a batch of loads before its
+// stores) and writes it once.  Q1 160^3: 108 and 711 us.
 #include <algorithm>
 #include "cg_device.cuh"
 
@@ -11,7 +12,7 @@ namespace cgk {
 
 namespace {
 constexpr int kLayoutBlock = 256;
-constexpr int kFillWarps = 152 * 48;
+constexpr int kFillWarps = 152 * 48;  // what the fill of long rows is spread over
 constexpr int kBatch = 5;  // entries per lane whose loads are under way together
 
 unsigned layout_grid(int32_t s0, int32_t s1) {

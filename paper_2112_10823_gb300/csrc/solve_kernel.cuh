@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   ring_init(sm);
   task_load(&task, P, blockIdx.x);
   if (threadIdx.x >= kBlock) {
-    if (producer(sm, P.A, blockIdx.x, false, P.wait_limit_ns) != kStreamDone) solve_fail(P, threadIdx.x == kBlock);
+    if (producer(sm, P.A, blockIdx.x, false, P.A.keep != 0, P.wait_limit_ns) != kStreamDone) solve_fail(P, threadIdx.x == kBlock);
     return;
   }
   // the neighbour wait at the end of a step pays off on large shares (160^3:
