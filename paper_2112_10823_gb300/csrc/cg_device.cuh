@@ -847,7 +847,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
   struct Chunk {
     int cnt;      // entries per lane (warp-uniform; 0: the step has none; -1: no chunk)
     int len;      // of them, those this lane's segment has
-    int place;    // of this lane's entries: base, and the stride in bits 16.. (ChunkPlace; 32: the full form)
+    int place;    // of this lane's entries: base, and the stride in bits 16.. (ChunkPlace); 32 << 16: the full form
     bool ends;    // the last one of its step
     int slot;
     int val_off;  // its values' place in the slot
@@ -876,9 +876,14 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
     c.cnt = min(step_chunk(d), d.z - u);
     c.len = max(0, min(seg - u, c.cnt));
     c.slot = tail;
-    const ChunkPlace at = chunk_place<C>(d, u, c.cnt, seg, lane);
-    c.place = at.base | at.stride << 16;
-    c.val_off = (at.tot * static_cast<int>(sizeof(C)) + kUnit - 1) & ~(kUnit - 1);
+    if (step_padded<C>(d) || __all_sync(0xffffffffu, u + c.cnt <= seg)) {  // (chunk_place's full form)
+      c.place = 32 << 16;
+      c.val_off = c.cnt * 32 * static_cast<int>(sizeof(C));
+    } else {
+      const ChunkPlace at = chunk_place<C>(d, u, c.cnt, seg, lane);
+      c.place = at.base | at.stride << 16;
+      c.val_off = (at.tot * static_cast<int>(sizeof(C)) + kUnit - 1) & ~(kUnit - 1);
+    }
     u += c.cnt;
     c.row = d.x;
     c.kind = d.y;
@@ -894,12 +899,10 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
     dn = load_step(io, step_at(s + 1));
     seg_n = load_seg_len(io, min(s + 1, s1 - 1), lane);
   };
-  auto full = [](const Chunk& c) { return c.place >> 16 == 32; };
-  // this lane's entry 0
-  auto cols = [&](const Chunk& c) { return reinterpret_cast<const C*>(sm.slot(w, c.slot)) + (c.place & 0xffff); };
-  auto vals = [&](const Chunk& c) {
-    return reinterpret_cast<const T*>(sm.slot(w, c.slot) + c.val_off) + (c.place & 0xffff);
-  };
+  auto full = [](const Chunk& c) { return c.place == 32 << 16; };
+  auto base = [&](const Chunk& c) { return full(c) ? lane : c.place & 0xffff; };
+  auto cols = [&](const Chunk& c) { return reinterpret_cast<const C*>(sm.slot(w, c.slot)); };
+  auto vals = [&](const Chunk& c) { return reinterpret_cast<const T*>(sm.slot(w, c.slot) + c.val_off); };
   // x of the columns of the step of the chunk being gathered: 16-bit columns are
   // offsets from the step's smallest one
   auto x_of = [&]() -> const X* { return sizeof(C) == 2 ? x + d.w : x; };
@@ -913,6 +916,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
       const X* const xb = x_of();
       const C* cp = cols(c);
       if (full(c)) {
+        cp += lane;
 #pragma unroll
         for (int k = 0; k < kU; ++k) {
           if (k % 3 == 0 && k >= c.cnt) break;
@@ -920,6 +924,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
         }
       } else {
         const int stride = c.place >> 16;
+        cp += base(c);
 #pragma unroll
         for (int k = 0; k < kU; ++k, cp += stride) {
           if (k % 3 == 0 && k >= c.cnt) break;
@@ -930,6 +935,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
     auto sum = [&](const Chunk& c, const X* xv) {
       const T* vp = vals(c);
       if (full(c)) {
+        vp += lane;
 #pragma unroll
         for (int k = 0; k < kU; ++k) {
           if (k % 3 == 0 && k >= c.cnt) break;
@@ -937,6 +943,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
         }
       } else {
         const int stride = c.place >> 16;
+        vp += base(c);
 #pragma unroll
         for (int k = 0; k < kU; ++k, vp += stride) {
           if (k % 3 == 0 && k >= c.cnt) break;
@@ -995,7 +1002,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
   if (c.cnt > 0) {
     if (!wait_next()) return leave(false);
     const X* const xb = x_of();
-    const C* cp = cols(c);
+    const C* cp = cols(c) + base(c);
     const int stride = c.place >> 16;
 #pragma unroll
     for (int k = 0; k < kU; ++k, cp += stride)
@@ -1008,8 +1015,8 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
     if (n.cnt > 0 && !wait_next()) return leave(false);
     const X* const xb = x_of();
     if (full(c) && full(n)) {
-      const T* const vp = vals(c);
-      const C* const cp = cols(n);
+      const T* const vp = vals(c) + lane;
+      const C* const cp = cols(n) + lane;
       // straight-line code for each size of c
       dispatch_tree<0, kU>(c.cnt, [&](auto N) {
 #pragma unroll
@@ -1025,8 +1032,8 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
       }
     } else {
       // at least one of them in another form
-      const T* vp = vals(c);
-      const C* cp = cols(n);
+      const T* vp = vals(c) + base(c);
+      const C* cp = cols(n) + base(n);
       const int cs = c.place >> 16, ns = n.place >> 16;
 #pragma unroll
       for (int k = 0; k < kU; ++k, vp += cs, cp += ns) {
@@ -1035,7 +1042,7 @@ __device__ __forceinline__ double ring_pass(unsigned char* smem, int s, int s1, 
         if (k < n.len) xv[k] = xb[*cp];
       }
       if (n.cnt > c.cnt) {
-        cp = cols(n);
+        cp = cols(n) + base(n);
 #pragma unroll
         for (int k = 0; k < kU; ++k, cp += ns)
           if (k >= c.cnt && k < n.len) xv[k] = xb[*cp];
