@@ -10,7 +10,7 @@ namespace cgk {
 // its own steps of the CTA's rows from its own ring in shared memory, and one
 // producer warp, whose lane w fills warp w's ring with 1-D TMA bulk copies.
 // Nineteen computing warps (with the producer five per SM sub-partition), 96
-// registers per thread (at most 8 bytes spilled, in mixed precision).  15, 19, 23
+// registers per thread, nothing spilled.  15, 19, 23
 // warps, us per step of a Q1 solve: 32^3 14.2, 12.9, 13.1; 64^3 28.9, 27.6, 29.0;
 // 160^3 292, 267, 266; 160^3 mixed 230, 214, 207 (before the uneven chunks went
 // lane after lane).
